@@ -604,7 +604,7 @@ static sim_status enqueue_gate(sim* s, const sim_gate* g) {
     CK(cudaEventRecord(e1, s->st), "event record");
     s->ev_pending.emplace_back(e0, e1);
   }
-  CK(qc::launch_post(s->P, L.ctl, s->grid, s->st), "post kernel launch");
+  CK(qc::launch_post(s->P, L.ctl, grid, s->st), "post kernel launch");
   if (s->timing) {
     // the traffic counters after this gate, for the per-launch figures of sim_timing_launches
     const size_t k = s->ev_pending.size() - 1;
@@ -1135,7 +1135,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
         e = qc::launch_select(L, job_sim[j]->d_mlp, const_cast<uint8_t*>(L.sel_dec), sg, cs);
       }
       if (e == cudaSuccess) e = qc::launch_gate_batch(d_jobs + off[t], n, total[t], kc, g, cs);
-      if (e == cudaSuccess) e = qc::launch_post_batch(d_jobs + off[t], n, grid, cs);
+      if (e == cudaSuccess) e = qc::launch_post_batch(d_jobs + off[t], n, g, cs);
     }
     if (use_graph && cs != st) {
       cudaError_t e2 = cudaStreamEndCapture(cs, &graph);
