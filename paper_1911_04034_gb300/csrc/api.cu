@@ -9,6 +9,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstdarg>
+#include <cstddef>
 #include <cstdio>
 #include <cstring>
 #include <string>
@@ -1662,22 +1663,103 @@ sim_status sim_sv_set_stream(sim_sv_t* v, void* stream) {
   return SIM_OK;
 }
 
+// The gates of a group: consecutive gates whose non-diagonal targets are among the low
+// qubits and at most T - L others (a diagonal gate joins any group).
+static void sv_group(int n, const sim_gate* gates, const uint8_t* form, size_t count, qc::SvGroup& G) {
+  std::memset(&G, 0, offsetof(qc::SvGroup, g));
+  G.T = qc::sv_tile_log2(n);
+  G.L = qc::sv_low_bits(G.T);
+  uint64_t bits = (1ull << G.L) - 1ull;
+  for (size_t k = 0; k < count; ++k)
+    if (form[k] != 2) bits |= 1ull << gates[k].target;
+  for (int q = G.L; popcount64(bits) < G.T; ++q) bits |= 1ull << q;  // the lowest qubits fill the tile
+  int where[64];
+  for (int q = 0; q < n; ++q) {
+    where[q] = q < G.L ? q : -1;
+    if (q >= G.L && ((bits >> q) & 1ull)) {
+      where[q] = G.L + G.nhi;
+      G.hi[G.nhi++] = (uint8_t)q;
+    }
+  }
+  G.ngates = (int)count;
+  for (size_t k = 0; k < count; ++k) {
+    const sim_gate& s = gates[k];
+    qc::SvGate& g = G.g[k];
+    std::memset(&g, 0, sizeof(g));
+    g.g = coef_of(&s);
+    g.form = form[k];
+    g.out_mask = s.ctrl_mask & ~bits;
+    g.out_vals = s.ctrl_vals & ~bits;
+    for (int q = 0; q < n; ++q)
+      if (((s.ctrl_mask >> q) & 1ull) && where[q] >= 0) {
+        g.lo_mask |= 1u << where[q];
+        if ((s.ctrl_vals >> q) & 1ull) g.lo_vals |= 1u << where[q];
+      }
+    g.target = where[s.target];
+    g.tbit = (uint32_t)s.target;
+    const double* u = s.u;
+    const bool z01 = u[2] == 0.0 && u[3] == 0.0, z10 = u[4] == 0.0 && u[5] == 0.0;
+    g.copy = (u[0] == 1.0 && u[1] == 0.0 && z01 ? 1u : 0u) | (u[6] == 1.0 && u[7] == 0.0 && z10 ? 2u : 0u);
+    if (form[k] == 1) {
+      g.sk = std::ilogb(u[0]);
+      for (int q = 0; q < 16; ++q)
+        if (g.g.c[q] < 0.0) g.sgn |= 1u << q;
+    }
+  }
+  if (count == 1) {  // one gate alone reads and writes what it changes (CZ a quarter of the state)
+    const qc::SvGate& g = G.g[0];
+    G.need_mask = g.lo_mask;
+    G.need_vals = g.lo_vals;
+    if (g.form == 2 && g.target >= 0 && g.copy) {
+      G.need_mask |= 1u << g.target;
+      if (g.copy & 1u) G.need_vals |= 1u << g.target;
+    }
+  }
+}
+
 sim_status sim_sv_apply_circuit(sim_sv_t* v, const sim_gate* gates, size_t n_gates) {
   if (!v || (!gates && n_gates)) return fail(SIM_ERR_INVALID, "NULL argument");
   std::string why;
   for (size_t k = 0; k < n_gates; ++k)
     if (!gate_ok(gates + k, v->n, &why)) return fail(SIM_ERR_INVALID, "invalid gate %zu: %s", k, why.c_str());
+  const int T = qc::sv_tile_log2(v->n), L = qc::sv_low_bits(T);
+  qc::SvGroup G;
+  sim_gate run[qc::kSvMaxGates];
+  uint8_t form[qc::kSvMaxGates];
+  size_t count = 0;
+  uint64_t high = 0;  // the non-diagonal targets above the low qubits
+  auto flush = [&]() -> cudaError_t {
+    // a few diagonal gates that together change less than the state move less memory one by
+    // one (each reads and writes what it changes); of a small state only launches count
+    double moved = T == qc::kSvMaxTile ? 0.0 : 1.0;
+    for (size_t k = 0; k < count; ++k)
+      moved += form[k] != 2 ? 1.0
+                            : std::ldexp((run[k].u[0] == 1.0 && run[k].u[1] == 0.0) || (run[k].u[6] == 1.0 && run[k].u[7] == 0.0) ? 0.5 : 1.0,
+                                         -popcount64(run[k].ctrl_mask));
+    const size_t step = moved < 1.0 ? 1 : (count ? count : 1);
+    cudaError_t e = cudaSuccess;
+    for (size_t k = 0; k < count && e == cudaSuccess; k += step) {
+      sv_group(v->n, run + k, form + k, step, G);
+      e = qc::launch_sv_group(v->psi, v->n, G, v->st);
+    }
+    count = 0;
+    high = 0;
+    return e;
+  };
   for (size_t k = 0; k < n_gates; ++k) {
-    // which amplitudes of a pair the gate reads and writes (see k_sv_gate)
     const double* u = gates[k].u;
-    const bool z01 = u[2] == 0.0 && u[3] == 0.0, z10 = u[4] == 0.0 && u[5] == 0.0;
-    const bool wa = !(u[0] == 1.0 && u[1] == 0.0 && z01), wb = !(u[6] == 1.0 && u[7] == 0.0 && z10);
-    const uint32_t rows = (wa ? 1u : 0u) | (wb ? 2u : 0u) | ((wa || (wb && !z10)) ? 4u : 0u) |
-                          ((wb || (wa && !z01)) ? 8u : 0u);
-    CK(qc::launch_sv_gate(v->psi, v->n, coef_of(gates + k), gates[k].target, gates[k].ctrl_mask, gates[k].ctrl_vals,
-                          rows, v->st),
-       "state vector gate");
+    const bool diag = u[2] == 0.0 && u[3] == 0.0 && u[4] == 0.0 && u[5] == 0.0;
+    if (diag && u[0] == 1.0 && u[1] == 0.0 && u[6] == 1.0 && u[7] == 0.0) continue;  // the identity
+    int e = 0;
+    bool pow2 = u[0] != 0.0 && std::fabs(std::frexp(u[0], &e)) == 0.5 && e >= -9 && e <= 1;
+    for (int q = 1; q < 8 && pow2; ++q) pow2 = std::fabs(u[q]) == std::fabs(u[0]);
+    const uint64_t bit = !diag && gates[k].target >= L ? 1ull << gates[k].target : 0ull;
+    if (count == (size_t)qc::kSvMaxGates || popcount64(high | bit) > T - L) CK(flush(), "state vector gates");
+    high |= bit;
+    form[count] = diag ? 2 : (pow2 ? 1 : 0);
+    run[count++] = gates[k];
   }
+  CK(flush(), "state vector gates");
   CK(cudaStreamSynchronize(v->st), "sync");
   return SIM_OK;
 }

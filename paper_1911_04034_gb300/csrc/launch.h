@@ -109,8 +109,30 @@ cudaError_t launch_mode_counts(const Pool& P, unsigned long long nchunks, unsign
 cudaError_t launch_copy_image(const Pool& P, unsigned long long chunk, uint8_t* out, cudaStream_t st);
 
 cudaError_t launch_sv_init(double* psi, unsigned long long amps, cudaStream_t st);
-cudaError_t launch_sv_gate(double* psi, int n, const GateCoef& g, int target, unsigned long long cmask,
-                           unsigned long long cvals, uint32_t rows, cudaStream_t st);
+// A group of gates on the uncompressed state, applied tile by tile (see sv.cu).
+constexpr int kSvMaxTile = 12;   // tile bits
+constexpr int kSvMaxGates = 32;  // gates of a group
+struct SvGate {
+  GateCoef g;
+  unsigned long long out_mask, out_vals;  // controls outside the tile's bits
+  uint32_t lo_mask, lo_vals;              // controls among them (tile index)
+  int target;                             // tile bit of the target, -1: outside (diagonal gates only)
+  uint32_t tbit;                          // the target qubit
+  int form;                               // 0 kept-term sums, 1 all coefficient parts +-2^sk, 2 diagonal
+  uint32_t copy;                          // bit r: row pair r is a plain copy
+  uint32_t sgn;                           // form 1: bit q set if coefficient q (GateCoef order) is negative
+  int sk;
+};
+struct SvGroup {
+  int T, L, nhi;             // tile bits; its low qubits; its other qubits hi[0 .. nhi), ascending
+  uint8_t hi[kSvMaxTile];
+  int ngates;
+  uint32_t need_mask, need_vals;  // the tile's amplitudes that are read and written (all, unless the group is one gate)
+  SvGate g[kSvMaxGates];
+};
+int sv_tile_log2(int n);
+int sv_low_bits(int tile_log2);
+cudaError_t launch_sv_group(double* psi, int n, const SvGroup& G, cudaStream_t st);
 
 // Checkpoint: image lengths, gather of all images, and the rebuild of directory and
 // page arena from saved images (pages [0, used) in chunk order).

@@ -311,6 +311,40 @@ def test_uncompressed_path_within_1e12(n):
         assert np.array_equal(got, psi)
 
 
+@pytest.mark.parametrize("n", [1, 4, 9, 11, 13, 22])
+def test_uncompressed_path_groups_of_gates(n):
+    """Gates run in groups over tiles of the state: targets, controls and diagonal gates
+    anywhere, sqrt(X) / sqrt(Y) on values outside the range of their scaled form (zeros of
+    both signs, values near 2^-1000) and on sums that cancel, more gates than a group holds;
+    every bit, signs of zeros included."""
+    import torch
+
+    rng = np.random.default_rng(n)
+    psi = rng.standard_normal(1 << n) + 1j * rng.standard_normal(1 << n)
+    v = psi.view(np.float64)
+    v[1::4] = v[0::4]
+    v[rng.integers(0, v.size, v.size // 4 + 1)] = 0.0
+    v[rng.integers(0, v.size, v.size // 8 + 1)] = -0.0
+    v[rng.integers(0, v.size, v.size // 8 + 1)] *= 2.0 ** -1000
+    mats = [Cc.SX, Cc.SY, Cc.SX.conj(), Cc.SY.T.conj(), Cc.T, Cc.Z, Cc.H, Cc.X, Cc.rz(0.7), Cc.rx(0.3), Cc.phase(math.pi / 2)]
+    gs = []
+    for k in range(80 if n < 20 else 24):
+        t = int(rng.integers(0, n))
+        ctl = [int(q) for q in rng.permutation(n)[: rng.integers(0, 4) if k % 2 else 0] if q != t]
+        gs.append(Cc.gate(t, mats[int(rng.integers(0, len(mats)))], {q: int(rng.integers(0, 2)) for q in ctl}))
+    gates = np.array(gs, dtype=Cc.GATE_DTYPE)
+    sv = qc().StateVector(n)
+
+    class View:
+        __cuda_array_interface__ = dict(shape=(2 << n,), typestr="<f8", data=(sv.data_ptr(), False), version=3)
+
+    torch.as_tensor(View(), device="cuda").copy_(torch.from_numpy(v.copy()))
+    torch.cuda.synchronize()
+    sv.apply_circuit(gates)
+    O.sv_run(psi, n, gates)
+    assert np.array_equal(sv.amplitudes().view(np.uint64), psi.view(np.uint64))
+
+
 def test_edge_shapes_and_controls():
     rng = np.random.default_rng(2)
     # single chunk (n == kc), one and two qubits, the top qubit, multi-controls with
