@@ -329,7 +329,7 @@ sim_status sim_create_ex(int n_qubits, int block_log2, int chunk_log2, double er
     // in a pool sized by the caller, no more than let its warps' free-page caches (each
     // up to its capacity plus one refill, and one chunk's output pages) hold a quarter
     // of the pool; none if not even one CTA fits
-    const uint64_t need = ((s->nchunks + 1) / 2 + qc::fast_pairs() - 1) / qc::fast_pairs();
+    const uint64_t need = ((s->nchunks + 1) / 2 + qc::fast_items(0) - 1) / qc::fast_items(0);
     uint64_t cap = need;
     if (pool_bytes) {
       const uint64_t per_cta = (uint64_t)qc::fast_warps() * (qc::fast_warp_cache() + 32 + qc::max_pages(s->kc));
@@ -472,6 +472,9 @@ static GateLaunch make_launch(sim* s, const sim_gate* g) {
     const bool diag = u[2] == 0 && u[3] == 0 && u[4] == 0 && u[5] == 0;
     const bool perm = u[0] == 0 && u[1] == 0 && u[6] == 0 && u[7] == 0;
     L.gfeat = (real ? 1u : 0u) | (diag ? 2u : 0u) | (perm ? 4u : 0u) | (t < kc ? 8u : 0u);
+    // a cross-chunk diagonal gate with a row that is an exact copy: the row that is not
+    L.solo = -1;
+    if (t >= kc && diag) L.solo = u[0] == 1.0 && u[1] == 0.0 ? 1 : (u[6] == 1.0 && u[7] == 0.0 ? 0 : -1);
     // a coefficient that can turn a normal value into a subnormal (see next_level)
     L.ctl.wide_gate = 0;
     for (int k = 0; k < 8; ++k)
@@ -528,11 +531,11 @@ static bool fast_applies(const sim* s, const sim_gate* g, GateLaunch& L) {
   const double* u = g->u;
   const bool diag = u[2] == 0.0 && u[3] == 0.0 && u[4] == 0.0 && u[5] == 0.0;
   const bool anti = u[0] == 0.0 && u[1] == 0.0 && u[6] == 0.0 && u[7] == 0.0;
-  if (L.pair) L.fast_kind = 0;
+  if (L.pair) L.fast_kind = L.solo >= 0 ? 5 : 0;
   else if (diag) L.fast_kind = 3;
   else if (L.target < 2) L.fast_kind = 1;
   else if (L.target < 7) L.fast_kind = 2;
-  else return false;
+  else L.fast_kind = 4;
   // Eq. matrix1 / matrix2 with the coefficient order of GateCoef: a term with a zero
   // coefficient contributes an exact zero, so summing every term gives the kept-term
   // sums' value (a zero result may differ in sign, and the encoder stores +0 for both)
@@ -593,7 +596,7 @@ static sim_status enqueue_gate(sim* s, const sim_gate* g) {
   }
   if (fast) {
     // the streaming kernel first; the general kernel then runs the items it left
-    const unsigned long long want = (L.items + qc::fast_pairs() - 1) / qc::fast_pairs();
+    const unsigned long long per = (unsigned long long)qc::fast_items(L.fast_kind), want = (L.items + per - 1ull) / per;
     const int fg = (unsigned long long)s->fast_grid < want ? s->fast_grid : (int)want;
     CK(qc::launch_gate_fast(L, fg, s->st), "streaming gate kernel launch");
     L.list = 1;

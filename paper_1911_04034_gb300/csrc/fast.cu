@@ -17,6 +17,13 @@
 //             offsets -> packing into the output window -> finished 16-byte blocks out
 //             to freshly allocated pages.
 //
+// An in-chunk target t >= 7 puts the partner 2^(t-7) passes on: those passes are held in
+// shared memory (kind 4; the general kernel took them before: 26-qubit QAOA layer, its
+// share of the general kernel fell from 13.1 ms to under 1).  A cross-chunk diagonal gate
+// with a row that is an exact copy (T, CZ, a controlled phase) gives a warp an item to
+// itself and rewrites one chunk of it (kind 5): a pair of warps would leave one idle
+// (30 qubits with kind 4: 591.8 -> 516.8 ms a layer; 21 qubits 121 -> 66 us a gate).
+//
 // Scans are warp shuffles and every carry between passes (stream offsets, the
 // predecessor's leading bytes, the encoder's predecessor) stays in registers, so the
 // kernel has no CTA-wide barrier; the warps of an SM overlap their FP64 arithmetic
@@ -43,14 +50,20 @@ constexpr int kFastThreads = 32 * kFastWarps;
 #endif
 constexpr uint32_t kFastWin = 1056;   // bytes of a pass window: 1024 bytes of stream at most, plus alignment and read slack
 constexpr uint32_t kWinBlocks = kFastWin / 16;
+constexpr size_t kSmSharedBytes = 227u * 1024u;
 constexpr uint32_t kWarpCache = 64;   // page ids a warp keeps between its items
 
 __host__ __device__ __forceinline__ uint32_t fast_pg_words(int kc) { return (max_pages(kc) + 3u) & ~3u; }
+// Passes held in a warp's exchange area: two for the partner warp (cross-chunk pairs);
+// for an in-chunk target t >= 7 the 2^(t-7) passes between an amplitude and its partner.
+__host__ __device__ __forceinline__ uint32_t fast_held(int kind, int target) {
+  return kind == 4 && target > 8 ? 1u << (target - 7) : 2u;
+}
 // Per warp (one chunk): two input windows, one output window, the input and the output
-// page ids, the values it shows its partner warp (two passes), its page cache, one
-// sample per lane of each pass of the chunk's first half.
-__host__ __device__ __forceinline__ uint32_t fast_warp_bytes(int kc) {
-  return 3u * kFastWin + 8u * fast_pg_words(kc) + 2u * 1024u + 4u * kWarpCache + 16u + (1u << (kc - 1));
+// page ids, the exchange area (1 KB a pass), its page cache, one sample per lane of each
+// pass of the chunk's first half.
+__host__ __device__ __forceinline__ uint32_t fast_warp_bytes(int kc, uint32_t held) {
+  return 3u * kFastWin + 8u * fast_pg_words(kc) + held * 1024u + 4u * kWarpCache + 16u + (1u << (kc - 1));
 }
 // Largest STREAM image of a chunk at S <= 32 bits.
 __host__ __device__ __forceinline__ uint32_t fast_max_image(int kc) {
@@ -415,16 +428,41 @@ __device__ __forceinline__ void row_op(const GateLaunch& L, uint32_t r, uint32_t
   }
 }
 
-// A pair of amplitudes (slots k0 < k1) held by the same lane: both outputs.
+// Both outputs of an ARITH 4 pair held by one lane.  The first sums of the four chains of
+// signed_rows are +-(ar + ai) and +-(ar - ai): two additions serve all four, 10 FP64
+// additions instead of 12 (a zero sum's sign may differ; a zero is stored as +0).
+__device__ __forceinline__ void signed_pair(const GateLaunch& L, uint32_t ar, uint32_t ai, uint32_t br, uint32_t bi,
+                                            uint32_t mh, uint32_t o[4], bool& spec) {
+  const uint32_t sg = L.sgn;
+  const double sum = __dadd_rn(hi_as_double(ar), hi_as_double(ai)), dif = __dsub_rn(hi_as_double(ar), hi_as_double(ai));
+  auto first = [&](int q, bool im) {
+    const uint32_t sx = (sg >> (im ? q + 1 : q)) << 31, sy = (sg >> (im ? q : q + 1)) << 31;  // signs of ar, ai
+    const double m = sx == sy ? sum : dif;
+    return __hiloint2double((int)((uint32_t)__double2hiint(m) ^ sx), __double2loint(m));
+  };
+  auto t = [&](int q, uint32_t h) { return hi_as_double(h ^ ((sg >> q) << 31)); };
+  auto scaled = [&](double y) -> uint32_t {
+    const uint32_t hi = (uint32_t)__double2hiint(y);
+    if (((hi << 1) | (uint32_t)__double2loint(y)) == 0u) return 0u;
+    spec |= (hi & 0x7ff00000u) == 0x7ff00000u;
+    return (hi + ((uint32_t)L.sk << 20)) & mh;
+  };
+#pragma unroll
+  for (int r = 0; r < 2; ++r) {
+    o[2 * r] = scaled(__dadd_rn(__dadd_rn(first(8 * r, false), t(8 * r + 2, br)), t(8 * r + 3, bi)));
+    o[2 * r + 1] = scaled(__dadd_rn(__dadd_rn(first(8 * r + 4, true), t(8 * r + 6, bi)), t(8 * r + 7, br)));
+  }
+}
+
+// A pair of amplitudes (a, b) held by the same lane, a at in-chunk index i: both outputs in
+// place, truncated.
 template <int ARITH>
-__device__ __forceinline__ void fast_pair_in_lane(const GateLaunch& L, uint32_t ibase, int k0, int k1, uint32_t v[8],
-                                                  uint32_t mh, bool& spec) {
-  const uint32_t ar = v[2 * k0], ai = v[2 * k0 + 1], br = v[2 * k1], bi = v[2 * k1 + 1];
+__device__ __forceinline__ void fast_pair(const GateLaunch& L, uint32_t i, uint32_t& ar, uint32_t& ai, uint32_t& br,
+                                          uint32_t& bi, uint32_t mh, bool& spec) {
   uint32_t o[4] = {ar & mh, ai & mh, br & mh, bi & mh};
-  if (((ibase + (uint32_t)k0) & L.lo_mask) == L.lo_vals) {
+  if ((i & L.lo_mask) == L.lo_vals) {
     if constexpr (ARITH == 4) {
-      signed_rows(L, 0u, ar, ai, br, bi, mh, o[0], o[1], spec);
-      signed_rows(L, 1u, ar, ai, br, bi, mh, o[2], o[3], spec);
+      signed_pair(L, ar, ai, br, bi, mh, o, spec);
     } else if constexpr (ARITH == 0 || ARITH == 3) {
       const double2 a = make_double2(hi_as_double(ar), hi_as_double(ai)), b = make_double2(hi_as_double(br), hi_as_double(bi));
       const double2 x = ARITH == 0 ? dense_rows(L.cf, a, b) : real_rows(L.cf, a, b);
@@ -438,10 +476,10 @@ __device__ __forceinline__ void fast_pair_in_lane(const GateLaunch& L, uint32_t 
       row_op(L, 1u, ar, ai, mh, o[2], o[3], spec);
     }
   }
-  v[2 * k0] = o[0];
-  v[2 * k0 + 1] = o[1];
-  v[2 * k1] = o[2];
-  v[2 * k1 + 1] = o[3];
+  ar = o[0];
+  ai = o[1];
+  br = o[2];
+  bi = o[3];
 }
 
 // Shared-memory buffers of one warp (its chunk of the pair's item).
@@ -451,11 +489,11 @@ struct FastWarp {
   uint32_t* owin;
   uint32_t* ipg;
   uint32_t* opg;
-  uint32_t* xch;  // [2][256]: the pass's decoded high words, for the partner warp
+  uint32_t* xch;  // [held passes][256]: decoded high words for the partner warp, or held for the partner pass
   uint32_t* half;  // [passes / 2][32]: one sample per lane of each first-half pass
 };
 
-__device__ __forceinline__ FastWarp fast_warp(uint8_t* base, int kc) {
+__device__ __forceinline__ FastWarp fast_warp(uint8_t* base, int kc, uint32_t held) {
   FastWarp f;
   f.iwin0 = reinterpret_cast<uint32_t*>(base);
   f.iwin1 = f.iwin0 + kFastWin / 4u;
@@ -463,12 +501,12 @@ __device__ __forceinline__ FastWarp fast_warp(uint8_t* base, int kc) {
   f.ipg = f.owin + kFastWin / 4u;
   f.opg = f.ipg + fast_pg_words(kc);
   f.xch = f.opg + fast_pg_words(kc);
-  f.half = f.xch + 512u + kWarpCache + 4u;
+  f.half = f.xch + 256u * held + kWarpCache + 4u;
   return f;
 }
 
-// One work item: this warp's chunk (side 0 or 1 of the pair).  Returns 0 when both
-// chunks were committed, 1 when the pair left the item to the general kernel (nothing
+// One work item: this warp's chunk (side 0 or 1 of the pair; kind 5: the warp alone, side =
+// the row that is not a copy).  Returns 0 when both chunks were committed, 1 when the pair left the item to the general kernel (nothing
 // of the state changed), 2 when the pair stops (a device error is set).
 // Per-phase SM cycles of a warp when profiling (lane 0 counts): 0 staging (directory
 // entries, headers, the partners' agreement, waits for input windows), 1 decoding, 2 the
@@ -503,6 +541,12 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
   // directory entry and header: a STREAM image at S <= 32, granted no selector trial
   uint32_t ib = 0, inp = 0, Sin = 0, bits_in = 0;
   bool ok = whole && (!L.sel_dec || L.sel_dec[2ull * item + side] == 0u);
+  if constexpr (KIND == 5) {
+    // the other chunk of the item: an exact copy of itself, whose image stays if it is what
+    // the encoder would write (its reading overlaps with this chunk's)
+    if (L.sel_dec) ok = ok && L.sel_dec[2ull * item + (side ^ 1u)] == 0u;
+    ok = ok && image_stands(P, ch ^ L.pair_bit, S, kDefaultModes);
+  }
   if (ok) {
     const uint32_t* e = dir_entry(P, ch);
     const uint2 h = *reinterpret_cast<const uint2*>(e);
@@ -531,23 +575,14 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
   unsigned int err = 0;
   if (lane == 0) err = *(volatile unsigned int*)&P.ctl->err;
   err = __shfl_sync(0xffffffffu, err, 0);
-  {
+  if constexpr (KIND == 5) {  // the warp has the item to itself
+    if (err) return 2;
+    if (!ok) return 1;
+  } else {
     const uint32_t mine = (ok ? 1u : 0u) | (err ? 2u : 0u);
     const uint32_t other = pair_agree(slots, seq, phase, side, mine, P.ctl, 1u);
     if ((mine | other) & 2u) return 2;
     if (!((mine & other) & 1u)) return 1;
-  }
-  if constexpr (KIND == 0 && ARITH == 1) {
-    // A diagonal row that is an exact copy (T's and CZ's first row) leaves this chunk's
-    // values as they are; already coded at the gate's S, they would be re-encoded to the
-    // same bytes (truncation is idempotent, and the smallest-image choice sees the same
-    // values), so the image stays and the warp only joins the pair's final agreement
-    // (there are no meetings in between for a diagonal gate).
-    if (L.rop[side] == 1 && Sin == S) {
-      const uint32_t other = pair_agree(slots, seq, phase, side, 1u, P.ctl, 3u);
-      if (other & 2u) return 2;
-      return (other & 1u) ? 0 : 1;
-    }
   }
   const uint32_t nbs = (ib - 16u - cb) >> 4;
   // the code word of this lane's values in pass p (image byte 16 + 64 p + 4 (lane / 2))
@@ -567,7 +602,15 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
   const uint32_t mh = (uint32_t)(trunc_mask(S) >> 32), mhin = (uint32_t)(trunc_mask(Sin) >> 32);
   uint32_t ioff = 0u, ooff = 0u, lead = 0u, prv = 0u, refr = 0u, refi = 0u, nzor = 0u;
   bool spec = false, cst = true, halves = true, lost = false;
-  for (uint32_t p = 0; p < NP; ++p) {
+  // KIND 4: an amplitude's partner lies `dist` passes on.  In each group of 2 dist passes,
+  // dist steps decode and hold the first half, dist steps decode the second half, form
+  // both outputs, encode the first half's and hold the second's, dist steps encode those.
+  const uint32_t dist = KIND == 4 ? 1u << (L.target - 7) : 0u;
+  uint32_t step = 0u, pdec = 0u, penc = 0u;  // the step in its group, passes decoded and encoded
+  while (penc < NP) {
+    uint32_t v[8];
+    if (KIND != 4 || step < 2u * dist) {
+    const uint32_t p = pdec;
     uint32_t* const win = (p & 1u) ? fw.iwin1 : fw.iwin0;
     uint32_t* const wnext = (p & 1u) ? fw.iwin0 : fw.iwin1;
     // residual lengths of this lane's 8 values, their offsets in the pass
@@ -585,7 +628,6 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
     __syncwarp();
     ph.mark(0);
     // explicit parts, leading bytes from the predecessors
-    uint32_t v[8];
     {
       const uint32_t W = fast_extract(win, 4u * (ps >> 7), o, cw, Sin, mhin, v);
       uint32_t after;
@@ -600,6 +642,33 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
       for (int k = 0; k < 8; ++k) spec |= ((v[k] & 0x7fffffffu) - 1u) < ((64u << 20) - 1u);  // nonzero, exponent < 64
     }
     ph.mark(1);
+    ++pdec;
+    }
+    if constexpr (KIND == 4) {
+      const uint32_t at = step++;
+      if (step == 3u * dist) step = 0u;
+      uint4* const hold = reinterpret_cast<uint4*>(fw.xch) + 64u * (at & (dist - 1u));
+      const uint4 h0 = hold[lane], h1 = hold[32u + lane];
+      if (at >= dist) {
+        uint32_t a[8] = {h0.x, h0.y, h0.z, h0.w, h1.x, h1.y, h1.z, h1.w};
+        if (at < 2u * dist) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k)
+            fast_pair<ARITH>(L, 128u * penc + 4u * lane + (uint32_t)k, a[2 * k], a[2 * k + 1], v[2 * k], v[2 * k + 1], mh, spec);
+        }
+        if (at < 2u * dist) {
+          hold[lane] = make_uint4(v[0], v[1], v[2], v[3]);
+          hold[32u + lane] = make_uint4(v[4], v[5], v[6], v[7]);
+        }
+#pragma unroll
+        for (int k = 0; k < 8; ++k) v[k] = a[k];
+      } else {
+        hold[lane] = make_uint4(v[0], v[1], v[2], v[3]);
+        hold[32u + lane] = make_uint4(v[4], v[5], v[6], v[7]);
+        continue;
+      }
+    }
+    const uint32_t p = penc++;
     // the gate on every amplitude pair whose in-chunk control bits match; results
     // truncated to S bits in place
     const uint32_t ibase = 128u * p + 4u * lane;  // the lane's first amplitude in the chunk
@@ -608,12 +677,12 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
       // the partner warp holds the other amplitude of every pair, at the same position
       // (a diagonal gate needs only the amplitude itself)
       uint32_t* xs = fw.xch + 256u * (p & 1u);
-      reinterpret_cast<uint4*>(xs)[2u * lane] = make_uint4(v[0], v[1], v[2], v[3]);
-      reinterpret_cast<uint4*>(xs)[2u * lane + 1u] = make_uint4(v[4], v[5], v[6], v[7]);
+      reinterpret_cast<uint4*>(xs)[lane] = make_uint4(v[0], v[1], v[2], v[3]);
+      reinterpret_cast<uint4*>(xs)[32u + lane] = make_uint4(v[4], v[5], v[6], v[7]);
       ++phase;
       if (!lost) lost = !pair_sync(seq, side, phase, P.ctl, 2u);
       const uint32_t* xo = xpeer + 256u * (p & 1u);
-      const uint4 w0 = reinterpret_cast<const uint4*>(xo)[2u * lane], w1 = reinterpret_cast<const uint4*>(xo)[2u * lane + 1u];
+      const uint4 w0 = reinterpret_cast<const uint4*>(xo)[lane], w1 = reinterpret_cast<const uint4*>(xo)[32u + lane];
       w[0] = w0.x; w[1] = w0.y; w[2] = w0.z; w[3] = w0.w; w[4] = w1.x; w[5] = w1.y; w[6] = w1.z; w[7] = w1.w;
     } else if constexpr (KIND == 2) {
       // partner amplitude i ^ 2^t (2 <= t <= 6): the same slot of lane ^ 2^(t-2)
@@ -623,22 +692,22 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
     if constexpr (KIND == 1) {
       // partner in the lane: amplitudes k and k ^ 2^t, t = 0 or 1
       if (L.target == 0) {
-        fast_pair_in_lane<ARITH>(L, ibase, 0, 1, v, mh, spec);
-        fast_pair_in_lane<ARITH>(L, ibase, 2, 3, v, mh, spec);
+        fast_pair<ARITH>(L, ibase, v[0], v[1], v[2], v[3], mh, spec);
+        fast_pair<ARITH>(L, ibase + 2u, v[4], v[5], v[6], v[7], mh, spec);
       } else {
-        fast_pair_in_lane<ARITH>(L, ibase, 0, 2, v, mh, spec);
-        fast_pair_in_lane<ARITH>(L, ibase, 1, 3, v, mh, spec);
+        fast_pair<ARITH>(L, ibase, v[0], v[1], v[4], v[5], mh, spec);
+        fast_pair<ARITH>(L, ibase + 1u, v[2], v[3], v[6], v[7], mh, spec);
       }
-    } else {
+    } else if constexpr (KIND != 4) {
       // which row pair this lane's amplitudes take: the pair's second amplitude (b) takes
-      // rows 2-3 (kind 0: the second warp; kind 2: lanes with bit t - 2 set; kind 3 per
-      // amplitude, bit t)
-      const uint32_t lane_row = KIND == 0 ? side : (KIND == 2 ? ((lane >> (L.target - 2)) & 1u) : 0u);
+      // rows 2-3 (kinds 0 and 5: the chunk with the target bit; kind 2: lanes with bit t - 2
+      // set; kind 3 per amplitude, bit t)
+      const uint32_t lane_row = KIND == 0 || KIND == 5 ? side : (KIND == 2 ? ((lane >> (L.target - 2)) & 1u) : 0u);
 #pragma unroll
       for (int k = 0; k < 4; ++k) {
         const uint32_t i = ibase + (uint32_t)k;
         const uint32_t row = KIND == 3 ? ((i >> L.target) & 1u) : lane_row;
-        const uint32_t i0 = i & ~(1u << (KIND == 0 ? 31u : (uint32_t)L.target));
+        const uint32_t i0 = i & ~(1u << (KIND == 0 || KIND == 5 ? 31u : (uint32_t)L.target));
         uint32_t outr = v[2 * k] & mh, outi = v[2 * k + 1] & mh;  // unchanged amplitude, truncated
         if ((i0 & L.lo_mask) == L.lo_vals) {
           if constexpr (ARITH == 4) {
@@ -735,7 +804,7 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
   const bool keep = !any_spec && !all_cst && any_nz && !all_halves;
   if (corrupt && lane == 0) atomicOr(&P.ctl->err, (unsigned)E_CORRUPT);
   const uint32_t mine = (keep ? 1u : 0u) | ((corrupt || oom || lost) ? 2u : 0u);
-  const uint32_t other = lost ? 2u : pair_agree(slots, seq, phase, side, mine, P.ctl, 3u);
+  const uint32_t other = KIND == 5 ? mine : (lost ? 2u : pair_agree(slots, seq, phase, side, mine, P.ctl, 3u));
   if (((mine | other) & 2u) || !((mine & other) & 1u)) {
     wp_free(P, wp, fw.opg, onp);
     cp_async_wait_all();
@@ -749,8 +818,7 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
   uint32_t* e = dir_entry(P, ch);
   for (uint32_t k = lane; k < onp; k += 32u) e[4 + k] = fw.opg[k];
   if (lane == 0) {
-    e[0] = bytes;
-    e[1] = onp;
+    *reinterpret_cast<uint4*>(e) = make_uint4(bytes, onp, kDefaultModes, 0u);
     dE += (long long)bytes - (long long)ib;
     rd += ib;
     wr += bytes;
@@ -767,7 +835,7 @@ __global__ void __launch_bounds__(kFastThreads, QC_FAST_MIN_CTAS) k_gate_fast(co
   __shared__ uint32_t s_seq[kFastPairs][2];
   const int kc = L.P.kc;
   const uint32_t lane = threadIdx.x & 31u, wid = threadIdx.x >> 5;
-  const uint32_t pr = wid >> 1, side = wid & 1u;
+  const uint32_t pr = wid >> 1, side = KIND == 5 ? (uint32_t)L.solo : wid & 1u;
   if (threadIdx.x < 2u * kFastPairs) s_seq[threadIdx.x >> 1][threadIdx.x & 1u] = 0u;
   __syncthreads();  // the only CTA-wide barrier: every sequence number starts at 0
   DevCtl* ctl = L.P.ctl;
@@ -776,12 +844,13 @@ __global__ void __launch_bounds__(kFastThreads, QC_FAST_MIN_CTAS) k_gate_fast(co
     if (blockIdx.x == 0 && threadIdx.x == 0) ctl->fast_all = 1u;
     return;
   }
-  uint8_t* wb = smem + (size_t)wid * fast_warp_bytes(kc);
-  const FastWarp fw = fast_warp(wb, kc);
-  const uint32_t* xpeer = fast_warp(smem + (size_t)(wid ^ 1u) * fast_warp_bytes(kc), kc).xch;
+  const uint32_t held = fast_held(KIND, L.target);
+  uint8_t* wb = smem + (size_t)wid * fast_warp_bytes(kc, held);
+  const FastWarp fw = fast_warp(wb, kc, held);
+  const uint32_t* xpeer = fast_warp(smem + (size_t)(wid ^ 1u) * fast_warp_bytes(kc, held), kc, held).xch;
   // the warp's page cache, kept in global memory between launches
   WarpPages wp;
-  wp.ids = fw.xch + 512u;
+  wp.ids = fw.xch + 256u * held;
   wp.n = wp.ids + kWarpCache;
   const size_t gw = (size_t)blockIdx.x * kFastWarps + wid;
   const uint32_t n_start = L.P.wcache_n[gw];
@@ -802,17 +871,19 @@ __global__ void __launch_bounds__(kFastThreads, QC_FAST_MIN_CTAS) k_gate_fast(co
   }
   long long dE = 0;
   unsigned long long rd = 0, wr = 0, done = 0, deferred = 0;
-  const unsigned long long pairs = (unsigned long long)gridDim.x * kFastPairs;
-  for (unsigned long long item = (unsigned long long)blockIdx.x * kFastPairs + pr; item < L.items; item += pairs) {
+  constexpr bool solo = KIND == 5;  // an item per warp instead of per pair of warps
+  const unsigned long long pairs = (unsigned long long)gridDim.x * (solo ? kFastWarps : kFastPairs);
+  for (unsigned long long item = (unsigned long long)blockIdx.x * (solo ? kFastWarps : kFastPairs) + (solo ? wid : pr);
+       item < L.items; item += pairs) {
     const int r = fast_item<KIND, ARITH>(L, item, S, fw, xpeer, wp, side, s_seq[pr], s_slots[pr], phase, dE, rd, wr, ph);
     if (r == 2) break;
     if (r == 1) {
-      if (side == 0 && lane == 0) {
+      if ((solo || side == 0) && lane == 0) {
         const unsigned long long k = atomicAdd(&ctl->ndefer, 1ull);
         L.defer[k] = (uint32_t)item;
         ++deferred;
       }
-    } else if (side == 0) {
+    } else if (solo || side == 0) {
       ++done;
     }
   }
@@ -845,14 +916,14 @@ static cudaError_t prep_fast(K kernel, size_t smem) {
   return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
 }
 
-size_t fast_smem_bytes(int kc) { return (size_t)kFastWarps * fast_warp_bytes(kc); }
+static size_t fast_smem_bytes(int kc, uint32_t held) { return (size_t)kFastWarps * fast_warp_bytes(kc, held); }
 int fast_warps() { return kFastWarps; }
-int fast_pairs() { return kFastPairs; }
+int fast_items(int kind) { return kind == 5 ? kFastWarps : kFastPairs; }
 int fast_warp_cache() { return (int)kWarpCache; }
 
 int fast_ctas_per_sm(int kc) {
   int n = 0;
-  const size_t smem = fast_smem_bytes(kc);
+  const size_t smem = fast_smem_bytes(kc, 2u);
   prep_fast(k_gate_fast<0, 0>, smem);
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, k_gate_fast<0, 0>, kFastThreads, smem) != cudaSuccess || n < 1)
     n = 1;
@@ -868,9 +939,13 @@ static cudaError_t launch_fast_as(const GateLaunch& L, int grid, size_t smem, cu
 }
 
 // Kinds and arithmetic forms that occur: cross-chunk pairs of any gate class, in-chunk
-// partners of dense, real, power-of-two or anti-diagonal gates, in-chunk diagonal gates.
+// partners of dense, real, power-of-two or anti-diagonal gates, in-chunk diagonal gates,
+// cross-chunk diagonal gates with a row that is an exact copy.
 cudaError_t launch_gate_fast(const GateLaunch& L, int grid, cudaStream_t st) {
-  const size_t smem = fast_smem_bytes(L.P.kc);
+  const uint32_t held = fast_held(L.fast_kind, L.target);
+  const size_t smem = fast_smem_bytes(L.P.kc, held);
+  // held passes take shared memory: no more CTAs than fit at once
+  if (held > 2u) grid = min(grid, num_sms() * max(1, (int)(kSmSharedBytes / (smem + 2048u))));
   switch (L.fast_kind * 8 + L.arith) {
     case 0: return launch_fast_as<0, 0>(L, grid, smem, st);
     case 1: return launch_fast_as<0, 1>(L, grid, smem, st);
@@ -886,6 +961,11 @@ cudaError_t launch_gate_fast(const GateLaunch& L, int grid, cudaStream_t st) {
     case 19: return launch_fast_as<2, 3>(L, grid, smem, st);
     case 20: return launch_fast_as<2, 4>(L, grid, smem, st);
     case 25: return launch_fast_as<3, 1>(L, grid, smem, st);
+    case 32: return launch_fast_as<4, 0>(L, grid, smem, st);
+    case 34: return launch_fast_as<4, 2>(L, grid, smem, st);
+    case 35: return launch_fast_as<4, 3>(L, grid, smem, st);
+    case 36: return launch_fast_as<4, 4>(L, grid, smem, st);
+    case 41: return launch_fast_as<5, 1>(L, grid, smem, st);
     default: return cudaErrorInvalidValue;
   }
 }

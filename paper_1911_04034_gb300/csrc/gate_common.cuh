@@ -29,4 +29,27 @@ __device__ __forceinline__ unsigned long long item_chunk(const GateLaunch& L, un
   return out;
 }
 
+// True if the chunk's image is what the encoder would write of its values at S bits under
+// `modes`: rewriting it unchanged can be left out.  Word 2 of a directory entry holds the
+// mode set its image was chosen from (0: unknown); the smallest image of a larger set is
+// the smallest of any subset that has it, and coding decoded values again at the same
+// width gives the same bytes.  `hdr`: the image's first header word.
+__device__ __forceinline__ bool entry_stands(const Pool& P, const uint32_t* e, uint32_t S, uint32_t modes,
+                                             uint32_t& hdr) {
+  const uint4 h = *reinterpret_cast<const uint4*>(e);
+  const uint32_t first = e[4];
+  hdr = first;
+  if ((modes & kDefaultModes) != kDefaultModes || (h.z & modes) != modes) return false;
+  if (h.y != 0u) {
+    if (first >= P.npages) return false;
+    hdr = *reinterpret_cast<const uint32_t*>(P.pages + (unsigned long long)first * kPage);
+  }
+  const uint32_t mode = hdr & 0xffu;
+  return mode < M_NMODES && ((modes >> mode) & 1u) != 0u && (mode == M_ZERO || ((hdr >> 8) & 0xffu) == S);
+}
+__device__ __forceinline__ bool image_stands(const Pool& P, unsigned long long chunk, uint32_t S, uint32_t modes) {
+  uint32_t hdr;
+  return entry_stands(P, dir_entry(P, chunk), S, modes, hdr);
+}
+
 }  // namespace qc

@@ -88,7 +88,8 @@ __device__ __forceinline__ void fence_to_bulk() { asm volatile("fence.proxy.asyn
 // call it; the images in shared memory must stay untouched until bulk_wait_read.
 __device__ __forceinline__ void commit_images(const Pool& P, unsigned long long c0, const uint8_t* img0, uint32_t n0,
                                               const uint32_t* pg0, uint32_t np0, bool has1, unsigned long long c1,
-                                              const uint8_t* img1, uint32_t n1, const uint32_t* pg1, uint32_t np1) {
+                                              const uint8_t* img1, uint32_t n1, const uint32_t* pg1, uint32_t np1,
+                                              uint32_t md0, uint32_t md1) {
   if (threadIdx.x < 32u) {
     const uint32_t tot = np0 + (has1 ? np1 : 0u);
     bool issued = false;
@@ -114,10 +115,7 @@ __device__ __forceinline__ void commit_images(const Pool& P, unsigned long long 
       } else {
         for (uint32_t q = lane; q < np; q += 32u) e[4 + q] = pg[q];
       }
-      if (lane == 0) {
-        e[0] = bytes;
-        e[1] = np;
-      }
+      if (lane == 0) *reinterpret_cast<uint4*>(e) = make_uint4(bytes, np, w ? md1 : md0, 0u);
     }
   }
 }
@@ -217,13 +215,15 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
   const bool have_entries = PREF && st.next_item == item;
   if (PREF && st.next_item != ~0ull) st.cur ^= 1;
   st.next_item = ~0ull;
-  uint32_t* const ent0 = m.ent[st.cur][0];
+  uint32_t* ent0 = m.ent[st.cur][0];
   uint32_t* const ent1 = m.ent[st.cur][1];
+  bool solo = false;  // only the chunk of row L.solo is rewritten: it takes the place of the first
   // the item's chunks (recomputed at commit rather than kept through the codec)
   auto chunks_of = [&](unsigned long long& x0, unsigned long long& x1) {
     if (L.pair) {
       x0 = item_chunk(L, item) | L.hi_vals;
       x1 = x0 | L.pair_bit;
+      if (solo && L.solo == 1) x0 = x1;
     } else {
       x0 = item_chunk(L, 2ull * item) | L.hi_vals;
       x1 = 2ull * item + 1 < L.nact ? (item_chunk(L, 2ull * item + 1) | L.hi_vals) : 0ull;
@@ -231,7 +231,7 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
   };
   unsigned long long c0, c1;
   chunks_of(c0, c1);
-  const bool has1 = L.pair || 2ull * item + 1 < L.nact;
+  bool has1 = L.pair || 2ull * item + 1 < L.nact;
   // stage 1: both directory entries (warp 0 and warp 1), unless prefetched
   if (!have_entries) {
     if (threadIdx.x < 32u) {
@@ -268,8 +268,8 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
     cp_async_commit();
     st.next_item = nx;
   }
-  const uint32_t np0 = ent0[1], np1 = has1 ? ent1[1] : 0u;
-  const uint32_t b0 = ent0[0], b1 = has1 ? ent1[0] : 0u;
+  uint32_t np0 = ent0[1], np1 = has1 ? ent1[1] : 0u;
+  uint32_t b0 = ent0[0], b1 = has1 ? ent1[0] : 0u;
   if (b0 > cap || b1 > cap || np0 > max_pages(kc) || np1 > max_pages(kc) || (np0 == 0u && b0 > inline_cap(kc)) ||
       (np1 == 0u && b1 > inline_cap(kc)) || (b0 & 15u) || (b1 & 15u)) {
     if (threadIdx.x == 0) atomicOr(&ctl->err, (unsigned)E_CORRUPT);
@@ -279,8 +279,8 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
   // stored as +0), and its image does not depend on the bound: skip it.
   const bool z0 = np0 == 0 && b0 == 16u && ent0[4] == 0u;
   const bool z1 = !has1 || (np1 == 0 && b1 == 16u && ent1[4] == 0u);
-  if (threadIdx.x == 0) st.acc->rd += b0 + b1;
   if (z0 && z1) {
+    if (threadIdx.x == 0) st.acc->rd += b0 + b1;
     QC_PHASE(5);
     return true;
   }
@@ -290,6 +290,7 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
   if (L.pair && L.lo_mask == 0u && inline_cap(kc) >= 32u && np0 == 0u && np1 == 0u &&
       (z0 || (ent0[4] & 0xffu) == M_CONST) && (z1 || (ent1[4] & 0xffu) == M_CONST)) {
     if (threadIdx.x == 0) {
+      st.acc->rd += b0 + b1;
       double2 a = make_double2(0.0, 0.0), b = make_double2(0.0, 0.0);
       if (!z0) a = make_double2(__longlong_as_double(((const long long*)(ent0 + 8))[0]),
                                 __longlong_as_double(((const long long*)(ent0 + 8))[1]));
@@ -310,6 +311,7 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
         }
         w0[0] = n0;
         w1[0] = n1;
+        w0[2] = w1[2] = L.modes;
         st.acc->dE += (long long)n0 + (long long)n1 - (long long)b0 - (long long)b1;
         auto wide = [](uint32_t h) { return ((h >> 8) & 0xffu) == 64u ? 1ll : 0ll; };
         st.acc->dn64 += wide(h0[0]) + wide(h1[0]) - (z0 ? 0ll : wide(ent0[4])) - (z1 ? 0ll : wide(ent1[4]));
@@ -319,6 +321,44 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
     QC_PHASE(5);
     return true;
   }
+  // chunk modes: the mode set, or Solution C's set plus the trials the selector granted
+  uint32_t md0 = L.modes, md1 = L.modes;
+  if (L.sel_dec) {
+    md0 = sel_modes(L.sel_dec[2ull * item]);
+    md1 = has1 ? sel_modes(L.sel_dec[2ull * item + 1ull]) : kDefaultModes;
+  }
+  // A diagonal gate between chunks whose other row is an exact copy (T, CZ, a controlled
+  // phase): the copy's image stays, if it is what the encoder would write, and only the
+  // other chunk is decoded and encoded: half the item's codec work.
+  if (L.solo >= 0 && !L.bc && !L.trace) {
+    uint32_t hdr;
+    solo = entry_stands(P, L.solo ? ent0 : ent1, S, L.solo ? md0 : md1, hdr);
+  }
+  if (solo) {
+    const uint32_t mdc = L.solo ? md0 : md1;  // the copy would have run these trials
+    if (threadIdx.x == 0) {
+      if ((mdc >> M_SPLIT) & 1u) atomicAdd(&ctl->split_trials, 1ull);
+      if ((mdc >> M_PALETTE) & 1u) atomicAdd(&ctl->palette_trials, 1ull);
+    }
+    if (L.solo) {
+      ent0 = ent1;
+      np0 = np1;
+      b0 = b1;
+      md0 = md1;
+    }
+    has1 = false;
+    np1 = b1 = 0u;
+    if (L.solo ? z1 : z0) {  // zeros stay zeros; their trials are counted as above
+      if (threadIdx.x == 0) {
+        st.acc->rd += b0;
+        if ((md0 >> M_SPLIT) & 1u) atomicAdd(&ctl->split_trials, 1ull);
+        if ((md0 >> M_PALETTE) & 1u) atomicAdd(&ctl->palette_trials, 1ull);
+      }
+      QC_PHASE(5);
+      return true;
+    }
+  }
+  if (threadIdx.x == 0) st.acc->rd += b0 + b1;
   // stage 2: both images in one pass (inline ones from the entry copies); page data is
   // copied asynchronously, so every copy of the thread is in flight at once
   {
@@ -343,7 +383,8 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
   // the next item's pages into L2: warp 0 for its first chunk, warp 1 for its second
   // (each warp waits only for the entry copies it issued itself)
   auto prefetch_next = [&]() {
-    if (PREF && st.next_item != ~0ull && threadIdx.x < 64u && (threadIdx.x < 32u || nhas1)) {
+    if (PREF && st.next_item != ~0ull && threadIdx.x < 64u && (threadIdx.x < 32u || nhas1) &&
+        !(solo && (int)(threadIdx.x >> 5) != L.solo)) {
       cp_async_wait_all();
       __syncwarp();
       const uint32_t* e = m.ent[st.cur ^ 1][threadIdx.x >> 5];
@@ -430,7 +471,14 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
   // apply the gate to every amplitude pair whose in-chunk control bits match
   double2* t0 = reinterpret_cast<double2*>(m.tile0);
   double2* t1 = reinterpret_cast<double2*>(m.tile1);
-  if (L.pair) {
+  if (solo) {
+    const double2 z = make_double2(0.0, 0.0);  // the other amplitude has a zero coefficient
+    for (uint32_t i = threadIdx.x; i < A; i += kThreads) {
+      if ((i & L.lo_mask) != L.lo_vals) continue;
+      const uint32_t pi = tile_amp(i);
+      t0[pi] = L.solo ? apply_rows23(L.g, z, t0[pi]) : apply_rows01(L.g, t0[pi], z);
+    }
+  } else if (L.pair) {
     for (uint32_t i = threadIdx.x; i < A; i += kThreads) {
       if ((i & L.lo_mask) != L.lo_vals) continue;
       const uint32_t pi = tile_amp(i);
@@ -456,12 +504,6 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
   }
   __syncthreads();
   QC_PHASE(2);
-  // chunk modes: the mode set, or Solution C's set plus the trials the selector granted
-  uint32_t md0 = L.modes, md1 = L.modes;
-  if (L.sel_dec) {
-    md0 = sel_modes(L.sel_dec[2ull * item]);
-    md1 = has1 ? sel_modes(L.sel_dec[2ull * item + 1ull]) : kDefaultModes;
-  }
   SelCtx sel;
   sel.gfeat = L.gfeat;
   sel.S_gate = S;
@@ -532,7 +574,7 @@ __device__ __forceinline__ bool gate_item(const GateLaunch& L, unsigned long lon
   {
     unsigned long long x0, x1;
     chunks_of(x0, x1);
-    commit_images(P, x0, m.img0, n0, ent0 + 4, m.np[0], has1, x1, m.img1, n1, ent1 + 4, m.np[1]);
+    commit_images(P, x0, m.img0, n0, ent0 + 4, m.np[0], has1, x1, m.img1, n1, ent1 + 4, m.np[1], md0, md1);
   }
   if (threadIdx.x == 0) {
     const uint32_t i0 = ent0[0], i1 = has1 ? ent1[0] : 0u;  // the old image lengths (entry copies)
@@ -757,7 +799,8 @@ __global__ void k_pool_init(const Pool P, unsigned long long nchunks) {
     uint32_t* e = dir_entry(P, c);
     e[0] = 16u;
     e[1] = 0u;
-    e[2] = e[3] = 0u;
+    e[2] = kAllModes;  // a ZERO image under any mode set
+    e[3] = 0u;
     e[4] = e[5] = e[6] = e[7] = 0u;
   }
 }
@@ -796,6 +839,7 @@ __global__ void __launch_bounds__(kThreads) k_init_chunk0(const Pool P, unsigned
   __syncthreads();
   if (!s_ok) return;
   store_image_block(P, 0ull, img, n0, pages, s_np);
+  if (threadIdx.x == 0) dir_entry(P, 0ull)[2] = kDefaultModes;
   if (threadIdx.x == 0) {
     P.ctl->E = 16ull * (nchunks - 1ull) + n0;
     P.ctl->Emax = P.ctl->E;
@@ -1054,7 +1098,7 @@ __global__ void k_ck_stack(const Pool P, unsigned long long used) {
 }
 
 // ------------------------------------------------------------- launchers -- //
-static int num_sms() {
+int num_sms() {
   static int sms = 0;
   if (!sms) {
     int dev = 0;

@@ -36,7 +36,9 @@ struct GateLaunch {
   uint8_t* bc;                   // block cache lines (kBcLines of bc_line_bytes) or nullptr
   uint32_t* defer;               // streaming kernel: items left to the general kernel (device list)
   int fast_kind;                 // streaming kernel: 0 cross-chunk pairs, 1 in-chunk target < 2, 2 in-chunk
-                                 // target 2..6 (partner in another lane), 3 in-chunk diagonal gate
+                                 // target 2..6 (partner in another lane), 3 in-chunk diagonal gate, 4 in-chunk
+                                 // target >= 7 (partner in another pass), 5 cross-chunk diagonal with a copy row
+  int solo;                      // cross-chunk diagonal gate with a row that is an exact copy: the other row, else -1
   int list;                      // general kernel: 1 = run the items the streaming kernel left
   // streaming kernel arithmetic (the same values as the kept-term sums of GateCoef):
   int arith;                     // 0 dense: the four sums with every coefficient, zeros included;
@@ -66,6 +68,7 @@ void set_last_error(const char* msg);
 // lossless stage); -1 for a bound outside {0} U [2^-52, 1).
 int sig_bits_of(double eps);
 
+int num_sms();
 int vpt_for(int kc);
 size_t gate_smem_bytes(int kc);
 size_t codec_smem_bytes(int kc);
@@ -77,7 +80,7 @@ cudaError_t launch_gate(const GateLaunch& L, int grid, cudaStream_t st);
 constexpr int kFastMinKC = 7;
 int fast_ctas_per_sm(int kc);
 int fast_warps();        // warps per CTA of the streaming kernel (a pair of warps per work item)
-int fast_pairs();        // work items a CTA of the streaming kernel runs at once
+int fast_items(int kind); // work items a CTA of the streaming kernel runs at once
 int fast_warp_cache();   // page ids each of its warps may hold
 cudaError_t launch_gate_fast(const GateLaunch& L, int grid, cudaStream_t st);
 cudaError_t launch_post(const Pool& P, const CtlParams& cp, int grid_ctas, cudaStream_t st);
