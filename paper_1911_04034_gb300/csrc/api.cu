@@ -570,10 +570,19 @@ static bool fast_applies(const sim* s, const sim_gate* g, GateLaunch& L) {
   return true;
 }
 
+// True if the gate is X between chunks with no control inside a chunk: whole images change
+// places (see k_swap).  Not where every item must be looked up (block cache), recorded
+// (traces) or decided anew (selector network).
+static bool swap_applies(const sim* s, const sim_gate* g, const GateLaunch& L) {
+  const double* u = g->u;
+  return s->fast && L.pair && L.lo_mask == 0u && !L.sel_dec && !L.bc && !L.trace && u[0] == 0.0 && u[1] == 0.0 &&
+         u[2] == 1.0 && u[3] == 0.0 && u[4] == 1.0 && u[5] == 0.0 && u[6] == 0.0 && u[7] == 0.0;
+}
+
 static sim_status enqueue_gate(sim* s, const sim_gate* g) {
   GateLaunch L = make_launch(s, g);
   const int grid = (uint64_t)s->grid < L.items ? s->grid : (int)L.items;
-  const bool fast = fast_applies(s, g, L);
+  const bool swap = swap_applies(s, g, L), fast = !swap && fast_applies(s, g, L);
   L.defer = s->d_defer;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (s->timing) {
@@ -592,6 +601,11 @@ static sim_status enqueue_gate(sim* s, const sim_gate* g) {
     const unsigned long long want = (n + 255ull) / 256ull;
     const int sg = (unsigned long long)s->grid < want ? s->grid : (int)want;
     CK(qc::launch_select(L, s->d_mlp, s->d_dec, sg, s->st), "selector kernel launch");
+    s->kernel_launches += 1;
+  }
+  if (swap) {
+    CK(qc::launch_swap(L, s->st), "image swap kernel launch");
+    L.list = 1;
     s->kernel_launches += 1;
   }
   if (fast) {

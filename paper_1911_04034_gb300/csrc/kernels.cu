@@ -664,6 +664,53 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : QC_GATE_MIN_CTAS)
   if (cur >= 0) cta_end(jobs[cur].L, st, s_ph);
 }
 
+// X between chunks (a cross-chunk target, both rows exact copies, no control inside a
+// chunk): every amplitude of one chunk takes its partner's place in the other, so two
+// images that stand as the encoder would write them are exchanged by exchanging their
+// directory entries; any other item is left to the general kernel.  A warp per item, bound
+// by directory traffic.  18 qubits, 2^10-amplitude chunks: 22 us a
+// gate decoded and encoded by the streaming kernel, 3.1 us exchanged.
+__global__ void __launch_bounds__(256) k_swap(const __grid_constant__ GateLaunch L) {
+  const Pool& P = L.P;
+  DevCtl* ctl = P.ctl;
+  if (*(volatile unsigned int*)&ctl->err != 0u) return;
+  const uint32_t lane = threadIdx.x & 31u, dw4 = P.dir_words / 4u;
+  const uint32_t S = gate_bits(L);
+  const unsigned long long warps = (unsigned long long)gridDim.x * (blockDim.x >> 5);
+  unsigned long long done = 0, left = 0, coded = 0;
+  for (unsigned long long item = (unsigned long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5); item < L.items;
+       item += warps) {
+    const unsigned long long c0 = item_chunk(L, item) | L.hi_vals;
+    uint32_t* const e0 = dir_entry(P, c0);
+    uint32_t* const e1 = dir_entry(P, c0 | L.pair_bit);
+    uint32_t h0, h1;
+    const bool s0 = entry_stands(P, e0, S, L.modes, h0), s1 = entry_stands(P, e1, S, L.modes, h1);
+    if (s0 && s1) {
+      // the trials a re-encoding would have counted (none for two constant chunks held inline)
+      if ((h0 & 0xffu) > M_CONST || (h1 & 0xffu) > M_CONST || (e0[1] | e1[1]) != 0u) coded += 2ull;
+      __syncwarp();  // every lane has read what the exchange overwrites
+      for (uint32_t i = lane; i < dw4; i += 32u) {
+        const uint4 a = reinterpret_cast<const uint4*>(e0)[i], b = reinterpret_cast<const uint4*>(e1)[i];
+        reinterpret_cast<uint4*>(e0)[i] = b;
+        reinterpret_cast<uint4*>(e1)[i] = a;
+      }
+      ++done;
+    } else {
+      if (lane == 0) L.defer[atomicAdd(&ctl->ndefer, 1ull)] = (uint32_t)item;
+      ++left;
+    }
+    __syncwarp();
+  }
+  if (lane == 0) {
+    if (S <= 32u) {
+      if (done) atomicAdd(&ctl->fast_items, done);
+      if (left) atomicAdd(&ctl->fast_deferred, left);
+    }
+    if (coded && ((L.modes >> M_SPLIT) & 1u)) atomicAdd(&ctl->split_trials, coded);
+    if (coded && ((L.modes >> M_PALETTE) & 1u)) atomicAdd(&ctl->palette_trials, coded);
+  }
+}
+
 // After a gate: free pages back to the stack, then the controller bookkeeping.
 // grid_ctas: the CTAs of the gate's general-kernel launch (no other CTA's cache holds
 // pages).  Called by one block of 1024 threads.
@@ -1146,6 +1193,12 @@ cudaError_t launch_gate(const GateLaunch& L, int grid, cudaStream_t st) {
     if (e != cudaSuccess) return e;
     k_gate<V><<<grid, kThreads, smem, st>>>(L);
   });
+  return cudaGetLastError();
+}
+
+cudaError_t launch_swap(const GateLaunch& L, cudaStream_t st) {
+  const unsigned long long want = (L.items + 7ull) / 8ull, most = (unsigned long long)num_sms() * 8ull;
+  k_swap<<<(unsigned)(want < most ? want : most), 256, 0, st>>>(L);
   return cudaGetLastError();
 }
 

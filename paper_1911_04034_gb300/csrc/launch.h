@@ -83,6 +83,9 @@ int fast_warps();        // warps per CTA of the streaming kernel (a pair of war
 int fast_items(int kind); // work items a CTA of the streaming kernel runs at once
 int fast_warp_cache();   // page ids each of its warps may hold
 cudaError_t launch_gate_fast(const GateLaunch& L, int grid, cudaStream_t st);
+// X between chunks: swaps the images of the work items that stand as they are, the others
+// appended to L.defer for launch_gate with L.list = 1 right after it.
+cudaError_t launch_swap(const GateLaunch& L, cudaStream_t st);
 cudaError_t launch_post(const Pool& P, const CtlParams& cp, int grid_ctas, cudaStream_t st);
 // The learned selector's decisions for every active chunk of the gate L describes,
 // written to dec (one byte per chunk, index 2 item + side) before the gate runs; mlp
