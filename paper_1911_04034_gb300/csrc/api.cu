@@ -325,20 +325,29 @@ sim_status sim_create_ex(int n_qubits, int block_log2, int chunk_log2, double er
     return fail(SIM_ERR_INVALID, "budget too large for 32-bit page ids");
   }
   if (s->fast_grid) {
-    // no more CTAs of the streaming kernel than the largest gate has items for, and,
-    // in a pool sized by the caller, no more than let its warps' free-page caches (each
-    // up to its capacity plus one refill, and one chunk's output pages) hold a quarter
-    // of the pool; none if not even one CTA fits
-    const uint64_t need = ((s->nchunks + 1) / 2 + qc::fast_items(0) - 1) / qc::fast_items(0);
-    uint64_t cap = need;
+    // No more CTAs of the streaming kernel than the largest gate has items for, and, in a
+    // pool sized by the caller, no more than let its warps' free-page caches (each up to
+    // its limit plus one refill, and one chunk's output pages) hold a quarter of the pool,
+    // or what the pool has beyond every chunk stored RAW; none if not even one CTA fits.
+    // The warps keep 64, 32 or 16 ids: the most that leaves every CTA its place.  (With
+    // 64 always, a 21-qubit state in a pool of 9/8 raw + 64 MB had 113 of 456 CTAs: 2048
+    // items took five rounds: 170 us a gate, now 57.)
+    const uint64_t items = (s->nchunks + 1) / 2, need = (items + qc::fast_items(0) - 1) / qc::fast_items(0);
+    uint64_t cap = (uint64_t)s->fast_grid < need ? (uint64_t)s->fast_grid : need;
     if (pool_bytes) {
-      const uint64_t per_cta = (uint64_t)qc::fast_warps() * (qc::fast_warp_cache() + 32 + qc::max_pages(s->kc));
-      const uint64_t fit = s->npages / 4 / per_cta;
+      const uint64_t most = s->nchunks * qc::max_pages(s->kc);
+      const uint64_t spare = s->npages > most ? s->npages - most : 0, quarter = s->npages / 4;
+      uint64_t fit = 0;
+      for (uint32_t keep = (uint32_t)qc::fast_warp_cache(); keep >= 16u && fit < cap; keep /= 2) {
+        s->P.wkeep = keep;
+        fit = (spare > quarter ? spare : quarter) / ((uint64_t)qc::fast_warps() * (keep + keep / 2 + qc::max_pages(s->kc)));
+      }
       cap = fit < cap ? fit : cap;
     }
     s->fast_grid = (uint64_t)s->fast_grid < cap ? s->fast_grid : (int)cap;
   }
   Pool& P = s->P;
+  if (!P.wkeep) P.wkeep = (uint32_t)qc::fast_warp_cache();
   P.kc = s->kc;
   P.npages = s->npages;
   P.dir_words = qc::dir_stride(s->kc) / 4;

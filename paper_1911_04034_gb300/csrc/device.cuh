@@ -163,6 +163,7 @@ struct Pool {
   unsigned long long npages;
   uint32_t dir_words;      // dir_stride / 4
   int kc;
+  uint32_t wkeep;          // streaming kernel: page ids a warp may keep (see sim_create_ex)
 };
 
 // ------------------------------------------------------- block cache ---- //

@@ -76,26 +76,27 @@ struct WarpPages {
   uint32_t* n;
 };
 
-// All lanes: at least `want` (<= 32) ids in the cache, refilled 32 at a time from the
-// global stack.  False (E_OOM set, the stack top restored) if the stack is dry.
+// All lanes: at least `want` (<= 32) ids in the cache, refilled from the global stack
+// half a cache (P.wkeep / 2) at a time.  False (E_OOM set, the stack top restored) if the stack is dry.
 __device__ __forceinline__ bool wp_reserve(const Pool& P, const WarpPages& wp, uint32_t want) {
   const uint32_t lane = threadIdx.x & 31u;
   const uint32_t n = *wp.n;
   if (n >= want) return true;
+  const uint32_t take = max(want - n, P.wkeep / 2u);  // at most 32
   long long old = 0;
   if (lane == 0)
-    old = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&P.ctl->top), (unsigned long long)(-32ll));
+    old = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&P.ctl->top), (unsigned long long)(-(long long)take));
   old = __shfl_sync(0xffffffffu, old, 0);
-  if (old - 32 < 0) {  // the stack is dry: give the reservation back (top never stays below 0)
+  if (old - (long long)take < 0) {  // the stack is dry: give the reservation back (top never stays below 0)
     if (lane == 0) {
-      atomicAdd(reinterpret_cast<unsigned long long*>(&P.ctl->top), 32ull);
+      atomicAdd(reinterpret_cast<unsigned long long*>(&P.ctl->top), (unsigned long long)take);
       atomicOr(&P.ctl->err, (unsigned)E_OOM);
     }
     return false;
   }
-  wp.ids[n + lane] = P.stack[old - 1 - (long long)lane];
+  if (lane < take) wp.ids[n + lane] = P.stack[old - 1 - (long long)lane];
   __syncwarp();
-  if (lane == 0) *wp.n = n + 32u;
+  if (lane == 0) *wp.n = n + take;
   __syncwarp();
   return true;
 }
@@ -104,7 +105,7 @@ __device__ __forceinline__ bool wp_reserve(const Pool& P, const WarpPages& wp, u
 // freed list (merged into the stack after the gate).
 __device__ __forceinline__ void wp_free(const Pool& P, const WarpPages& wp, const uint32_t* ids, uint32_t cnt) {
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t n = *wp.n, room = kWarpCache - n;
+  const uint32_t n = *wp.n, room = P.wkeep > n ? P.wkeep - n : 0u;
   unsigned long long base = 0;
   if (cnt > room) {
     if (lane == 0) base = atomicAdd(&P.ctl->nfreed, (unsigned long long)(cnt - room));
