@@ -94,8 +94,9 @@ typedef struct sim_stats_t {
   uint64_t split_trials;      /* chunk encodes that ran the Solution D trial */
   uint64_t cache_lookups;     /* block-cache lookups (work items that consulted it) */
   uint64_t cache_hits;        /* ... that took a cached result */
-  uint64_t fast_items;        /* work items the streaming gate kernel wrote (cumulative) */
-  uint64_t fast_deferred;     /* work items it left to the general gate kernel (cumulative) */
+  uint64_t fast_items;        /* work items at S <= 32 the fast path wrote (cumulative): by the streaming gate
+                               * kernel, by an image exchange, or in a whole-circuit launch as STREAM images */
+  uint64_t fast_deferred;     /* work items it left to the general path (cumulative) */
   uint64_t kernel_launches;   /* kernels the gates enqueued (selector, streaming, general and post kernels) */
   uint64_t palette_trials;    /* chunk encodes that ran the PALETTE trial */
   uint64_t graph_replays;     /* sim_batch_apply calls led by this handle that replayed its kept graph */
@@ -227,7 +228,8 @@ sim_status sim_set_budget(sim_t* sim, uint64_t bytes);
  * 1; the network needs sim_set_selector), "block_cache" (0/1, as sim_set_block_cache),
  * "timing" (0/1/2, as sim_set_timing), "tau_ppm" (tau in millionths, (0, 1e6]),
  * "fast_path" (1 default: gates run the streaming kernel first where it applies, see
- * sim_apply_gate; 0: every item through the general kernel -- same bytes, slower),
+ * sim_apply_gate, and circuits on small states run in one launch; 0: every gate through
+ * the general kernel -- same bytes, slower),
  * "ladder" (0/1/2; only before the first gate).  "chunk_log2" and "block_log2" are fixed
  * at creation.  Unknown keys or values out of range: SIM_ERR_INVALID. */
 sim_status sim_set_option(sim_t* sim, const char* key, int64_t value);

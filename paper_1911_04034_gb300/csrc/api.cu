@@ -156,13 +156,20 @@ struct sim {
   float* d_trace = nullptr;          // selector training records
   uint8_t* d_bc = nullptr;           // block cache lines (Section 3.4) or nullptr
   uint32_t* d_defer = nullptr;       // items the streaming kernel leaves to the general one
+  // whole circuits in one launch (k_run): staging for up to kRunBlock gate records
+  GateLaunch* h_run = nullptr;       // pinned
+  GateLaunch* d_run = nullptr;
+  qc::RunJob* h_run_jobs = nullptr;  // pinned, kRunSegments
+  qc::RunJob* d_run_jobs = nullptr;
+  size_t run_cap = 0;
+  int run_grid = 0;                  // its CTAs (0: not used for this state)
   int fast_grid = 0;                 // CTAs of the streaming kernel (0: chunk size outside its range)
   bool fast = true;                  // gates try the streaming kernel first
   uint64_t kernel_launches = 0;      // gate, streaming and post kernels enqueued
   uint64_t trace_cap = 0;
   // the graph of the last sim_batch_apply call this handle led, kept for replay
   cudaGraphExec_t bexec = nullptr;
-  qc::BatchJob* bjobs = nullptr;     // its job list (device)
+  void* bjobs = nullptr;             // its job list (device)
   std::vector<uint8_t> bkey;         // what its launches depend on
   std::vector<uint64_t> bupd;        // the amplitude updates it makes, per handle
   uint64_t uid = 0;                  // creation number (never reused)
@@ -178,6 +185,15 @@ struct sim {
     bkey.clear();
     bupd.clear();
   }
+  void drop_run() {
+    cudaFreeHost(h_run);
+    cudaFreeHost(h_run_jobs);
+    cudaFree(d_run);
+    cudaFree(d_run_jobs);
+    h_run = d_run = nullptr;
+    h_run_jobs = d_run_jobs = nullptr;
+    run_cap = 0;
+  }
   std::vector<cudaEvent_t> ev_pool;
   std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pending;
   size_t ev_next = 0;
@@ -192,6 +208,7 @@ struct sim {
     for (cudaEvent_t e : ev_pool) cudaEventDestroy(e);
     cudaFree(d_tlog);
     cudaFree(d_defer);
+    drop_run();
     cudaFree(d_mlp);
     cudaFree(d_dec);
     cudaFree(d_trace);
@@ -238,7 +255,7 @@ struct sim {
       unsigned int site = 0;
       cudaMemcpy(&site, &d_ctl->timeout_site, sizeof(site), cudaMemcpyDeviceToHost);
       poisoned = SIM_ERR_TIMEOUT;
-      return fail(SIM_ERR_TIMEOUT, "a bounded wait in the streaming gate kernel gave up (site %u)", site);
+      return fail(SIM_ERR_TIMEOUT, "a bounded wait in a gate kernel gave up (site %u)", site);
     }
     poisoned = SIM_ERR_CORRUPT;
     return fail(SIM_ERR_CORRUPT, "a chunk image failed its checks or held a non-finite value (flags 0x%x)", err);
@@ -345,6 +362,14 @@ sim_status sim_create_ex(int n_qubits, int block_log2, int chunk_log2, double er
       cap = fit < cap ? fit : cap;
     }
     s->fast_grid = (uint64_t)s->fast_grid < cap ? s->fast_grid : (int)cap;
+  }
+  // Whole circuits in one launch (see run_applies) where the resident CTAs take the largest
+  // gate in one round; from two rounds on the streaming kernel's throughput counts for more
+  // than its launches (2^10-amplitude chunks, 256 items 28 us a gate against 49; 512 items
+  // 55 against 49).
+  {
+    const uint64_t fit = (uint64_t)device_sms() * qc::run_ctas_per_sm(s->kc), items = (s->nchunks + 1) / 2;
+    if (items <= fit) s->run_grid = (int)items;
   }
   Pool& P = s->P;
   if (!P.wkeep) P.wkeep = (uint32_t)qc::fast_warp_cache();
@@ -458,6 +483,15 @@ sim_status sim_set_stream(sim_t* s, void* stream) {
   return SIM_OK;
 }
 
+// True if the gate is X between chunks with no control inside a chunk: whole images change
+// places (see k_swap).  Not where every item must be looked up (block cache), recorded
+// (traces) or decided anew (selector network).
+static bool swap_applies(const sim* s, const sim_gate* g, const GateLaunch& L) {
+  const double* u = g->u;
+  return s->fast && L.pair && L.lo_mask == 0u && !L.sel_dec && !L.bc && !L.trace && u[0] == 0.0 && u[1] == 0.0 &&
+         u[2] == 1.0 && u[3] == 0.0 && u[4] == 1.0 && u[5] == 0.0 && u[6] == 0.0 && u[7] == 0.0;
+}
+
 // Work description of one gate (Section 3.3 segments, see the top of this file).
 static GateLaunch make_launch(sim* s, const sim_gate* g) {
   const int kc = s->kc, t = g->target;
@@ -527,6 +561,7 @@ static GateLaunch make_launch(sim* s, const sim_gate* g) {
     q += len;
     p += len;
   }
+  L.swap = swap_applies(s, g, L) ? 1 : 0;
   return L;
 }
 
@@ -579,19 +614,114 @@ static bool fast_applies(const sim* s, const sim_gate* g, GateLaunch& L) {
   return true;
 }
 
-// True if the gate is X between chunks with no control inside a chunk: whole images change
-// places (see k_swap).  Not where every item must be looked up (block cache), recorded
-// (traces) or decided anew (selector network).
-static bool swap_applies(const sim* s, const sim_gate* g, const GateLaunch& L) {
-  const double* u = g->u;
-  return s->fast && L.pair && L.lo_mask == 0u && !L.sel_dec && !L.bc && !L.trace && u[0] == 0.0 && u[1] == 0.0 &&
-         u[2] == 1.0 && u[3] == 0.0 && u[4] == 1.0 && u[5] == 0.0 && u[6] == 0.0 && u[7] == 0.0;
+// True if circuits run by k_run: small states with no option that needs a kernel of its own
+// around each gate (timing, the selector network) or its counters (block cache, traces).
+static bool run_options(const sim* s) {
+  return s->fast && !s->timing && !s->phases && s->selector != 2 && !s->d_trace && !s->d_bc;
+}
+static bool run_applies(const sim* s) { return s->run_grid > 0 && run_options(s); }
+
+// Page ids each of a run's CTAs may keep between gates: all together no more than the pool
+// has beyond every chunk stored RAW, so that kept pages never make it run dry.
+static uint32_t run_keep(const sim* s, int ctas) {
+  const uint64_t most = s->nchunks * qc::max_pages(s->kc), spare = s->npages > most ? s->npages - most : 0;
+  const uint64_t q = spare / (uint64_t)ctas;
+  return (uint32_t)(q < (uint64_t)qc::kCacheCap ? q : (uint64_t)qc::kCacheCap);
+}
+
+// CTAs for each circuit of a batch: as few as let all of them end together.  A gate takes a
+// circuit's CTAs ceil(items / CTAs) rounds and one meeting (about 0.4 of a round).
+static std::vector<int> run_shares(const std::vector<const GateLaunch*>& first, const size_t* n_gates, int count,
+                                   int resident) {
+  std::vector<std::vector<double>> gates(count, std::vector<double>(64, 0.0));  // gates with 2^h items (items are powers of two)
+  std::vector<int> most(count, 1);
+  for (int k = 0; k < count; ++k)
+    for (size_t t = 0; t < n_gates[k]; ++t) {
+      const uint64_t items = first[k][t].items;
+      const int h = std::ilogb((double)items);
+      gates[k][h] += 1.0;
+      const int cap = items < (uint64_t)resident ? (int)items : resident;
+      most[k] = cap > most[k] ? cap : most[k];
+    }
+  auto span = [&](int k, int c) {
+    double t = 0.0;
+    for (int h = 0; h < 64; ++h)
+      if (gates[k][h] > 0.0) t += gates[k][h] * (std::ceil(std::ldexp(1.0, h) / c) + 0.4);
+    return t;
+  };
+  auto need = [&](int k, double t) {  // fewest CTAs that end by t (span falls as c grows)
+    int lo = 1, hi = most[k];
+    while (lo < hi) {
+      const int mid = (lo + hi) / 2;
+      if (span(k, mid) <= t) hi = mid;
+      else lo = mid + 1;
+    }
+    return lo;
+  };
+  double lo = 0.0, hi = 0.0;
+  for (int k = 0; k < count; ++k) hi = std::fmax(hi, span(k, 1));
+  std::vector<int> c(count, 1);
+  for (int it = 0; it < 40; ++it) {  // one CTA each always fits
+    const double mid = 0.5 * (lo + hi);
+    std::vector<int> w(count);
+    long sum = 0;
+    for (int k = 0; k < count; ++k) sum += w[k] = need(k, mid);
+    if (sum <= resident) {
+      c = w;
+      hi = mid;
+    } else {
+      lo = mid;
+    }
+  }
+  return c;
+}
+
+// Enqueues the gates as launches of k_run, the first ones short so that the device starts
+// while the host still prepares the rest.  False: no memory for the staging buffers.
+constexpr size_t kRunBlock = 4096;     // gate records staged at once
+constexpr size_t kRunSegments = 64;    // launches they make at most
+static sim_status run_circuit(sim* s, const sim_gate* gates, size_t n, bool* ran) {
+  *ran = false;
+  const size_t want = n < kRunBlock ? n : kRunBlock;
+  if (s->run_cap < want) {
+    s->drop_run();
+    if (cudaMallocHost(&s->h_run, want * sizeof(GateLaunch)) != cudaSuccess ||
+        cudaMallocHost(&s->h_run_jobs, kRunSegments * sizeof(qc::RunJob)) != cudaSuccess ||
+        cudaMalloc(&s->d_run, want * sizeof(GateLaunch)) != cudaSuccess ||
+        cudaMalloc(&s->d_run_jobs, kRunSegments * sizeof(qc::RunJob)) != cudaSuccess) {
+      cudaGetLastError();
+      s->drop_run();
+      return SIM_OK;
+    }
+    s->run_cap = want;
+  }
+  *ran = true;
+  for (size_t done = 0; done < n;) {
+    const size_t block = n - done < s->run_cap ? n - done : s->run_cap;
+    size_t off = 0, len = 16;
+    for (size_t seg = 0; off < block; ++seg, len = len < 256 ? 4 * len : len) {
+      const size_t m = block - off < len ? block - off : len;
+      for (size_t k = 0; k < m; ++k) {
+        s->h_run[off + k] = make_launch(s, gates + done + off + k);
+        s->amp_updates += s->h_run[off + k].nact << s->kc;
+      }
+      s->h_run_jobs[seg] = {s->d_run + off, (int)m, 0, s->run_grid, run_keep(s, s->run_grid)};
+      CK(cudaMemcpyAsync(s->d_run + off, s->h_run + off, m * sizeof(GateLaunch), cudaMemcpyHostToDevice, s->st), "gate records");
+      CK(cudaMemcpyAsync(s->d_run_jobs + seg, s->h_run_jobs + seg, sizeof(qc::RunJob), cudaMemcpyHostToDevice, s->st), "gate records");
+      CK(qc::launch_run(s->d_run_jobs + seg, 1, s->kc, s->run_grid, s->st), "circuit kernel launch");
+      s->kernel_launches += 1;
+      off += m;
+    }
+    done += block;
+    if (done < n) CK(cudaStreamSynchronize(s->st), "sync");  // the staging buffers are free again
+  }
+  return SIM_OK;
 }
 
 static sim_status enqueue_gate(sim* s, const sim_gate* g) {
   GateLaunch L = make_launch(s, g);
   const int grid = (uint64_t)s->grid < L.items ? s->grid : (int)L.items;
-  const bool swap = swap_applies(s, g, L), fast = !swap && fast_applies(s, g, L);
+  const bool swap = L.swap != 0, fast = !swap && fast_applies(s, g, L);
   L.defer = s->d_defer;
   cudaEvent_t e0 = nullptr, e1 = nullptr;
   if (s->timing) {
@@ -667,7 +797,10 @@ sim_status sim_apply_circuit(sim_t* s, const sim_gate* gates, size_t n_gates) {
   std::string why;
   for (size_t k = 0; k < n_gates; ++k)
     if (!gate_ok(gates + k, s->n, &why)) return fail(SIM_ERR_INVALID, "invalid gate %zu: %s", k, why.c_str());
-  for (size_t k = 0; k < n_gates; ++k)
+  bool ran = false;
+  if (run_applies(s) && n_gates)
+    if (sim_status r = run_circuit(s, gates, n_gates, &ran)) return r;
+  for (size_t k = 0; k < n_gates && !ran; ++k)
     if (sim_status r = enqueue_gate(s, gates + k)) return r;
   return s->check_device();
 }
@@ -1110,33 +1243,68 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
     if (e == cudaSuccess) ++lead->graph_replays;
   } else {
     if (use_graph) lead->drop_graph();
-    // step t holds gate t of every circuit that has one; its jobs' items are numbered
-    // consecutively
+    // Where every handle's circuit can run by k_run: one launch, each circuit on CTAs of its
+    // own and at its own pace.  Otherwise (an option that needs kernels around each gate)
+    // step by step: step t holds gate t of every circuit that has one, its jobs' items
+    // numbered consecutively.
+    const int resident = device_sms() * qc::run_ctas_per_sm(kc);
+    bool whole = count <= resident / 2;
+    for (int k = 0; k < count; ++k) whole = whole && run_options(sims[k]);
     std::vector<qc::BatchJob> jobs;
     std::vector<sim*> job_sim;  // the handle of each job
     std::vector<size_t> off(steps + 1, 0);
     std::vector<unsigned long long> total(steps, 0);
+    std::vector<uint8_t> run_list;  // whole: the RunJobs, then every circuit's gate records
+    int njobs = 0, run_grid = 0;
     int grid = sims[0]->grid;
-    for (int k = 1; k < count; ++k) grid = sims[k]->grid < grid ? sims[k]->grid : grid;
-    for (size_t t = 0; t < steps; ++t) {
-      off[t] = jobs.size();
-      unsigned long long begin = 0;
+    void* d_jobs = nullptr;
+    if (whole) {
+      size_t all = 0;
+      for (int k = 0; k < count; ++k) all += n_gates[k];
+      const size_t head = (count * sizeof(qc::RunJob) + 15) & ~(size_t)15;
+      run_list.resize(head + all * sizeof(GateLaunch));
+      GateLaunch* rec = reinterpret_cast<GateLaunch*>(run_list.data() + head);
+      std::vector<const GateLaunch*> first(count);
       for (int k = 0; k < count; ++k) {
-        if (t >= n_gates[k]) continue;
-        qc::BatchJob j;
-        j.L = make_launch(sims[k], circuits[k] + t);
-        j.begin = begin;
-        begin += j.L.items;
-        upd[k] += j.L.nact << sims[k]->kc;
-        jobs.push_back(j);
-        job_sim.push_back(sims[k]);
+        first[k] = rec;
+        for (size_t t = 0; t < n_gates[k]; ++t, ++rec) {
+          const GateLaunch L = make_launch(sims[k], circuits[k] + t);
+          upd[k] += L.nact << sims[k]->kc;
+          std::memcpy(rec, &L, sizeof L);
+        }
       }
-      total[t] = begin;
+      const std::vector<int> ctas = run_shares(first, n_gates, count, resident);
+      CK(cudaMalloc(&d_jobs, run_list.size()), "batch job list");
+      for (int k = 0; k < count; ++k) {
+        if (!n_gates[k]) continue;
+        const size_t at = (size_t)(reinterpret_cast<const uint8_t*>(first[k]) - run_list.data());
+        const qc::RunJob j{reinterpret_cast<const GateLaunch*>((const uint8_t*)d_jobs + at), (int)n_gates[k], run_grid,
+                           ctas[k], run_keep(sims[k], ctas[k])};
+        std::memcpy(run_list.data() + (size_t)njobs++ * sizeof j, &j, sizeof j);
+        run_grid += ctas[k];
+      }
+      e = cudaMemcpyAsync(d_jobs, run_list.data(), run_list.size(), cudaMemcpyHostToDevice, st);
+    } else {
+      for (int k = 1; k < count; ++k) grid = sims[k]->grid < grid ? sims[k]->grid : grid;
+      for (size_t t = 0; t < steps; ++t) {
+        off[t] = jobs.size();
+        unsigned long long begin = 0;
+        for (int k = 0; k < count; ++k) {
+          if (t >= n_gates[k]) continue;
+          qc::BatchJob j;
+          j.L = make_launch(sims[k], circuits[k] + t);
+          j.begin = begin;
+          begin += j.L.items;
+          upd[k] += j.L.nact << sims[k]->kc;
+          jobs.push_back(j);
+          job_sim.push_back(sims[k]);
+        }
+        total[t] = begin;
+      }
+      off[steps] = jobs.size();
+      CK(cudaMalloc(&d_jobs, jobs.size() * sizeof(qc::BatchJob)), "batch job list");
+      e = cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(qc::BatchJob), cudaMemcpyHostToDevice, st);
     }
-    off[steps] = jobs.size();
-    qc::BatchJob* d_jobs = nullptr;
-    CK(cudaMalloc(&d_jobs, jobs.size() * sizeof(qc::BatchJob)), "batch job list");
-    e = cudaMemcpyAsync(d_jobs, jobs.data(), jobs.size() * sizeof(qc::BatchJob), cudaMemcpyHostToDevice, st);
     // A graph is captured on a private stream (the legacy default stream cannot be
     // captured), ordered after the work already queued on the handles' stream.
     cudaStream_t cs = st;
@@ -1150,9 +1318,12 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
       if (e == cudaSuccess) e = cudaStreamWaitEvent(cs, lead->bready, 0);
       if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed);
     }
-    for (size_t t = 0; t < steps && e == cudaSuccess; ++t) {
+    if (whole && e == cudaSuccess)
+      e = qc::launch_run(reinterpret_cast<const qc::RunJob*>(d_jobs), njobs, kc, run_grid, cs);
+    for (size_t t = 0; t < steps && !whole && e == cudaSuccess; ++t) {
       const int n = (int)(off[t + 1] - off[t]);
       const int g = (unsigned long long)grid < total[t] ? grid : (int)total[t];
+      const qc::BatchJob* step = reinterpret_cast<const qc::BatchJob*>(d_jobs) + off[t];
       // the selector's decisions of every handle that runs the network, before the step
       for (size_t j = off[t]; j < off[t + 1] && e == cudaSuccess; ++j) {
         const GateLaunch& L = jobs[j].L;
@@ -1161,8 +1332,8 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
         const int sg = (unsigned long long)grid < (na + 255ull) / 256ull ? grid : (int)((na + 255ull) / 256ull);
         e = qc::launch_select(L, job_sim[j]->d_mlp, const_cast<uint8_t*>(L.sel_dec), sg, cs);
       }
-      if (e == cudaSuccess) e = qc::launch_gate_batch(d_jobs + off[t], n, total[t], kc, g, cs);
-      if (e == cudaSuccess) e = qc::launch_post_batch(d_jobs + off[t], n, g, cs);
+      if (e == cudaSuccess) e = qc::launch_gate_batch(step, n, total[t], kc, g, cs);
+      if (e == cudaSuccess) e = qc::launch_post_batch(step, n, g, cs);
     }
     if (use_graph && cs != st) {
       cudaError_t e2 = cudaStreamEndCapture(cs, &graph);

@@ -91,12 +91,14 @@ struct DevCtl {
   unsigned int fast_pad;
   unsigned long long fast_items;       // work items the streaming kernel committed (cumulative)
   unsigned long long fast_deferred;    // work items it left to the general kernel (cumulative)
-  unsigned int timeout_site;           // where a bounded wait gave up (E_TIMEOUT): 1 item start, 2 pass, 3 item end
+  unsigned int timeout_site;           // where a bounded wait gave up (E_TIMEOUT): 1 item start, 2 pass, 3 item end, 4 between gates (k_run)
   unsigned int timeout_pad;
   unsigned long long wc_pages;         // free pages the streaming kernel's warps keep in their caches
   unsigned long long palette_trials;   // chunk encodes that ran the PALETTE trial
   long long n64;                       // images whose header says S = 64 (as of the last gate)
   long long dn64;                      // ... its change during the running gate
+  unsigned int run_arrived;            // k_run: CTAs that finished a gate (cumulative over the launch)
+  unsigned int run_gate;               // k_run: gates finished and booked in the launch
 };
 
 // Controller parameters (host-computed, constant for the handle).

@@ -10,7 +10,7 @@ namespace qc {
 constexpr int kMaxRuns = 6;
 
 // One gate on the compressed state.
-struct GateLaunch {
+struct alignas(16) GateLaunch {
   Pool P;
   CtlParams ctl;
   GateCoef g;
@@ -25,6 +25,7 @@ struct GateLaunch {
   uint32_t lo_mask, lo_vals;     // controls inside a chunk
   int target;                    // target bit (in-chunk gates)
   int pair;                      // 1: target >= chunk_log2
+  int swap;                      // 1: X between chunks that may exchange whole images (see swap_item)
   int prof;                      // 1: accumulate per-phase SM cycles
   uint32_t modes;                // chunk modes the encoder may choose (bit m = mode m)
   const uint8_t* sel_dec;        // the selector's decisions, one byte per active chunk (index 2 item + side;
@@ -60,6 +61,14 @@ struct BatchJob {
   unsigned long long begin;
 };
 
+// A run of gates of one simulator inside a launch of k_run.
+struct RunJob {
+  const GateLaunch* gates;  // device
+  int ngates;
+  int first, ctas;          // its CTAs: [first, first + ctas)
+  uint32_t keep;            // page ids a CTA may keep between gates
+};
+
 // Records the message sim_last_error() returns on the calling thread.
 void set_last_error(const char* msg);
 
@@ -83,6 +92,11 @@ int fast_warps();        // warps per CTA of the streaming kernel (a pair of war
 int fast_items(int kind); // work items a CTA of the streaming kernel runs at once
 int fast_warp_cache();   // page ids each of its warps may hold
 cudaError_t launch_gate_fast(const GateLaunch& L, int grid, cudaStream_t st);
+// Whole circuits in one launch: every simulator's gates in order by the general kernel's
+// items, its CTAs meeting after each gate.  All CTAs must be resident at once: at most
+// run_ctas_per_sm * num_sms().
+int run_ctas_per_sm(int kc);
+cudaError_t launch_run(const RunJob* jobs, int njobs, int kc, int grid, cudaStream_t st);
 // X between chunks: swaps the images of the work items that stand as they are, the others
 // appended to L.defer for launch_gate with L.list = 1 right after it.
 cudaError_t launch_swap(const GateLaunch& L, cudaStream_t st);

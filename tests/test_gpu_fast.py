@@ -138,3 +138,38 @@ def test_power_of_two_gates_near_the_bottom_of_the_normal_range():
         assert all_images(gpu) == [orc.image(q) for q in range(orc.nchunks)], k
     st = gpu.stats()
     assert st["fast_items"] > 0 and st["fast_deferred"] > 0
+
+
+@pytest.mark.parametrize("modes", [0x1F, 0x7F])
+@pytest.mark.parametrize("kc", [3, 7, 9, 11])
+def test_gate_by_gate_and_whole_circuit_agree(kc, modes):
+    """The same circuit gate by gate (a launch of the streaming or the image-exchange kernel
+    per gate), as whole circuits in one launch, and through the general kernel alone: the
+    oracle's images and the same counters, trials of a mode set with SPLIT and PALETTE
+    included, in a pool with room and (one launch) in one that just holds every chunk RAW."""
+    n = 13
+    raw = 16 << n
+    circuits = [Cc.rcs_n(n, 6, seed=kc), Cc.qaoa_maxcut(n + 1, 1, 3, seed=4)[0], Cc.qft(n, seed=5)[0], Cc.grover(n, 2, seed=6)[0]]
+    keys = ("gates", "encoded_bytes", "max_encoded_bytes", "eps_switch_gate", "chunks_by_mode", "fidelity_lb_sum", "wide_images",
+            "split_trials", "palette_trials", "pages_in_use_bytes", "peak_pages_bytes", "amp_updates")
+    for ci, gates in enumerate(circuits):
+        m = n + (ci == 1)
+        got = []
+        for how in ("gates", "circuit", "general", "tight"):
+            s = qc().Sim(m, m, 1e-4, chunk_log2=kc, budget=raw // 3,
+                         pool_bytes=(512 * ((16 << kc) // 512 + 1) << (m - kc)) if how == "tight" else 2 * (16 << m) + (64 << 20))
+            s.set_modes(modes)
+            if how == "general":
+                s.set_option("fast_path", 0)
+            if how == "gates":
+                for g in gates:
+                    s.apply_gate(g)
+            else:
+                s.apply_circuit(gates[:50])
+                s.apply_circuit(gates[50:])
+            got.append((all_images(s), {k: s.stats()[k] for k in keys}))
+        for g in got[1:]:
+            assert g == got[0], ci
+        orc = O.CSim(m, m, kc, 1e-4, raw // 3, modes=modes)
+        orc.apply(gates)
+        assert got[0][0] == [orc.image(c) for c in range(orc.nchunks)], ci
