@@ -395,6 +395,10 @@ sim_status sim_codec_encode(const double* in, uint64_t n_chunks, int chunk_log2,
  * (see sim_set_modes). */
 sim_status sim_codec_encode_ex(const double* in, uint64_t n_chunks, int chunk_log2, double eps, int force_mode,
                                uint32_t modes, uint8_t* out, uint64_t out_stride, uint32_t* out_len, int on_device);
+/* sim_codec_encode_ex that also clears the rest of every image's out_stride slot: the
+ * caller need not. */
+sim_status sim_codec_encode_padded(const double* in, uint64_t n_chunks, int chunk_log2, double eps, int force_mode,
+                               uint32_t modes, uint8_t* out, uint64_t out_stride, uint32_t* out_len, int on_device);
 
 /* Decodes n_chunks images (image k at in + k * in_stride, length in_len[k]) into
  * out = n_chunks * 2^(chunk_log2+1) doubles.  SIM_ERR_CORRUPT if any image fails

@@ -1733,14 +1733,9 @@ sim_status sim_checkpoint_load(sim_t* s, const void* in, uint64_t in_len, int in
 }
 
 // ------------------------------------------------------------ codec ------ //
-sim_status sim_codec_encode(const double* in, uint64_t n_chunks, int chunk_log2, double eps, int force_mode,
-                            uint8_t* out, uint64_t out_stride, uint32_t* out_len, int on_device) {
-  return sim_codec_encode_ex(in, n_chunks, chunk_log2, eps, force_mode, qc::kDefaultModes, out, out_stride, out_len,
-                             on_device);
-}
-
-sim_status sim_codec_encode_ex(const double* in, uint64_t n_chunks, int chunk_log2, double eps, int force_mode,
-                               uint32_t modes, uint8_t* out, uint64_t out_stride, uint32_t* out_len, int on_device) {
+static sim_status codec_encode(const double* in, uint64_t n_chunks, int chunk_log2, double eps, int force_mode,
+                               uint32_t modes, uint8_t* out, uint64_t out_stride, uint32_t* out_len, int on_device,
+                               bool pad) {
   if ((modes & qc::kDefaultModes) != qc::kDefaultModes || (modes >> qc::M_NMODES))
     return fail(SIM_ERR_INVALID, "the mode set must contain ZERO..RAW (0x1F) and only known modes");
   if (!in || !out || !out_len) return fail(SIM_ERR_INVALID, "NULL argument");
@@ -1760,7 +1755,7 @@ sim_status sim_codec_encode_ex(const double* in, uint64_t n_chunks, int chunk_lo
   uint32_t* dlen = out_len;
   unsigned int* derr = nullptr;
   void* tmp = nullptr;
-  size_t tmp_bytes = sizeof(unsigned int) + (on_device ? 0 : in_bytes + n_chunks * out_stride + n_chunks * 4 + 64);
+  size_t tmp_bytes = 16 + (on_device ? 0 : in_bytes + n_chunks * out_stride + n_chunks * 4 + 64);
   CK(cudaMalloc(&tmp, tmp_bytes), "codec buffers");
   derr = reinterpret_cast<unsigned int*>(tmp);
   if (!on_device) {
@@ -1770,9 +1765,9 @@ sim_status sim_codec_encode_ex(const double* in, uint64_t n_chunks, int chunk_lo
     dlen = reinterpret_cast<uint32_t*>(dout + n_chunks * out_stride);
     cudaMemcpy((void*)din, in, in_bytes, cudaMemcpyHostToDevice);
   }
-  cudaMemset(derr, 0, sizeof(unsigned int));
+  cudaMemset(derr, 0, 2 * sizeof(unsigned int));  // the error word, and the chunks left to the general encoder
   cudaError_t e = qc::launch_codec_encode(din, n_chunks, chunk_log2, (uint32_t)S, force_mode, modes, dout, out_stride,
-                                          dlen, derr, 0);
+                                          dlen, derr, derr + 1, pad, 0);
   unsigned int herr = 0;
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e == cudaSuccess) e = cudaMemcpy(&herr, derr, sizeof(herr), cudaMemcpyDeviceToHost);
@@ -1785,6 +1780,23 @@ sim_status sim_codec_encode_ex(const double* in, uint64_t n_chunks, int chunk_lo
   if (herr & qc::E_NONFINITE) return fail(SIM_ERR_INVALID, "input holds a non-finite value");
   if (herr & qc::E_MODE) return fail(SIM_ERR_INVALID, "forced mode does not apply to a chunk");
   return SIM_OK;
+}
+
+sim_status sim_codec_encode(const double* in, uint64_t n_chunks, int chunk_log2, double eps, int force_mode,
+                            uint8_t* out, uint64_t out_stride, uint32_t* out_len, int on_device) {
+  return codec_encode(in, n_chunks, chunk_log2, eps, force_mode, qc::kDefaultModes, out, out_stride, out_len, on_device,
+                      false);
+}
+
+sim_status sim_codec_encode_ex(const double* in, uint64_t n_chunks, int chunk_log2, double eps, int force_mode,
+                               uint32_t modes, uint8_t* out, uint64_t out_stride, uint32_t* out_len, int on_device) {
+  return codec_encode(in, n_chunks, chunk_log2, eps, force_mode, modes, out, out_stride, out_len, on_device, false);
+}
+
+sim_status sim_codec_encode_padded(const double* in, uint64_t n_chunks, int chunk_log2, double eps, int force_mode,
+                                   uint32_t modes, uint8_t* out, uint64_t out_stride, uint32_t* out_len,
+                                   int on_device) {
+  return codec_encode(in, n_chunks, chunk_log2, eps, force_mode, modes, out, out_stride, out_len, on_device, true);
 }
 
 sim_status sim_codec_decode(const uint8_t* in, uint64_t in_stride, const uint32_t* in_len, uint64_t n_chunks,

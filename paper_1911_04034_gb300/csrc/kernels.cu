@@ -202,7 +202,9 @@ __global__ void __launch_bounds__(kThreads) k_init_chunk0(const Pool P, unsigned
 template <int VPT>
 __global__ void __launch_bounds__(kThreads)
     k_codec_encode(const double* in, unsigned long long nchunks, int kc, uint32_t S, int force, uint32_t modes,
-                   uint8_t* out, unsigned long long stride, uint32_t* lens, unsigned int* err) {
+                   uint8_t* out, unsigned long long stride, uint32_t* lens, unsigned int* err,
+                   const unsigned int* todo, int pad) {
+  if (todo && *todo == 0u) return;  // only the chunks of length 0 (k_stream_encode), of which there are none
   extern __shared__ __align__(16) uint8_t smem[];
   const uint32_t N = 2u << kc, cap = codedcap(kc);
   uint64_t* tile = reinterpret_cast<uint64_t*>(smem);
@@ -211,6 +213,7 @@ __global__ void __launch_bounds__(kThreads)
   ScanSmem& s = *reinterpret_cast<ScanSmem*>(pages + pagelist_words(kc));
   int pp = 0;
   for (unsigned long long c = blockIdx.x; c < nchunks; c += gridDim.x) {
+    if (todo && lens[c] != 0u) continue;
     const unsigned long long* src = reinterpret_cast<const unsigned long long*>(in) + c * N;
     for (uint32_t j = threadIdx.x; j < N; j += kThreads) tile[tile_val(j)] = src[j];
     __syncthreads();
@@ -218,137 +221,14 @@ __global__ void __launch_bounds__(kThreads)
     uint4* dst = reinterpret_cast<uint4*>(out + c * stride);
     const uint4* sv = reinterpret_cast<const uint4*>(img);
     for (uint32_t u = threadIdx.x; u < n / 16u; u += kThreads) dst[u] = sv[u];
+    if (pad)
+      for (unsigned long long u = n / 16u + threadIdx.x; u < stride / 16u; u += kThreads) dst[u] = make_uint4(0u, 0u, 0u, 0u);
     if (threadIdx.x == 0) lens[c] = n;
     __syncthreads();
   }
 }
 
-template <int VPT>
-__global__ void __launch_bounds__(kThreads)
-    k_codec_decode(const uint8_t* in, unsigned long long stride, const uint32_t* lens, unsigned long long nchunks,
-                   int kc, double* out, unsigned int* err) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  const uint32_t N = 2u << kc, cap = codedcap(kc);
-  uint64_t* tile = reinterpret_cast<uint64_t*>(smem);
-  uint8_t* img = reinterpret_cast<uint8_t*>(tile + tile_words(kc));
-  uint32_t* pages = reinterpret_cast<uint32_t*>(img + cap);
-  ScanSmem& s = *reinterpret_cast<ScanSmem*>(pages + pagelist_words(kc));
-  int pp = 0;
-  for (unsigned long long c = blockIdx.x; c < nchunks; c += gridDim.x) {
-    const uint32_t len = lens[c];
-    const bool fits = len <= cap && (len & 15u) == 0u && len >= 16u;
-    if (fits) {
-      const uint4* src = reinterpret_cast<const uint4*>(in + c * stride);
-      uint4* d = reinterpret_cast<uint4*>(img);
-      for (uint32_t u = threadIdx.x; u < len / 16u; u += kThreads) d[u] = src[u];
-    } else if (threadIdx.x == 0) {
-      reinterpret_cast<uint32_t*>(img)[0] = 0xffu;  // fails the header checks
-    }
-    __syncthreads();
-    const bool ok = decode_block<VPT>(img, fits ? len : 16u, kc, tile, s, pp);
-    if (!ok && threadIdx.x == 0) atomicOr(err, (unsigned)E_CORRUPT);
-    unsigned long long* dst = reinterpret_cast<unsigned long long*>(out) + c * N;
-    for (uint32_t j = threadIdx.x; j < N; j += kThreads) dst[j] = tile[tile_val(j)];
-    __syncthreads();
-  }
-}
-
 // --------------------------------------------------------------- readout -- //
-// Decodes the chunks overlapping [first_amp, first_amp + count) into out.
-template <int VPT>
-__global__ void __launch_bounds__(kThreads)
-    k_decode_range(const Pool P, unsigned long long first_amp, unsigned long long count, double* out) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  const int kc = P.kc;
-  const uint32_t A = 1u << kc, cap = imgcap(kc);
-  uint64_t* tile = reinterpret_cast<uint64_t*>(smem);
-  uint8_t* img = reinterpret_cast<uint8_t*>(tile + tile_words(kc));
-  uint32_t* pages = reinterpret_cast<uint32_t*>(img + cap);
-  ScanSmem& s = *reinterpret_cast<ScanSmem*>(pages + pagelist_words(kc));
-  int pp = 0;
-  const unsigned long long cfirst = first_amp >> kc, clast = (first_amp + count - 1ull) >> kc;
-  for (unsigned long long c = cfirst + blockIdx.x; c <= clast; c += gridDim.x) {
-    const uint32_t* e = dir_entry(P, c);
-    const uint32_t b = e[0];
-    if (b > cap || e[1] > max_pages(kc)) {
-      if (threadIdx.x == 0) atomicOr(&P.ctl->err, (unsigned)E_CORRUPT);
-      return;
-    }
-    load_image_block(P, c, img, pages, cap);
-    if (!decode_block<VPT>(img, b, kc, tile, s, pp) && threadIdx.x == 0) atomicOr(&P.ctl->err, (unsigned)E_CORRUPT);
-    const unsigned long long base = c << kc;
-    unsigned long long* dst = reinterpret_cast<unsigned long long*>(out);
-    for (uint32_t i = threadIdx.x; i < A; i += kThreads) {
-      const unsigned long long a = base + i;
-      if (a >= first_amp && a < first_amp + count) {
-        dst[2 * (a - first_amp)] = tile[tile_val(2 * i)];
-        dst[2 * (a - first_amp) + 1] = tile[tile_val(2 * i + 1)];
-      }
-    }
-    __syncthreads();
-  }
-}
-
-// Per chunk: sum over its amplitudes of fma(re, re, im*im) (measurement), or the
-// partial inner product with a reference state and the norm (fidelity).
-template <int VPT, bool DOT>
-__global__ void __launch_bounds__(kThreads)
-    k_chunk_reduce(const Pool P, unsigned long long cfirst, unsigned long long nchunks, const double* ref, double* out) {
-  extern __shared__ __align__(16) uint8_t smem[];
-  const int kc = P.kc;
-  const uint32_t A = 1u << kc, cap = imgcap(kc);
-  uint64_t* tile = reinterpret_cast<uint64_t*>(smem);
-  uint8_t* img = reinterpret_cast<uint8_t*>(tile + tile_words(kc));
-  uint32_t* pages = reinterpret_cast<uint32_t*>(img + cap);
-  ScanSmem& s = *reinterpret_cast<ScanSmem*>(pages + pagelist_words(kc));
-  int pp = 0;
-  __shared__ double red[3][kThreads];
-  for (unsigned long long cl = blockIdx.x; cl < nchunks; cl += gridDim.x) {
-    const unsigned long long c = cfirst + cl;
-    const uint32_t* e = dir_entry(P, c);
-    const uint32_t b = e[0];
-    if (b > cap || e[1] > max_pages(kc)) {
-      if (threadIdx.x == 0) atomicOr(&P.ctl->err, (unsigned)E_CORRUPT);
-      return;
-    }
-    load_image_block(P, c, img, pages, cap);
-    if (!decode_block<VPT>(img, b, kc, tile, s, pp) && threadIdx.x == 0) atomicOr(&P.ctl->err, (unsigned)E_CORRUPT);
-    const double* v = reinterpret_cast<const double*>(tile);
-    double x = 0.0, y = 0.0, z = 0.0;
-    for (uint32_t i = threadIdx.x; i < A; i += kThreads) {
-      const double pr = v[tile_val(2 * i)], pi = v[tile_val(2 * i + 1)];
-      z += __fma_rn(pr, pr, __dmul_rn(pi, pi));
-      if (DOT) {
-        const double rr = ref[(cl << kc) * 2 + 2 * i], ri = ref[(cl << kc) * 2 + 2 * i + 1];
-        x += rr * pr + ri * pi;
-        y += rr * pi - ri * pr;
-      }
-    }
-    red[0][threadIdx.x] = x;
-    red[1][threadIdx.x] = y;
-    red[2][threadIdx.x] = z;
-    __syncthreads();
-    for (int h = kThreads / 2; h > 0; h >>= 1) {
-      if ((int)threadIdx.x < h) {
-        red[0][threadIdx.x] += red[0][threadIdx.x + h];
-        red[1][threadIdx.x] += red[1][threadIdx.x + h];
-        red[2][threadIdx.x] += red[2][threadIdx.x + h];
-      }
-      __syncthreads();
-    }
-    if (threadIdx.x == 0) {
-      if (DOT) {
-        out[3 * cl] = red[0][0];
-        out[3 * cl + 1] = red[1][0];
-        out[3 * cl + 2] = red[2][0];
-      } else {
-        out[cl] = red[2][0];
-      }
-    }
-    __syncthreads();
-  }
-}
-
 // Chunks per mode (counts[8]) and, if wide is not null, the images whose header says
 // S = 64 (added to *wide).
 __global__ void k_mode_counts(const Pool P, unsigned long long nchunks, unsigned long long* counts,
@@ -529,68 +409,27 @@ cudaError_t launch_init_chunk0(const Pool& P, unsigned long long nchunks, cudaSt
 cudaError_t launch_codec_encode(const double* in, unsigned long long nchunks, int kc, uint32_t S, int force,
                                 uint8_t* out, unsigned long long stride, uint32_t* lens, unsigned int* err,
                                 cudaStream_t st) {
-  return launch_codec_encode(in, nchunks, kc, S, force, kDefaultModes, out, stride, lens, err, st);
+  return launch_codec_encode(in, nchunks, kc, S, force, kDefaultModes, out, stride, lens, err, nullptr, false, st);
 }
 
 cudaError_t launch_codec_encode(const double* in, unsigned long long nchunks, int kc, uint32_t S, int force,
                                 uint32_t modes, uint8_t* out, unsigned long long stride, uint32_t* lens,
-                                unsigned int* err, cudaStream_t st) {
+                                unsigned int* err, unsigned int* todo, bool pad, cudaStream_t st) {
   const size_t smem = codec_smem_bytes(kc);
-  const unsigned long long g = nchunks < (unsigned long long)num_sms() * 8 ? nchunks : (unsigned long long)num_sms() * 8;
+  const unsigned long long sms = (unsigned long long)num_sms(), g = nchunks < sms * 8 ? nchunks : sms * 8;
+  // Solution C's modes at S <= 32 on enough chunks: a warp per chunk first, then the general
+  // encoder on the chunks it left.  (Below two CTAs an SM a CTA per chunk is sooner done.)
+  const bool warp = todo && force < 0 && modes == kDefaultModes && S <= 32u && kc >= kFastMinKC &&
+                    nchunks >= 2ull * kWarps * sms && (reinterpret_cast<uintptr_t>(in) & 15u) == 0u;
+  if (warp) {
+    const cudaError_t e = launch_stream_encode(in, nchunks, kc, S, out, stride, lens, todo, pad, st);
+    if (e != cudaSuccess) return e;
+  }
   QC_VPT_DISPATCH(kc, {
     cudaError_t e = prep(k_codec_encode<V>, smem);
     if (e != cudaSuccess) return e;
-    k_codec_encode<V><<<(unsigned)g, kThreads, smem, st>>>(in, nchunks, kc, S, force, modes, out, stride, lens, err);
-  });
-  return cudaGetLastError();
-}
-
-cudaError_t launch_codec_decode(const uint8_t* in, unsigned long long stride, const uint32_t* lens,
-                                unsigned long long nchunks, int kc, double* out, unsigned int* err, cudaStream_t st) {
-  const size_t smem = codec_smem_bytes(kc);
-  const unsigned long long g = nchunks < (unsigned long long)num_sms() * 8 ? nchunks : (unsigned long long)num_sms() * 8;
-  QC_VPT_DISPATCH(kc, {
-    cudaError_t e = prep(k_codec_decode<V>, smem);
-    if (e != cudaSuccess) return e;
-    k_codec_decode<V><<<(unsigned)g, kThreads, smem, st>>>(in, stride, lens, nchunks, kc, out, err);
-  });
-  return cudaGetLastError();
-}
-
-cudaError_t launch_decode_range(const Pool& P, unsigned long long first_amp, unsigned long long count, double* out,
-                                cudaStream_t st) {
-  if (count == 0) return cudaSuccess;
-  const size_t smem = codec_smem_bytes(P.kc);
-  const unsigned long long nch = ((first_amp + count - 1ull) >> P.kc) - (first_amp >> P.kc) + 1ull;
-  const unsigned long long g = nch < (unsigned long long)num_sms() * 8 ? nch : (unsigned long long)num_sms() * 8;
-  QC_VPT_DISPATCH(P.kc, {
-    cudaError_t e = prep(k_decode_range<V>, smem);
-    if (e != cudaSuccess) return e;
-    k_decode_range<V><<<(unsigned)g, kThreads, smem, st>>>(P, first_amp, count, out);
-  });
-  return cudaGetLastError();
-}
-
-cudaError_t launch_chunk_norms(const Pool& P, unsigned long long cfirst, unsigned long long nchunks, double* out,
-                              cudaStream_t st) {
-  const size_t smem = codec_smem_bytes(P.kc);
-  const unsigned long long g = nchunks < (unsigned long long)num_sms() * 8 ? nchunks : (unsigned long long)num_sms() * 8;
-  QC_VPT_DISPATCH(P.kc, {
-    cudaError_t e = prep(k_chunk_reduce<V, false>, smem);
-    if (e != cudaSuccess) return e;
-    k_chunk_reduce<V, false><<<(unsigned)g, kThreads, smem, st>>>(P, cfirst, nchunks, nullptr, out);
-  });
-  return cudaGetLastError();
-}
-
-cudaError_t launch_chunk_dots(const Pool& P, unsigned long long cfirst, unsigned long long nchunks, const double* ref,
-                             double* out, cudaStream_t st) {
-  const size_t smem = codec_smem_bytes(P.kc);
-  const unsigned long long g = nchunks < (unsigned long long)num_sms() * 8 ? nchunks : (unsigned long long)num_sms() * 8;
-  QC_VPT_DISPATCH(P.kc, {
-    cudaError_t e = prep(k_chunk_reduce<V, true>, smem);
-    if (e != cudaSuccess) return e;
-    k_chunk_reduce<V, true><<<(unsigned)g, kThreads, smem, st>>>(P, cfirst, nchunks, ref, out);
+    k_codec_encode<V><<<(unsigned)g, kThreads, smem, st>>>(in, nchunks, kc, S, force, modes, out, stride, lens, err,
+                                                          warp ? todo : nullptr, pad ? 1 : 0);
   });
   return cudaGetLastError();
 }

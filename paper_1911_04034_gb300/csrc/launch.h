@@ -115,7 +115,12 @@ cudaError_t launch_codec_encode(const double* in, unsigned long long nchunks, in
                                 cudaStream_t st);
 cudaError_t launch_codec_encode(const double* in, unsigned long long nchunks, int kc, uint32_t S, int force,
                                 uint32_t modes, uint8_t* out, unsigned long long stride, uint32_t* lens,
-                                unsigned int* err, cudaStream_t st);
+                                unsigned int* err, unsigned int* todo, bool pad, cudaStream_t st);
+// todo: a device word set to 0 (or nullptr: no warp-per-chunk pass); pad: clear the rest of
+// every slot.
+cudaError_t launch_stream_encode(const double* in, unsigned long long nchunks, int kc, uint32_t S, uint8_t* out,
+                                 unsigned long long stride, uint32_t* lens, unsigned int* todo, bool pad,
+                                 cudaStream_t st);
 cudaError_t launch_codec_decode(const uint8_t* in, unsigned long long stride, const uint32_t* lens,
                                 unsigned long long nchunks, int kc, double* out, unsigned int* err, cudaStream_t st);
 cudaError_t launch_decode_range(const Pool& P, unsigned long long first_amp, unsigned long long count, double* out,

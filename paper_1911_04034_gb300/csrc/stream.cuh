@@ -1,0 +1,250 @@
+// stream.cuh -- STREAM images at S <= 32 bits, one warp a chunk, 256 values a pass (8 per
+// lane): what the streaming gate kernel (fast.cu) and the readout and codec kernels
+// (stream_io.cu) share.
+#pragma once
+#include "gate_common.cuh"
+
+namespace qc {
+
+constexpr uint32_t kFastWin = 1056;   // bytes of a pass window: 1024 bytes of stream at most, plus alignment and read slack
+constexpr uint32_t kWinBlocks = kFastWin / 16;
+__host__ __device__ __forceinline__ uint32_t fast_pg_words(int kc) { return (max_pages(kc) + 3u) & ~3u; }
+// Largest STREAM image of a chunk at S <= 32 bits.
+__host__ __device__ __forceinline__ uint32_t fast_max_image(int kc) {
+  return 16u + code_bytes(2u << kc) + resid_bytes(32u * (2u << kc));
+}
+
+// Bit position (within a lane's 16-bit code field) of the 2-bit code of the lane's
+// value k: four codes per byte, the first in the top bits, bytes in memory order.
+__host__ __device__ constexpr uint32_t code_shift(int k) { return 8u * (uint32_t)(k >> 2) + 6u - 2u * (uint32_t)(k & 3); }
+// 8 * (code of value k) from the lane's code field.
+template <int k>
+__device__ __forceinline__ uint32_t code8(uint32_t cw) {
+  constexpr uint32_t s = code_shift(k);
+  if constexpr (s >= 3) return (cw >> (s - 3)) & 0x18u;
+  else return (cw << (3 - s)) & 0x18u;
+}
+__device__ __forceinline__ uint32_t code8_at(uint32_t cw, int k) {
+  switch (k) {
+    case 0: return code8<0>(cw);
+    case 1: return code8<1>(cw);
+    case 2: return code8<2>(cw);
+    case 3: return code8<3>(cw);
+    case 4: return code8<4>(cw);
+    case 5: return code8<5>(cw);
+    case 6: return code8<6>(cw);
+    default: return code8<7>(cw);
+  }
+}
+__device__ __forceinline__ uint32_t rlen(uint32_t S, uint32_t c8) { return S > c8 ? S - c8 : 0u; }
+
+// Sum of the residual lengths max(S - 8c, 0) of the 8 codes of a lane's 16-bit field.
+__device__ __forceinline__ uint32_t rsum8(uint32_t cw, uint32_t S) {
+  const uint32_t lo = cw & 0x5555u, hi = (cw >> 1) & 0x5555u;
+  const uint32_t n1 = __popc(lo & ~hi), n2 = __popc(hi & ~lo), n3 = __popc(lo & hi);
+  return (8u - n1 - n2 - n3) * S + n1 * rlen(S, 8u) + n2 * rlen(S, 16u) + n3 * rlen(S, 24u);
+}
+
+// Exclusive warp scan (plus the warp total, to all lanes).
+__device__ __forceinline__ uint32_t warp_excl(uint32_t v, uint32_t& total) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t inc = v;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t u = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= (uint32_t)d) inc += u;
+  }
+  total = __shfl_sync(0xffffffffu, inc, 31);
+  return inc - v;
+}
+
+// The leading-byte run of a lane, packed: bits 8..31 the bytes its values set, bits 0..1
+// the smallest code among them (3: none set).  Composition (earlier A, later B): B's
+// explicit bytes replace A's; the smallest code is the smaller of the two.
+__device__ __forceinline__ uint32_t lead_compose(uint32_t A, uint32_t B) {
+  const uint32_t mb = B & 3u;
+  const uint32_t ex = 0xFFFFFF00u & (0xFFFFFFFFu >> (8u * mb));
+  return (A & ~ex & 0xFFFFFF00u) | (B & 0xFFFFFF00u) | min(A & 3u, mb);
+}
+// Exclusive warp scan of lead runs after `carry` (the top bytes of the value before the
+// warp's first): returns the top bytes of the lane's predecessor; `after` receives (on
+// all lanes) the top bytes of the warp's last value.
+__device__ __forceinline__ uint32_t lead_scan_warp(uint32_t W, uint32_t carry, uint32_t& after) {
+  const uint32_t lane = threadIdx.x & 31u;
+  if (__all_sync(0xffffffffu, (W & 3u) == 0u)) {
+    // every lane has a value with code 0 (all three leading bytes explicit): a lane's
+    // predecessor's leading bytes are the previous lane's run alone
+    uint32_t exc = __shfl_up_sync(0xffffffffu, W, 1);
+    if (lane == 0) exc = carry;
+    after = __shfl_sync(0xffffffffu, W, 31) & 0xFFFFFF00u;
+    return exc & 0xFFFFFF00u;
+  }
+  uint32_t inc = W;
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint32_t u = __shfl_up_sync(0xffffffffu, inc, d);
+    if (lane >= (uint32_t)d) inc = lead_compose(u, inc);
+  }
+  uint32_t exc = __shfl_up_sync(0xffffffffu, inc, 1);
+  if (lane == 0) exc = 3u;  // empty run
+  const uint32_t last = __shfl_sync(0xffffffffu, inc, 31);
+  const uint32_t cw = (carry & 0xFFFFFF00u) | 3u;
+  after = lead_compose(cw, last) & 0xFFFFFF00u;
+  return lead_compose(cw, exc) & 0xFFFFFF00u;
+}
+
+// Where a warp reads an image from: pool pages listed in shared memory, or one buffer.
+struct PagedImage {
+  const uint8_t* pages;
+  const uint32_t* ids;
+  __device__ __forceinline__ const uint8_t* at(uint32_t b) const {
+    return pages + (unsigned long long)ids[b >> 9] * kPage + (b & (kPage - 1u));
+  }
+};
+struct FlatImage {
+  const uint8_t* base;
+  __device__ __forceinline__ const uint8_t* at(uint32_t b) const { return base + b; }
+};
+
+// Stages stream blocks [wb, wb + kWinBlocks) of the input image (only those inside its
+// nbs stream blocks) into a window with cp.async.  16-byte block k of the stream is
+// image byte 16 + cb + 16k.
+template <class Image>
+__device__ __forceinline__ void fast_issue_window(const Image& img, uint32_t* win, uint32_t cb, uint32_t wb, uint32_t nbs) {
+  const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll
+  for (uint32_t k = lane; k < kWinBlocks; k += 32u) {
+    const uint32_t blk = wb + k;
+    if (blk < nbs) cp_async16(win + 4u * k, img.at(16u + cb + 16u * blk));
+  }
+}
+
+__device__ __forceinline__ double hi_as_double(uint32_t h) { return __longlong_as_double((long long)((uint64_t)h << 32)); }
+
+// The truncated high word of a result (S <= 32: the low word is always cut); a signed
+// zero becomes +0.  `spec` is set for a subnormal or non-finite result: a chunk holding
+// one is coded at 64 bits or is an error, which the general kernel handles.
+__device__ __forceinline__ uint32_t fast_trunc(double v, uint32_t mh, bool& spec) {
+  const uint64_t u = (uint64_t)__double_as_longlong(v);
+  const uint32_t hi = (uint32_t)(u >> 32), ahi = hi & 0x7fffffffu;
+  const bool zero = (ahi | (uint32_t)u) == 0u;
+  spec |= (ahi - 0x00100000u) >= 0x7fe00000u && !zero;
+  return zero ? 0u : (hi & mh);
+}
+
+// The explicit parts of a lane's 8 values from the input window (stream unit q at
+// win[(q ^ 1) - w4]), starting at stream bit o; e[k] receives bits [8c, S) of value k's
+// high word; returns the lane's lead run (see lead_compose).
+__device__ __forceinline__ uint32_t fast_extract(const uint32_t* win, uint32_t w4, uint32_t o, uint32_t cw,
+                                                 uint32_t S, uint32_t mh, uint32_t e[8]) {
+  uint32_t W = 3u;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const uint32_t c8 = code8_at(cw, k);
+    const uint32_t q = o >> 5;
+    const uint32_t x = __funnelshift_l(win[((q + 1u) ^ 1u) - w4], win[(q ^ 1u) - w4], o);
+    e[k] = (x >> c8) & mh;
+    o += rlen(S, c8);
+    const uint32_t ex = 0xFFFFFF00u & (0xFFFFFFFFu >> c8);
+    W = (W & ~ex & 0xFFFFFF00u) | (e[k] & ex) | min(W & 3u, c8 >> 3);
+  }
+  return W;
+}
+
+// Rebuilds the high words from the explicit parts: value k takes its copied leading
+// bytes from its predecessor (P: the top bytes of the lane's predecessor).
+__device__ __forceinline__ void fast_rebuild(uint32_t e[8], uint32_t cw, uint32_t P) {
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    P = e[k] | (P & ~(0xFFFFFFFFu >> code8_at(cw, k)));
+    e[k] = P;
+  }
+}
+
+// Codes of a lane's 8 truncated values (predecessor of the first: pr), as the lane's
+// 16-bit code field; `sum` receives their residual-length sum.
+__device__ __forceinline__ uint32_t fast_codes(const uint32_t t[8], uint32_t pr, uint32_t S, uint32_t& sum) {
+  uint32_t cw = 0u, s = 0u;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const uint32_t x = t[k] ^ (k ? t[k - 1] : pr);
+    const uint32_t c8 = min((uint32_t)__clz((int)x), 24u) & 0x18u;
+    s += rlen(S, c8);
+    cw |= (c8 >> 3) << code_shift(k);
+  }
+  sum = s;
+  return cw;
+}
+
+// Packs the residuals of a lane's 8 values (high words t, codes in the lane's code
+// field cw) at stream bit o of a cleared window whose block 0 is stream block w4 / 4
+// (stream unit q is win[(q ^ 1) - w4]).  The first unit the lane touches and its last,
+// unfinished one may be shared with the neighbouring lanes: atomicOr; units in
+// between are stored.
+__device__ __forceinline__ void fast_pack(uint32_t* win, uint32_t w4, uint32_t o, const uint32_t t[8], uint32_t cw,
+                                          uint32_t S) {
+  uint32_t q = o >> 5, fill = o & 31u, cur = 0u;
+  bool first = true;
+#pragma unroll
+  for (int k = 0; k < 8; ++k) {
+    const uint32_t c8 = code8_at(cw, k);
+    const uint32_t r = rlen(S, c8);
+    const uint32_t f = t[k] << c8;  // the residual in the top r bits, zeros below
+    cur |= f >> fill;
+    const uint32_t nf = fill + r;
+    if (nf >= 32u) {
+      if (first) atomicOr(&win[(q ^ 1u) - w4], cur);
+      else win[(q ^ 1u) - w4] = cur;
+      first = false;
+      ++q;
+      cur = __funnelshift_r(0u, f, fill);
+      fill = nf - 32u;
+    } else {
+      fill = nf;
+    }
+  }
+  if (fill > 0u && cur) atomicOr(&win[(q ^ 1u) - w4], cur);
+}
+
+// Decodes a STREAM image of ib bytes (header checked: width S, `bits` residual bits) pass by
+// pass: f(p, v) receives the high words of the lane's 8 values of pass p.  win: two windows
+// of kFastWin bytes.  False if the residual lengths disagree with the header.
+template <class Image, class F>
+__device__ __forceinline__ bool stream_decode(const Image& img, int kc, uint32_t S, uint32_t bits, uint32_t ib,
+                                              uint32_t* win0, uint32_t* win1, const F& f) {
+  const uint32_t lane = threadIdx.x & 31u, N = 2u << kc, cb = N >> 2, NP = N >> 8, nbs = (ib - 16u - cb) >> 4;
+  const uint32_t mh = (uint32_t)(trunc_mask(S) >> 32);
+  auto codes = [&](uint32_t p) { return *reinterpret_cast<const uint32_t*>(img.at(16u + 64u * p + 4u * (lane >> 1))); };
+  uint32_t cw_next = codes(0u), off = 0u, lead = 0u;
+  fast_issue_window(img, win0, cb, 0u, nbs);
+  cp_async_commit();
+  for (uint32_t p = 0; p < NP; ++p) {
+    uint32_t* const win = (p & 1u) ? win1 : win0;
+    const uint32_t cw = (cw_next >> (16u * (lane & 1u))) & 0xffffu;
+    if (p + 1u < NP) cw_next = codes(p + 1u);
+    uint32_t tot;
+    const uint32_t ps = off, o = ps + warp_excl(rsum8(cw, S), tot);
+    off += tot;
+    if (p + 1u < NP) fast_issue_window(img, (p & 1u) ? win0 : win1, cb, off >> 7, nbs);
+    cp_async_commit();
+    cp_async_wait_group<1>();
+    __syncwarp();
+    uint32_t v[8], after;
+    const uint32_t W = fast_extract(win, 4u * (ps >> 7), o, cw, S, mh, v);
+    const uint32_t before = lead_scan_warp(W, lead, after);
+    lead = after;
+    fast_rebuild(v, cw, before);
+    f(p, v);
+    __syncwarp();  // every lane is done with the window the next pass refills
+  }
+  return off == bits;
+}
+
+// True if image header hd (length ib) is a STREAM image at S <= 32 bits of a chunk of 2^kc.
+__device__ __forceinline__ bool stream32_header(const uint4& hd, uint32_t ib, int kc) {
+  const uint32_t N = 2u << kc, cb = N >> 2, S = (hd.x >> 8) & 0xffu;
+  return ib >= 16u + cb && ib <= fast_max_image(kc) && (ib & 15u) == 0u && (hd.x & 0xffu) == M_STREAM &&
+         (hd.x >> 16) == 0u && S >= 13u && S <= 32u && hd.y + 16u == ib && hd.z == N && cb + resid_bytes(hd.w) == hd.y;
+}
+
+}  // namespace qc

@@ -100,6 +100,7 @@ def lib():
             "sim_codec_decode": [vp, u64, vp, u64, i32, vp, i32],
             "sim_codec_encode_ex": [vp, u64, i32, dbl, i32, C.c_uint32, vp, u64, vp, i32],
             "sim_set_modes": [vp, C.c_uint32],
+            "sim_codec_encode_padded": [vp, u64, i32, dbl, i32, C.c_uint32, vp, u64, vp, i32],
             "sim_codec_encode_noalloc": [vp, u64, i32, dbl, i32, vp, u64, vp],
             "sim_batch_apply": [vp, i32, vp, vp, i32],
             "sim_autotune_chunk": [i32, i32, dbl, vp, sz, vp, i32, C.POINTER(C.c_int), vp],
@@ -442,9 +443,9 @@ def codec_encode(values, chunk_log2: int, eps: float, force_mode: int = -1, mode
         import torch
 
         n = values.numel() // (2 << chunk_log2)
-        out = torch.zeros(n * stride, dtype=torch.uint8, device=values.device)
-        lens = torch.zeros(n, dtype=torch.int32, device=values.device)
-        _check(lib().sim_codec_encode_ex(C.c_void_p(_ptr(values)), n, chunk_log2, float(eps), force_mode, modes,
+        out = torch.empty(n * stride, dtype=torch.uint8, device=values.device)  # every slot written whole
+        lens = torch.empty(n, dtype=torch.int32, device=values.device)
+        _check(lib().sim_codec_encode_padded(C.c_void_p(_ptr(values)), n, chunk_log2, float(eps), force_mode, modes,
                                          C.c_void_p(_ptr(out)), stride, C.c_void_p(_ptr(lens)), 1), "sim_codec_encode")
         return out, lens, stride
     x = np.ascontiguousarray(values, dtype=np.complex128)

@@ -179,3 +179,34 @@ def test_palette_mode_forced_and_decoded_like_the_oracle(kc):
             assert imgs[0] == ref, (P, eps)
             dec = q.codec_decode([ref], kc)
             assert np.array_equal(dec.view(np.uint64), O.decode_chunk(ref, kc).view(np.uint64))
+
+
+@pytest.mark.parametrize("eps", [1e-5, 1e-3])
+@pytest.mark.parametrize("kc", [7, 8, 10])
+def test_many_chunks_at_once_match_oracle(kc, eps):
+    """Enough chunks for the warp-per-chunk encoder and decoder (not a multiple of eight),
+    every structure among them: bytes, lengths, cleared slots and decoded values."""
+    import torch
+
+    rng = np.random.default_rng(kc)
+    chunks = chunk_families(rng, kc, 2459 if kc < 10 else 2440)
+    x = np.concatenate(chunks)
+    dev = torch.from_numpy(x.view(np.float64).copy()).cuda()
+    out, lens, stride = qc().codec_encode(dev, kc, eps)
+    buf, n = out.cpu().numpy().reshape(-1, stride), lens.cpu().numpy()
+    S = O.sig_bits(eps)
+    refs = [O.encode_chunk(a, kc, S) for a in chunks]
+    for k, ref in enumerate(refs):
+        assert n[k] == len(ref) and buf[k, : n[k]].tobytes() == ref, k
+        assert not buf[k, n[k]:].any(), k
+    back = torch.empty_like(dev)
+    rc = qc().lib().sim_codec_decode(out.data_ptr(), stride, lens.data_ptr(), len(chunks), kc, back.data_ptr(), 1)
+    assert rc == qc().OK
+    got = back.cpu().numpy().reshape(len(chunks), -1)
+    for k, ref in enumerate(refs):
+        assert np.array_equal(got[k].view(np.uint64), O.decode_chunk(ref, kc).view(np.uint64).reshape(-1)), k
+    bad = out.clone().view(-1, stride)
+    k = next(k for k, ref in enumerate(refs) if ref[0] == 3)  # a STREAM image with a damaged code
+    bad[k, 16] ^= 0xC0
+    rc = qc().lib().sim_codec_decode(bad.data_ptr(), stride, lens.data_ptr(), len(chunks), kc, back.data_ptr(), 1)
+    assert rc == qc().ERR_CORRUPT

@@ -173,3 +173,35 @@ def test_gate_by_gate_and_whole_circuit_agree(kc, modes):
         orc = O.CSim(m, m, kc, 1e-4, raw // 3, modes=modes)
         orc.apply(gates)
         assert got[0][0] == [orc.image(c) for c in range(orc.nchunks)], ci
+
+
+@pytest.mark.parametrize("eps", [0.0, 1e-4])
+def test_readout_of_many_chunks(eps):
+    """Enough chunks for the warp-per-chunk readout: ragged ranges into aligned and
+    unaligned buffers, measurement and fidelity, with STREAM and other images mixed."""
+    import torch
+
+    n, kc = 20, 8
+    s = qc().Sim(n, n, eps, chunk_log2=kc, budget=(16 << n) // 2 if eps else 2 * (16 << n), pool_bytes=2 * (16 << n) + (64 << 20))
+    s.apply_circuit(Cc.rcs_n(n, 3, seed=2))
+    s.apply_circuit(Cc.to_array([Cc.gate(n - 1, Cc.X, {q: 1 for q in range(8, n - 1)})]))
+    whole = np.concatenate([s.amplitudes(a, 1 << 17) for a in range(0, 1 << n, 1 << 17)])  # few chunks a call: a CTA each
+    assert np.array_equal(s.amplitudes().view(np.uint64), whole.view(np.uint64))
+    for first, count, skew in ((0, 1 << n, 0), (12345, (1 << n) - 20000, 0), (1, (1 << n) - 1, 1)):
+        out = torch.full((2 * count + 3,), 7.0, dtype=torch.float64, device="cuda")
+        s.amplitudes(first, count, out=out[skew: skew + 2 * count])
+        got = out.cpu().numpy()
+        assert np.array_equal(got[skew: skew + 2 * count].view(np.uint64), whole[first: first + count].view(np.float64).view(np.uint64))
+        assert (got[skew + 2 * count:] == 7.0).all() and (got[:skew] == 7.0).all()
+    ref = np.random.default_rng(1).standard_normal(2 << n).view(np.complex128)
+    ref /= np.linalg.norm(ref)
+    for skew in (0, 1):
+        dev = torch.empty((2 << n) + 1, dtype=torch.float64, device="cuda")[skew: skew + (2 << n)]
+        dev.copy_(torch.from_numpy(ref.view(np.float64).copy()))
+        f = s.fidelity(dev)
+        assert f["F"] == pytest.approx(abs(np.vdot(ref, whole)), rel=1e-10)
+        assert f["norm2"] == pytest.approx(float(np.vdot(whole, whole).real), rel=1e-12)
+    p = np.abs(whole) ** 2
+    for seed in range(5):
+        outcome, prob = s.measure(seed)
+        assert prob == pytest.approx(p[outcome] / p.sum(), rel=1e-10)
