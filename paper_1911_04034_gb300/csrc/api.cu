@@ -516,6 +516,8 @@ static GateLaunch make_launch(sim* s, const sim_gate* g) {
     const bool perm = u[0] == 0 && u[1] == 0 && u[6] == 0 && u[7] == 0;
     L.gfeat = (real ? 1u : 0u) | (diag ? 2u : 0u) | (perm ? 4u : 0u) | (t < kc ? 8u : 0u);
     // a cross-chunk diagonal gate with a row that is an exact copy: the row that is not
+    L.diag = diag ? 1 : 0;
+    L.copy = diag ? (u[0] == 1.0 && u[1] == 0.0 ? 1u : 0u) | (u[6] == 1.0 && u[7] == 0.0 ? 2u : 0u) : 0u;
     L.solo = -1;
     if (t >= kc && diag) L.solo = u[0] == 1.0 && u[1] == 0.0 ? 1 : (u[6] == 1.0 && u[7] == 0.0 ? 0 : -1);
     // a coefficient that can turn a normal value into a subnormal (see next_level)
@@ -615,11 +617,30 @@ static bool fast_applies(const sim* s, const sim_gate* g, GateLaunch& L) {
 }
 
 // True if circuits run by k_run: small states with no option that needs a kernel of its own
-// around each gate (timing, the selector network) or its counters (block cache, traces).
+// around each gate (timing, the selector network) or its counters (block cache, traces,
+// trials).
 static bool run_options(const sim* s) {
-  return s->fast && !s->timing && !s->phases && s->selector != 2 && !s->d_trace && !s->d_bc;
+  return s->fast && s->modes == qc::kDefaultModes && !s->timing && !s->phases && s->selector != 2 && !s->d_trace && !s->d_bc;
 }
 static bool run_applies(const sim* s) { return s->run_grid > 0 && run_options(s); }
+
+// For every gate of a launch the longest step of k_run that could begin with it: gates that
+// leave pairs of chunks to themselves, i.e. at most one chunk-index bit among their
+// non-diagonal targets.  An image exchange (swap) is a step of its own.
+static void mark_groups(GateLaunch* rec, size_t n) {
+  for (size_t k = 0; k < n; ++k) {
+    GateLaunch& L = rec[k];
+    L.group = 1;
+    L.group_bit = L.pair && !L.diag ? L.pair_bit : 0ull;
+    if (L.swap) continue;
+    for (size_t j = k + 1; j < n && j - k < (size_t)qc::kRunGroup && !rec[j].swap; ++j) {
+      const uint64_t bit = rec[j].pair && !rec[j].diag ? rec[j].pair_bit : 0ull;
+      if (bit && L.group_bit && bit != L.group_bit) break;
+      if (bit) L.group_bit = bit;
+      L.group = (int)(j - k) + 1;
+    }
+  }
+}
 
 // Page ids each of a run's CTAs may keep between gates: all together no more than the pool
 // has beyond every chunk stored RAW, so that kept pages never make it run dry.
@@ -705,6 +726,7 @@ static sim_status run_circuit(sim* s, const sim_gate* gates, size_t n, bool* ran
         s->h_run[off + k] = make_launch(s, gates + done + off + k);
         s->amp_updates += s->h_run[off + k].nact << s->kc;
       }
+      mark_groups(s->h_run + off, m);
       s->h_run_jobs[seg] = {s->d_run + off, (int)m, 0, s->run_grid, run_keep(s, s->run_grid)};
       CK(cudaMemcpyAsync(s->d_run + off, s->h_run + off, m * sizeof(GateLaunch), cudaMemcpyHostToDevice, s->st), "gate records");
       CK(cudaMemcpyAsync(s->d_run_jobs + seg, s->h_run_jobs + seg, sizeof(qc::RunJob), cudaMemcpyHostToDevice, s->st), "gate records");
@@ -1249,7 +1271,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
     // numbered consecutively.
     const int resident = device_sms() * qc::run_ctas_per_sm(kc);
     bool whole = count <= resident / 2;
-    for (int k = 0; k < count; ++k) whole = whole && run_options(sims[k]);
+    for (int k = 0; k < count; ++k) whole = whole && run_options(sims[k]) && n_gates[k] < (1u << 20);
     std::vector<qc::BatchJob> jobs;
     std::vector<sim*> job_sim;  // the handle of each job
     std::vector<size_t> off(steps + 1, 0);
@@ -1272,6 +1294,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
           upd[k] += L.nact << sims[k]->kc;
           std::memcpy(rec, &L, sizeof L);
         }
+        mark_groups(rec - n_gates[k], n_gates[k]);
       }
       const std::vector<int> ctas = run_shares(first, n_gates, count, resident);
       CK(cudaMalloc(&d_jobs, run_list.size()), "batch job list");

@@ -57,6 +57,9 @@ __host__ __device__ __forceinline__ uint32_t max_pages(int kc) { return (max_ima
 __host__ __device__ __forceinline__ uint32_t dir_stride(int kc) { return round16(16u + 4u * max_pages(kc)); }
 __host__ __device__ __forceinline__ uint32_t inline_cap(int kc) { return dir_stride(kc) - 16u; }
 
+// Most gates in a step of k_run.
+constexpr int kRunGroup = 32;
+
 // ------------------------------------------------------------- device state -- //
 // Counters and controller state of one simulator, in device memory.
 struct DevCtl {
@@ -97,8 +100,11 @@ struct DevCtl {
   unsigned long long palette_trials;   // chunk encodes that ran the PALETTE trial
   long long n64;                       // images whose header says S = 64 (as of the last gate)
   long long dn64;                      // ... its change during the running gate
-  unsigned int run_arrived;            // k_run: CTAs that finished a gate (cumulative over the launch)
-  unsigned int run_gate;               // k_run: gates finished and booked in the launch
+  unsigned int run_arrived;            // k_run: CTAs that finished a step (cumulative over the launch)
+  unsigned int run_gate;               // k_run: steps finished and booked in the launch
+  long long run_dE[kRunGroup];         // k_run: changes of E, n64 and pages by each gate of the running step
+  long long run_dn64[kRunGroup];
+  long long run_dpages[kRunGroup];
 };
 
 // Controller parameters (host-computed, constant for the handle).

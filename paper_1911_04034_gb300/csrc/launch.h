@@ -25,6 +25,10 @@ struct alignas(16) GateLaunch {
   uint32_t lo_mask, lo_vals;     // controls inside a chunk
   int target;                    // target bit (in-chunk gates)
   int pair;                      // 1: target >= chunk_log2
+  int diag;                      // 1: the matrix is diagonal
+  uint32_t copy;                 // diagonal: bit r, row r is an exact copy
+  int group;                     // k_run: gates, this one first, that one step can take (see mark_groups)
+  unsigned long long group_bit;  // ... and the chunk-index bit of their cross-chunk target, 0 if none
   int swap;                      // 1: X between chunks that may exchange whole images (see swap_item)
   int prof;                      // 1: accumulate per-phase SM cycles
   uint32_t modes;                // chunk modes the encoder may choose (bit m = mode m)
