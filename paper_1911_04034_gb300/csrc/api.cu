@@ -159,10 +159,12 @@ struct sim {
   // whole circuits in one launch (k_run): staging for up to kRunBlock gate records
   GateLaunch* h_run = nullptr;       // pinned
   GateLaunch* d_run = nullptr;
-  qc::RunJob* h_run_jobs = nullptr;  // pinned, kRunSegments
+  qc::RunJob* h_run_jobs = nullptr;  // pinned, run_cap + kRunSegments
   qc::RunJob* d_run_jobs = nullptr;
   size_t run_cap = 0;
   int run_grid = 0;                  // its CTAs (0: not used for this state)
+  int group_grid = 0;                // CTAs of k_group (0: not used for this state)
+  int rest_grid = 0;                 // ... and of the k_run launch after it
   int fast_grid = 0;                 // CTAs of the streaming kernel (0: chunk size outside its range)
   bool fast = true;                  // gates try the streaming kernel first
   uint64_t kernel_launches = 0;      // gate, streaming and post kernels enqueued
@@ -364,12 +366,18 @@ sim_status sim_create_ex(int n_qubits, int block_log2, int chunk_log2, double er
     s->fast_grid = (uint64_t)s->fast_grid < cap ? s->fast_grid : (int)cap;
   }
   // Whole circuits in one launch (see run_applies) where the resident CTAs take the largest
-  // gate in one round; from two rounds on the streaming kernel's throughput counts for more
-  // than its launches (2^10-amplitude chunks, 256 items 28 us a gate against 49; 512 items
-  // 55 against 49).
+  // gate in one round; from two rounds on groups of gates by the streaming code are faster
+  // (2^10-amplitude chunks, 256 items 19 us a gate here; 512 items 36 against 23 by groups
+  // and 50 gate by gate).
   {
     const uint64_t fit = (uint64_t)device_sms() * qc::run_ctas_per_sm(s->kc), items = (s->nchunks + 1) / 2;
     if (items <= fit) s->run_grid = (int)items;
+    // larger states: groups of gates (see group_circuit)
+    if (!s->run_grid && s->fast_grid && cp.nlevels > 0 && cp.S[cp.nlevels - 1] <= 32) {
+      const int resident = device_sms() * qc::group_ctas_per_sm(s->kc), room = s->fast_grid * qc::fast_warps() / qc::group_warps();
+      s->group_grid = resident < room ? resident : room;
+      s->rest_grid = (int)(items < fit ? items : fit);
+    }
   }
   Pool& P = s->P;
   if (!P.wkeep) P.wkeep = (uint32_t)qc::fast_warp_cache();
@@ -697,25 +705,31 @@ static std::vector<int> run_shares(const std::vector<const GateLaunch*>& first, 
   return c;
 }
 
-// Enqueues the gates as launches of k_run, the first ones short so that the device starts
-// while the host still prepares the rest.  False: no memory for the staging buffers.
 constexpr size_t kRunBlock = 4096;     // gate records staged at once
 constexpr size_t kRunSegments = 64;    // launches they make at most
-static sim_status run_circuit(sim* s, const sim_gate* gates, size_t n, bool* ran) {
-  *ran = false;
+// The staging buffers for a circuit of n gates; false: no memory for them.
+static bool run_stage(sim* s, size_t n) {
   const size_t want = n < kRunBlock ? n : kRunBlock;
   if (s->run_cap < want) {
     s->drop_run();
     if (cudaMallocHost(&s->h_run, want * sizeof(GateLaunch)) != cudaSuccess ||
-        cudaMallocHost(&s->h_run_jobs, kRunSegments * sizeof(qc::RunJob)) != cudaSuccess ||
+        cudaMallocHost(&s->h_run_jobs, (want + kRunSegments) * sizeof(qc::RunJob)) != cudaSuccess ||
         cudaMalloc(&s->d_run, want * sizeof(GateLaunch)) != cudaSuccess ||
-        cudaMalloc(&s->d_run_jobs, kRunSegments * sizeof(qc::RunJob)) != cudaSuccess) {
+        cudaMalloc(&s->d_run_jobs, (want + kRunSegments) * sizeof(qc::RunJob)) != cudaSuccess) {
       cudaGetLastError();
       s->drop_run();
-      return SIM_OK;
+      return false;
     }
     s->run_cap = want;
   }
+  return true;
+}
+
+// Enqueues the gates as launches of k_run, the first ones short so that the device starts
+// while the host still prepares the rest.  False: no memory for the staging buffers.
+static sim_status run_circuit(sim* s, const sim_gate* gates, size_t n, bool* ran) {
+  *ran = false;
+  if (!run_stage(s, n)) return SIM_OK;
   *ran = true;
   for (size_t done = 0; done < n;) {
     const size_t block = n - done < s->run_cap ? n - done : s->run_cap;
@@ -727,7 +741,7 @@ static sim_status run_circuit(sim* s, const sim_gate* gates, size_t n, bool* ran
         s->amp_updates += s->h_run[off + k].nact << s->kc;
       }
       mark_groups(s->h_run + off, m);
-      s->h_run_jobs[seg] = {s->d_run + off, (int)m, 0, s->run_grid, run_keep(s, s->run_grid)};
+      s->h_run_jobs[seg] = {s->d_run + off, (int)m, 0, s->run_grid, run_keep(s, s->run_grid), nullptr};
       CK(cudaMemcpyAsync(s->d_run + off, s->h_run + off, m * sizeof(GateLaunch), cudaMemcpyHostToDevice, s->st), "gate records");
       CK(cudaMemcpyAsync(s->d_run_jobs + seg, s->h_run_jobs + seg, sizeof(qc::RunJob), cudaMemcpyHostToDevice, s->st), "gate records");
       CK(qc::launch_run(s->d_run_jobs + seg, 1, s->kc, s->run_grid, s->st), "circuit kernel launch");
@@ -805,6 +819,86 @@ static sim_status enqueue_gate(sim* s, const sim_gate* g) {
   return SIM_OK;
 }
 
+// True if a large state's circuits run by groups of gates once the bound is settled.
+static bool group_applies(const sim* s) { return s->group_grid > 0 && s->rest_grid > 0 && run_options(s); }
+
+// The gates [0, L.group) from L on as one step of k_group.
+static void fill_group(const sim* s, const sim_gate* gates, const GateLaunch* rec, qc::GroupLaunch& G) {
+  G.P = s->P;
+  G.S = (uint32_t)s->cp.S[s->cp.nlevels - 1];
+  G.ngates = rec[0].group;
+  G.bit = rec[0].group_bit ? rec[0].group_bit : 1ull;
+  G.items = s->nchunks / 2ull;
+  G.defer = s->d_defer;
+  for (int k = 0; k < G.ngates; ++k) {
+    GateLaunch L = rec[k];
+    fast_applies(s, gates + k, L);  // the arithmetic form
+    qc::GroupGate& g = G.g[k];
+    g.fixed = (s->nchunks - 1ull) & ~(L.free_mask | L.pair_bit);
+    g.hi_vals = L.hi_vals;
+    g.pair_bit = L.pair_bit;
+    g.lo_mask = L.lo_mask;
+    g.lo_vals = L.lo_vals;
+    g.target = L.target;
+    g.kind = L.diag ? 3 : (L.pair ? 4 : (L.target < 2 ? 0 : (L.target < 7 ? 1 : 2)));
+    g.arith = L.arith;
+    g.copy = L.copy;
+    g.sgn = L.sgn;
+    g.sk = L.sk;
+    for (int r = 0; r < 2; ++r) g.rop[r] = L.rop[r];
+    for (int q = 0; q < 16; ++q) g.cf[q] = L.cf[q];
+    for (int q = 0; q < 4; ++q) g.du[q] = L.du[q];
+  }
+}
+
+// A circuit on a large state: gate by gate until the bound is settled (the host looks every
+// kSettleGates gates), then by groups, a gate that makes a group by itself by its own kernels.
+constexpr size_t kSettleGates = 8;
+static sim_status group_circuit(sim* s, const sim_gate* gates, size_t n) {
+  size_t i = 0;
+  for (;;) {
+    int level = 0;
+    CK(cudaMemcpyAsync(&level, &s->d_ctl->level, sizeof level, cudaMemcpyDeviceToHost, s->st), "controller level");
+    CK(cudaStreamSynchronize(s->st), "sync");
+    if (level >= s->cp.nlevels || i == n) break;
+    for (const size_t end = i + kSettleGates < n ? i + kSettleGates : n; i < end; ++i)
+      if (sim_status r = enqueue_gate(s, gates + i)) return r;
+  }
+  if (i < n && !run_stage(s, n - i)) {  // no room for the gate records
+    for (; i < n; ++i)
+      if (sim_status r = enqueue_gate(s, gates + i)) return r;
+  }
+  qc::GroupLaunch G;
+  while (i < n) {
+    const size_t block = n - i < s->run_cap ? n - i : s->run_cap;
+    for (size_t k = 0; k < block; ++k) s->h_run[k] = make_launch(s, gates + i + k);
+    mark_groups(s->h_run, block);
+    size_t jobs = 0;
+    for (size_t k = 0; k < block; k += (size_t)s->h_run[k].group)
+      if (s->h_run[k].group > 1)
+        s->h_run_jobs[jobs++] = {s->d_run + k, s->h_run[k].group, 0, s->rest_grid, 0u, s->d_defer};
+    CK(cudaMemcpyAsync(s->d_run, s->h_run, block * sizeof(GateLaunch), cudaMemcpyHostToDevice, s->st), "gate records");
+    CK(cudaMemcpyAsync(s->d_run_jobs, s->h_run_jobs, jobs * sizeof(qc::RunJob), cudaMemcpyHostToDevice, s->st), "gate records");
+    jobs = 0;
+    for (size_t k = 0; k < block;) {
+      const int len = s->h_run[k].group;
+      if (len == 1) {
+        if (sim_status r = enqueue_gate(s, gates + i + k)) return r;
+      } else {
+        fill_group(s, gates + i + k, s->h_run + k, G);
+        CK(qc::launch_group(G, s->group_grid, s->st), "gate group kernel launch");
+        CK(qc::launch_run(s->d_run_jobs + jobs++, 1, s->kc, s->rest_grid, s->st), "circuit kernel launch");
+        s->kernel_launches += 2;
+        for (int q = 0; q < len; ++q) s->amp_updates += s->h_run[k + q].nact << s->kc;
+      }
+      k += (size_t)len;
+    }
+    i += block;
+    if (i < n) CK(cudaStreamSynchronize(s->st), "sync");  // the staging buffers are free again
+  }
+  return SIM_OK;
+}
+
 sim_status sim_apply_gate(sim_t* s, const sim_gate* g) {
   if (!s || !g) return fail(SIM_ERR_INVALID, "NULL argument");
   if (sim_status r = s->guard()) return r;
@@ -822,6 +916,10 @@ sim_status sim_apply_circuit(sim_t* s, const sim_gate* gates, size_t n_gates) {
   bool ran = false;
   if (run_applies(s) && n_gates)
     if (sim_status r = run_circuit(s, gates, n_gates, &ran)) return r;
+  if (!ran && n_gates > 1 && group_applies(s)) {
+    if (sim_status r = group_circuit(s, gates, n_gates)) return r;
+    ran = true;
+  }
   for (size_t k = 0; k < n_gates && !ran; ++k)
     if (sim_status r = enqueue_gate(s, gates + k)) return r;
   return s->check_device();
@@ -1302,7 +1400,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
         if (!n_gates[k]) continue;
         const size_t at = (size_t)(reinterpret_cast<const uint8_t*>(first[k]) - run_list.data());
         const qc::RunJob j{reinterpret_cast<const GateLaunch*>((const uint8_t*)d_jobs + at), (int)n_gates[k], run_grid,
-                           ctas[k], run_keep(sims[k], ctas[k])};
+                           ctas[k], run_keep(sims[k], ctas[k]), nullptr};
         std::memcpy(run_list.data() + (size_t)njobs++ * sizeof j, &j, sizeof j);
         run_grid += ctas[k];
       }

@@ -49,7 +49,6 @@ constexpr int kFastThreads = 32 * kFastWarps;
 #define QC_FAST_MIN_CTAS 3
 #endif
 constexpr size_t kSmSharedBytes = 227u * 1024u;
-constexpr uint32_t kWarpCache = 64;   // page ids a warp keeps between its items
 
 // Passes held in a warp's exchange area: two for the partner warp (cross-chunk pairs);
 // for an in-chunk target t >= 7 the 2^(t-7) passes between an amplitude and its partner.
@@ -61,237 +60,6 @@ __host__ __device__ __forceinline__ uint32_t fast_held(int kind, int target) {
 // pass of the chunk's first half.
 __host__ __device__ __forceinline__ uint32_t fast_warp_bytes(int kc, uint32_t held) {
   return 3u * kFastWin + 8u * fast_pg_words(kc) + held * 1024u + 4u * kWarpCache + 16u + (1u << (kc - 1));
-}
-
-// A warp's own page cache in shared memory: ids[0, *n).
-struct WarpPages {
-  uint32_t* ids;
-  uint32_t* n;
-};
-
-// All lanes: at least `want` (<= 32) ids in the cache, refilled from the global stack
-// half a cache (P.wkeep / 2) at a time.  False (E_OOM set, the stack top restored) if the stack is dry.
-__device__ __forceinline__ bool wp_reserve(const Pool& P, const WarpPages& wp, uint32_t want) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t n = *wp.n;
-  if (n >= want) return true;
-  const uint32_t take = max(want - n, P.wkeep / 2u);  // at most 32
-  long long old = 0;
-  if (lane == 0)
-    old = (long long)atomicAdd(reinterpret_cast<unsigned long long*>(&P.ctl->top), (unsigned long long)(-(long long)take));
-  old = __shfl_sync(0xffffffffu, old, 0);
-  if (old - (long long)take < 0) {  // the stack is dry: give the reservation back (top never stays below 0)
-    if (lane == 0) {
-      atomicAdd(reinterpret_cast<unsigned long long*>(&P.ctl->top), (unsigned long long)take);
-      atomicOr(&P.ctl->err, (unsigned)E_OOM);
-    }
-    return false;
-  }
-  if (lane < take) wp.ids[n + lane] = P.stack[old - 1 - (long long)lane];
-  __syncwarp();
-  if (lane == 0) *wp.n = n + take;
-  __syncwarp();
-  return true;
-}
-
-// All lanes: pushes ids[0, cnt) into the cache; what does not fit goes to the global
-// freed list (merged into the stack after the gate).
-__device__ __forceinline__ void wp_free(const Pool& P, const WarpPages& wp, const uint32_t* ids, uint32_t cnt) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t n = *wp.n, room = P.wkeep > n ? P.wkeep - n : 0u;
-  unsigned long long base = 0;
-  if (cnt > room) {
-    if (lane == 0) base = atomicAdd(&P.ctl->nfreed, (unsigned long long)(cnt - room));
-    base = __shfl_sync(0xffffffffu, base, 0);
-  }
-  for (uint32_t q = lane; q < cnt; q += 32u) {
-    const uint32_t id = ids[q];
-    if (q < room) {
-      wp.ids[n + q] = id;
-    } else {
-      const unsigned long long at = base + (q - room);
-      if (at < P.npages) P.freed[at] = id;  // the list holds every page at most once
-      else atomicOr(&P.ctl->err, (unsigned)E_CORRUPT);
-    }
-  }
-  __syncwarp();
-  if (lane == 0) *wp.n = n + min(cnt, room);
-  __syncwarp();
-}
-
-// All lanes: the output page list grows to `need` pages.
-__device__ __forceinline__ bool wp_grow(const Pool& P, const WarpPages& wp, uint32_t* opg, uint32_t& onp,
-                                        uint32_t need) {
-  while (onp < need) {
-    const uint32_t k = min(need - onp, 32u);
-    if (!wp_reserve(P, wp, k)) return false;
-    const uint32_t lane = threadIdx.x & 31u;
-    const uint32_t n = *wp.n;
-    if (lane < k) opg[onp + lane] = wp.ids[n - 1u - lane];
-    __syncwarp();
-    if (lane == 0) *wp.n = n - k;
-    __syncwarp();
-    onp += k;
-  }
-  return true;
-}
-
-// The two warps of a pair meet through a sequence number per warp in shared memory:
-// each raises its own to `phase` (after its earlier shared-memory writes) and waits
-// until the partner's has reached it.  The wait is bounded: after kSpinLimit polls it
-// sets E_TIMEOUT (and the site) and returns false, so no protocol error can hang the
-// kernel.
-constexpr uint32_t kSpinLimit = 1u << 22;
-__device__ __forceinline__ bool pair_sync(volatile uint32_t* seq, uint32_t side, uint32_t phase, DevCtl* ctl,
-                                          uint32_t site) {
-  __syncwarp();
-  bool ok = true;
-  if ((threadIdx.x & 31u) == 0) {
-    __threadfence_block();
-    seq[side] = phase;
-    uint32_t it = 0;
-    while ((int)(seq[side ^ 1u] - phase) < 0) {
-      if (++it > kSpinLimit) {
-        ok = false;
-        atomicOr(&ctl->err, (unsigned)E_TIMEOUT);
-        atomicExch(&ctl->timeout_site, site);
-        break;
-      }
-    }
-    __threadfence_block();
-  }
-  ok = __shfl_sync(0xffffffffu, ok ? 1u : 0u, 0) != 0u;
-  __syncwarp();  // orders lane 0's acquire before the other lanes' reads
-  return ok;
-}
-
-// The two warps of a pair agree on a flag word: each publishes its own, then both read
-// both.  Slots alternate, so a slot is rewritten only after the partner has passed the
-// next meeting, i.e. after it read the slot.  A failed wait reads as an error (bit 1).
-__device__ __forceinline__ uint32_t pair_agree(uint32_t* slots, volatile uint32_t* seq, uint32_t& phase,
-                                               uint32_t side, uint32_t mine, DevCtl* ctl, uint32_t site) {
-  volatile uint32_t* s = slots + 2u * (phase & 1u);
-  if ((threadIdx.x & 31u) == 0) s[side] = mine;
-  ++phase;
-  if (!pair_sync(seq, side, phase, ctl, site)) return 2u;
-  return s[side ^ 1u];
-}
-
-// One output amplitude of a dense-class gate: row pair (r, r + 1) of Eq. matrix1 /
-// matrix2 over every coefficient (cf: that row pair's eight, from GateLaunch.cf), in
-// the order of the kept-term sums; zero coefficients add exact zeros.
-__device__ __forceinline__ double2 dense_rows(const double* cf, double2 a, double2 b) {
-  return make_double2(__fma_rn(cf[3], b.y, __fma_rn(cf[2], b.x, __fma_rn(cf[1], a.y, __dmul_rn(cf[0], a.x)))),
-                      __fma_rn(cf[7], b.x, __fma_rn(cf[6], b.y, __fma_rn(cf[5], a.x, __dmul_rn(cf[4], a.y)))));
-}
-
-// The same output for a real matrix (every imaginary coefficient zero): the chains
-// above with their zero terms left out -- each dropped term adds an exact zero -- so
-// the products of the real parts alone, in the same order (cf[0] = cf[4] = the row's
-// first real coefficient, cf[2] = cf[6] its second).
-__device__ __forceinline__ double2 real_rows(const double* cf, double2 a, double2 b) {
-  return make_double2(__fma_rn(cf[2], b.x, __dmul_rn(cf[0], a.x)), __fma_rn(cf[2], b.y, __dmul_rn(cf[0], a.y)));
-}
-
-// The same output for a gate whose coefficient parts are all +-2^k, none zero (sqrt(X),
-// sqrt(Y)): every product of the chains above is exact, so each chain equals 2^k times
-// the chain of the signed inputs in the same order (scaling by a power of two commutes
-// with rounding while no partial sum leaves the normal range): three additions per
-// output part, then the scale added to the exponent field.  The inputs are checked
-// once per pass (an item holding a value below 2^-959 goes to the general kernel), and
-// then no partial sum leaves the normal range: inputs of at least 2^-959 truncated to at
-// most 20 mantissa bits are multiples of 2^-979, so a nonzero sum is at least that, and
-// 2^k <= 1.  Only an overflow to infinity is left to catch.  Bit q of L.sgn is the sign
-// of coefficient cf[q].
-__device__ __forceinline__ void signed_rows(const GateLaunch& L, uint32_t r, uint32_t ar, uint32_t ai, uint32_t br,
-                                            uint32_t bi, uint32_t mh, uint32_t& outr, uint32_t& outi, bool& spec) {
-  const uint32_t sg = L.sgn >> (8u * r);
-  auto t = [&](int q, uint32_t h) { return hi_as_double(h ^ ((sg >> q) << 31)); };
-  const double re = __dadd_rn(__dadd_rn(__dadd_rn(t(0, ar), t(1, ai)), t(2, br)), t(3, bi));
-  const double im = __dadd_rn(__dadd_rn(__dadd_rn(t(4, ai), t(5, ar)), t(6, bi)), t(7, br));
-  auto scaled = [&](double y) -> uint32_t {
-    const uint64_t u = (uint64_t)__double_as_longlong(y);
-    const uint32_t hi = (uint32_t)(u >> 32);
-    if ((hi & 0x7fffffffu) == 0u && (uint32_t)u == 0u) return 0u;
-    spec |= (hi & 0x7ff00000u) == 0x7ff00000u;
-    return (hi + ((uint32_t)L.sk << 20)) & mh;
-  };
-  outr = scaled(re);
-  outi = scaled(im);
-}
-
-// Row r of a diagonal (x = the amplitude itself) or anti-diagonal (x = its partner)
-// gate on x, given as high words: a complex product in the order of the kept-term sums,
-// or an exact copy / negation done on the high words (no FP64); results truncated.
-__device__ __forceinline__ void row_op(const GateLaunch& L, uint32_t r, uint32_t xr, uint32_t xi, uint32_t mh,
-                                       uint32_t& outr, uint32_t& outi, bool& spec) {
-  const int op = L.rop[r];
-  if (op == 0) {
-    const double ur = L.du[2u * r], ui = L.du[2u * r + 1u];
-    const double x = hi_as_double(xr), y = hi_as_double(xi);
-    outr = fast_trunc(__fma_rn(-ui, y, __dmul_rn(ur, x)), mh, spec);
-    outi = fast_trunc(__fma_rn(ui, x, __dmul_rn(ur, y)), mh, spec);
-  } else if (op == 1) {
-    outr = xr & mh;
-    outi = xi & mh;
-  } else {
-    outr = xr ? ((xr ^ 0x80000000u) & mh) : 0u;
-    outi = xi ? ((xi ^ 0x80000000u) & mh) : 0u;
-  }
-}
-
-// Both outputs of an ARITH 4 pair held by one lane.  The first sums of the four chains of
-// signed_rows are +-(ar + ai) and +-(ar - ai): two additions serve all four, 10 FP64
-// additions instead of 12 (a zero sum's sign may differ; a zero is stored as +0).
-__device__ __forceinline__ void signed_pair(const GateLaunch& L, uint32_t ar, uint32_t ai, uint32_t br, uint32_t bi,
-                                            uint32_t mh, uint32_t o[4], bool& spec) {
-  const uint32_t sg = L.sgn;
-  const double sum = __dadd_rn(hi_as_double(ar), hi_as_double(ai)), dif = __dsub_rn(hi_as_double(ar), hi_as_double(ai));
-  auto first = [&](int q, bool im) {
-    const uint32_t sx = (sg >> (im ? q + 1 : q)) << 31, sy = (sg >> (im ? q : q + 1)) << 31;  // signs of ar, ai
-    const double m = sx == sy ? sum : dif;
-    return __hiloint2double((int)((uint32_t)__double2hiint(m) ^ sx), __double2loint(m));
-  };
-  auto t = [&](int q, uint32_t h) { return hi_as_double(h ^ ((sg >> q) << 31)); };
-  auto scaled = [&](double y) -> uint32_t {
-    const uint32_t hi = (uint32_t)__double2hiint(y);
-    if (((hi << 1) | (uint32_t)__double2loint(y)) == 0u) return 0u;
-    spec |= (hi & 0x7ff00000u) == 0x7ff00000u;
-    return (hi + ((uint32_t)L.sk << 20)) & mh;
-  };
-#pragma unroll
-  for (int r = 0; r < 2; ++r) {
-    o[2 * r] = scaled(__dadd_rn(__dadd_rn(first(8 * r, false), t(8 * r + 2, br)), t(8 * r + 3, bi)));
-    o[2 * r + 1] = scaled(__dadd_rn(__dadd_rn(first(8 * r + 4, true), t(8 * r + 6, bi)), t(8 * r + 7, br)));
-  }
-}
-
-// A pair of amplitudes (a, b) held by the same lane, a at in-chunk index i: both outputs in
-// place, truncated.
-template <int ARITH>
-__device__ __forceinline__ void fast_pair(const GateLaunch& L, uint32_t i, uint32_t& ar, uint32_t& ai, uint32_t& br,
-                                          uint32_t& bi, uint32_t mh, bool& spec) {
-  uint32_t o[4] = {ar & mh, ai & mh, br & mh, bi & mh};
-  if ((i & L.lo_mask) == L.lo_vals) {
-    if constexpr (ARITH == 4) {
-      signed_pair(L, ar, ai, br, bi, mh, o, spec);
-    } else if constexpr (ARITH == 0 || ARITH == 3) {
-      const double2 a = make_double2(hi_as_double(ar), hi_as_double(ai)), b = make_double2(hi_as_double(br), hi_as_double(bi));
-      const double2 x = ARITH == 0 ? dense_rows(L.cf, a, b) : real_rows(L.cf, a, b);
-      const double2 y = ARITH == 0 ? dense_rows(L.cf + 8, a, b) : real_rows(L.cf + 8, a, b);
-      o[0] = fast_trunc(x.x, mh, spec);
-      o[1] = fast_trunc(x.y, mh, spec);
-      o[2] = fast_trunc(y.x, mh, spec);
-      o[3] = fast_trunc(y.y, mh, spec);
-    } else {  // anti-diagonal: a' from b, b' from a
-      row_op(L, 0u, br, bi, mh, o[0], o[1], spec);
-      row_op(L, 1u, ar, ai, mh, o[2], o[3], spec);
-    }
-  }
-  ar = o[0];
-  ai = o[1];
-  br = o[2];
-  bi = o[3];
 }
 
 // Shared-memory buffers of one warp (its chunk of the pair's item).

@@ -71,6 +71,32 @@ struct RunJob {
   int ngates;
   int first, ctas;          // its CTAs: [first, first + ctas)
   uint32_t keep;            // page ids a CTA may keep between gates
+  const uint32_t* list;     // not null: the gates are one step, on the chunk pairs k_group listed here (its ndefer)
+};
+
+// A gate inside a step of k_group (the streaming kernels' arithmetic: see GateLaunch).
+struct GroupGate {
+  unsigned long long fixed, hi_vals;  // chunk-index bits its controls fix, and their values
+  unsigned long long pair_bit;        // chunk-index bit of a cross-chunk target, else 0
+  uint32_t lo_mask, lo_vals;
+  int target;
+  int kind;                           // 0 target < 2, 1 target 2..6, 2 target >= 7, 3 diagonal, 4 cross-chunk
+  int arith;
+  int rop[2];
+  uint32_t copy;
+  uint32_t sgn;
+  int sk;
+  double cf[16];
+  double du[4];
+};
+struct GroupLaunch {
+  Pool P;
+  uint32_t S;                         // significant bits of the settled bound (<= 32)
+  int ngates;
+  unsigned long long bit;             // pairs are chunks c and c | bit
+  unsigned long long items;
+  uint32_t* defer;
+  GroupGate g[kRunGroup];
 };
 
 // Records the message sim_last_error() returns on the calling thread.
@@ -101,6 +127,12 @@ cudaError_t launch_gate_fast(const GateLaunch& L, int grid, cudaStream_t st);
 // run_ctas_per_sm * num_sms().
 int run_ctas_per_sm(int kc);
 cudaError_t launch_run(const RunJob* jobs, int njobs, int kc, int grid, cudaStream_t st);
+// Several gates on the chunk pairs of a large state at the settled bound; the pairs it
+// leaves go to launch_run with job.list right after it, which also books the gates.  grid:
+// at most group_ctas_per_sm * num_sms(), and at most the warps wcache has room for.
+int group_ctas_per_sm(int kc);
+int group_warps();
+cudaError_t launch_group(const GroupLaunch& L, int grid, cudaStream_t st);
 // X between chunks: swaps the images of the work items that stand as they are, the others
 // appended to L.defer for launch_gate with L.list = 1 right after it.
 cudaError_t launch_swap(const GateLaunch& L, cudaStream_t st);

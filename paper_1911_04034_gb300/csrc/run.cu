@@ -295,6 +295,7 @@ __device__ __forceinline__ void run_book(const Pool& P, const CtlParams& cp, int
   if (threadIdx.x == 0) {
     ctl->top = (long long)(top + nf);
     ctl->nfreed = 0;
+    ctl->ndefer = 0;
     unsigned long long E = ctl->E, Emax = ctl->Emax, gates = ctl->gates;
     long long n64 = ctl->n64, sw = ctl->switch_gate;
     double lb_sum = ctl->lb_sum, lb_prod = ctl->lb_prod;
@@ -389,11 +390,11 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : QC_RUN_MIN_CTAS)
     const uint32_t S = gate_bits(L);
     // (every CTA reads the same level: it changes only while they meet)
     const bool settled = L.ctl.nlevels == 0 || *(volatile int*)&ctl->level >= L.ctl.nlevels;
-    const int G = settled ? L.group : 1;
-    const bool swap = L.swap != 0;
+    const int G = job.list ? job.ngates : (settled ? L.group : 1);
+    const bool swap = L.swap != 0 && !job.list;
     unsigned long long bit = G > 1 ? L.group_bit : L.pair_bit;
     if (!bit) bit = 1ull;
-    const unsigned long long low = bit - 1ull, items = nchunks > 1ull ? nchunks / 2ull : 1ull;
+    const unsigned long long low = bit - 1ull, items = job.list ? *(volatile unsigned long long*)&ctl->ndefer : (nchunks > 1ull ? nchunks / 2ull : 1ull);
     const unsigned long long swaps = L.items;
     if (swap) {  // X between chunks: a warp per pair, the others by the general way below
       for (unsigned long long item = rank; item < swaps; item += (unsigned)job.ctas) {
@@ -415,7 +416,8 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : QC_RUN_MIN_CTAS)
       }
     } else {
       bool reload = false;
-      for (unsigned long long item = rank; item < items; item += (unsigned)job.ctas) {
+      for (unsigned long long it = rank; it < items; it += (unsigned)job.ctas) {
+        const unsigned long long item = job.list ? job.list[it] : it;
         const unsigned long long c0 = ((item & ~low) << 1) | (item & low);
         if (!run_item<VPT>(P, s_rec, b, job, k, G, c0, c0 | bit, nchunks > 1ull, S, reload, m, st, s_sums)) break;
         reload = G > 2;  // the first record's buffer has held others

@@ -205,3 +205,55 @@ def test_readout_of_many_chunks(eps):
     for seed in range(5):
         outcome, prob = s.measure(seed)
         assert prob == pytest.approx(p[outcome] / p.sum(), rel=1e-10)
+
+
+def group_circuit(n, kc, seed):
+    """Lossy after its first layers, then runs of gates that share a pass over the state:
+    gates of every class inside chunks, diagonal gates and controls anywhere, several gates
+    on one cross-chunk target (a controlled X, RZ and a controlled X among them), image
+    exchanges in between, more gates in a run than a group holds."""
+    rng = np.random.default_rng(seed)
+    g = [Cc.gate(q, Cc.H) for q in range(n)] + [Cc.gate(q, [Cc.SX, Cc.SY, Cc.T][int(rng.integers(3))]) for q in range(n)]
+    some = lambda lo, hi, t, k: {int(q): int(rng.integers(2)) for q in rng.permutation(np.arange(lo, hi))[:k] if q != t}
+    for hi in rng.permutation(np.arange(kc, n))[:3]:
+        hi = int(hi)
+        for _ in range(14):
+            t = int(rng.integers(0, kc))
+            g.append(Cc.gate(t, [Cc.SX, Cc.SY, Cc.rx(0.3), Cc.ry(0.4), Cc.X, Cc.H][int(rng.integers(6))], some(0, n, t, int(rng.integers(3)))))
+            t = int(rng.integers(0, n))
+            g.append(Cc.gate(t, [Cc.T, Cc.Z, Cc.rz(0.7)][int(rng.integers(3))], some(0, n, t, int(rng.integers(3)))))
+        for c in (int(rng.integers(0, kc)), int((hi + 1 - kc) % (n - kc) + kc)):
+            g += [Cc.gate(hi, Cc.X, {c: 1}), Cc.gate(hi, Cc.rz(0.3)), Cc.gate(hi, Cc.X, {c: 1})]
+        g += [Cc.gate(hi, Cc.SY), Cc.gate(3, Cc.SX), Cc.gate(hi, Cc.SX, some(0, kc, hi, 1))]
+    g.append(Cc.gate(0, Cc.ry(2.0 ** -900)))  # a coefficient below 2^-52: subnormal and tiny results
+    g += [Cc.gate(1, Cc.SX), Cc.gate(kc - 1, Cc.SY), Cc.gate(n - 1, Cc.H)]
+    return Cc.to_array(g)
+
+
+@pytest.mark.parametrize("kc,n", [(7, 17), (8, 18), (9, 19), (11, 20)])
+def test_groups_of_gates_on_larger_states(kc, n):
+    """States of more chunk pairs than a whole-circuit launch takes: once the bound is
+    settled, groups of gates per pass (pairs of chunks that leave the STREAM form on the way
+    taken through the same gates by the general path) end in the oracle's images, and in the
+    counters of the same circuit gate by gate: bytes and pages after every gate."""
+    keys = ("gates", "encoded_bytes", "max_encoded_bytes", "eps_switch_gate", "chunks_by_mode", "fidelity_lb_sum", "wide_images",
+            "pages_in_use_bytes", "peak_pages_bytes", "amp_updates", "level", "sig_bits_current")
+    for gates, eps, ladder in ((group_circuit(n, kc, kc), 1e-4, 0), (Cc.grover(n, 1, seed=6)[0][: 3 * n], 1e-3, 1)):
+        sims = []
+        for whole in (True, False):
+            s = qc().Sim(n, n, eps, chunk_log2=kc, budget=(16 << n) // 4, ladder=ladder, pool_bytes=2 * (16 << n) + (64 << 20))
+            if whole:
+                s.apply_circuit(gates[: n + 5])
+                s.apply_circuit(gates[n + 5:])
+            else:
+                for x in gates:
+                    s.apply_gate(x)
+            sims.append(s)
+        a, b = (s.stats() for s in sims)
+        assert {k: a[k] for k in keys} == {k: b[k] for k in keys}
+        assert a["kernel_launches"] < b["kernel_launches"]
+        orc = O.CSim(n, n, kc, eps, (16 << n) // 4, ladder=ladder)
+        orc.apply(gates)
+        want = [orc.image(c) for c in range(orc.nchunks)]
+        assert all_images(sims[0]) == want
+        assert all_images(sims[1]) == want
