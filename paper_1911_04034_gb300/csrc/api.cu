@@ -164,6 +164,7 @@ struct sim {
   qc::RunJob* d_run_jobs = nullptr;
   size_t run_cap = 0;
   int run_grid = 0;                  // its CTAs (0: not used for this state)
+  bool run_wide = false;             // ... two an SM
   int group_grid = 0;                // CTAs of k_group (0: not used for this state)
   int rest_grid = 0;                 // ... and of the k_run launch after it
   int fast_grid = 0;                 // CTAs of the streaming kernel (0: chunk size outside its range)
@@ -371,8 +372,13 @@ sim_status sim_create_ex(int n_qubits, int block_log2, int chunk_log2, double er
   // (2^10-amplitude chunks, 256 items 19 us a gate here; 512 items 36 against 23 by groups
   // and 50 gate by gate).
   {
-    const uint64_t fit = (uint64_t)device_sms() * qc::run_ctas_per_sm(s->kc), items = (s->nchunks + 1) / 2;
-    if (items <= fit) s->run_grid = (int)items;
+    const uint64_t sms = (uint64_t)device_sms(), wide = sms * qc::run_ctas_per_sm(s->kc, true);
+    const uint64_t fit = sms * qc::run_ctas_per_sm(s->kc, false), items = (s->nchunks + 1) / 2;
+    // a lossless run has nothing to settle: its groups share passes at any size (23 qubits,
+    // 11.1 ms a random-circuit layer gate by gate, 7.1 ms by groups)
+    const bool any = cp.nlevels == 0 && s->nchunks <= (1ull << 20);
+    s->run_wide = wide > 0 && (items <= wide || (any && items > fit));
+    if (items <= fit || any) s->run_grid = (int)(s->run_wide ? (items < wide ? items : wide) : (items < fit ? items : fit));
     // larger states: groups of gates (see group_circuit)
     if (!s->run_grid && s->fast_grid && cp.nlevels > 0 && cp.S[cp.nlevels - 1] <= 32) {
       const int resident = device_sms() * qc::group_ctas_per_sm(s->kc), room = s->fast_grid * qc::fast_warps() / qc::group_warps();
@@ -745,7 +751,7 @@ static sim_status run_circuit(sim* s, const sim_gate* gates, size_t n, bool* ran
       s->h_run_jobs[seg] = {s->d_run + off, (int)m, 0, s->run_grid, run_keep(s, s->run_grid), nullptr};
       CK(cudaMemcpyAsync(s->d_run + off, s->h_run + off, m * sizeof(GateLaunch), cudaMemcpyHostToDevice, s->st), "gate records");
       CK(cudaMemcpyAsync(s->d_run_jobs + seg, s->h_run_jobs + seg, sizeof(qc::RunJob), cudaMemcpyHostToDevice, s->st), "gate records");
-      CK(qc::launch_run(s->d_run_jobs + seg, 1, s->kc, s->run_grid, s->st), "circuit kernel launch");
+      CK(qc::launch_run(s->d_run_jobs + seg, 1, s->kc, s->run_grid, s->run_wide, s->st), "circuit kernel launch");
       s->kernel_launches += 1;
       off += m;
     }
@@ -888,7 +894,7 @@ static sim_status group_circuit(sim* s, const sim_gate* gates, size_t n) {
       } else {
         fill_group(s, gates + i + k, s->h_run + k, G);
         CK(qc::launch_group(G, s->group_grid, s->st), "gate group kernel launch");
-        CK(qc::launch_run(s->d_run_jobs + jobs++, 1, s->kc, s->rest_grid, s->st), "circuit kernel launch");
+        CK(qc::launch_run(s->d_run_jobs + jobs++, 1, s->kc, s->rest_grid, false, s->st), "circuit kernel launch");
         s->kernel_launches += 2;
         for (int q = 0; q < len; ++q) s->amp_updates += s->h_run[k + q].nact << s->kc;
       }
@@ -1368,7 +1374,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
     // own and at its own pace.  Otherwise (an option that needs kernels around each gate)
     // step by step: step t holds gate t of every circuit that has one, its jobs' items
     // numbered consecutively.
-    const int resident = device_sms() * qc::run_ctas_per_sm(kc);
+    const int resident = device_sms() * qc::run_ctas_per_sm(kc, false);
     bool whole = count <= resident / 2;
     for (int k = 0; k < count; ++k) whole = whole && run_options(sims[k]) && n_gates[k] < (1u << 20);
     std::vector<qc::BatchJob> jobs;
@@ -1441,7 +1447,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
       if (e == cudaSuccess) e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeRelaxed);
     }
     if (whole && e == cudaSuccess)
-      e = qc::launch_run(reinterpret_cast<const qc::RunJob*>(d_jobs), njobs, kc, run_grid, cs);
+      e = qc::launch_run(reinterpret_cast<const qc::RunJob*>(d_jobs), njobs, kc, run_grid, false, cs);
     for (size_t t = 0; t < steps && !whole && e == cudaSuccess; ++t) {
       const int n = (int)(off[t + 1] - off[t]);
       const int g = (unsigned long long)grid < total[t] ? grid : (int)total[t];

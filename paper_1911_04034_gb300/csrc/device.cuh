@@ -1036,7 +1036,8 @@ __device__ __forceinline__ uint32_t xor_code32(uint32_t v, uint32_t prev) {
 template <int VPT, bool W32>
 __device__ __forceinline__ uint32_t encode_core(uint64_t* tile, int kc, uint32_t S, int force_mode, uint32_t modes,
                                                 uint8_t* img, uint32_t img_cap, ScanSmem& s, int& pp,
-                                                unsigned int* err, const SelCtx* sel, uint64_t t[VPT]) {
+                                                unsigned int* err, const SelCtx* sel, uint64_t t[VPT],
+                                                bool write) {
   const uint32_t N = 2u << kc, A = 1u << kc;
   const uint32_t j0 = threadIdx.x * VPT;
   const bool act = VPT >= 2 || j0 < N;  // every value of a run with VPT >= 2 exists
@@ -1225,6 +1226,10 @@ __device__ __forceinline__ uint32_t encode_core(uint64_t* tile, int kc, uint32_t
     h[2] = nv;
     h[3] = rbits;
   }
+  if (!write) {  // the size and the header were asked for
+    __syncthreads();
+    return best;
+  }
   uint64_t* pay64 = reinterpret_cast<uint64_t*>(img + 16);
   if (mode == M_PALETTE) {
     // the list is in place; each value's index by binary search, packed k bits each
@@ -1283,14 +1288,15 @@ __device__ __forceinline__ uint32_t encode_core(uint64_t* tile, int kc, uint32_t
 // force_mode < 0: smallest image (never larger than RAW).  Returns the image length,
 // or 0 with *err set (non-finite value, or a forced mode that does not apply or does
 // not fit in img_cap).
+// write false: the length, the header and the truncated tile only.
 template <int VPT>
 __device__ uint32_t encode_block(uint64_t* tile, int kc, uint32_t S_req, int force_mode, uint32_t modes, uint8_t* img,
                                  uint32_t img_cap, ScanSmem& s, int& pp, unsigned int* err,
-                                 const SelCtx* sel = nullptr) {
+                                 const SelCtx* sel = nullptr, bool write = true) {
   const uint32_t N = 2u << kc;
   const uint32_t j0 = threadIdx.x * VPT;
   // 0. clear the payload area the packers OR into (the buffer is free here)
-  {
+  if (write) {
     const uint32_t span = min(img_cap, max_coded_bytes(kc)) - 16u;
     uint4* z = reinterpret_cast<uint4*>(img + 16);
     for (uint32_t u = threadIdx.x; u < span / 16u; u += kThreads) z[u] = make_uint4(0u, 0u, 0u, 0u);
@@ -1318,8 +1324,8 @@ __device__ uint32_t encode_block(uint64_t* tile, int kc, uint32_t S_req, int for
     anysub = true;
   }
   const uint32_t S = anysub ? 64u : S_req;
-  if (S <= 32u) return encode_core<VPT, true>(tile, kc, S, force_mode, modes, img, img_cap, s, pp, err, sel, t);
-  return encode_core<VPT, false>(tile, kc, S, force_mode, modes, img, img_cap, s, pp, err, sel, t);
+  if (S <= 32u) return encode_core<VPT, true>(tile, kc, S, force_mode, modes, img, img_cap, s, pp, err, sel, t, write);
+  return encode_core<VPT, false>(tile, kc, S, force_mode, modes, img, img_cap, s, pp, err, sel, t, write);
 }
 
 // Step 3 of encode_core (W32) for one chunk of a pair: the codes of this thread's
@@ -1353,7 +1359,7 @@ template <int VPT>
 __device__ __forceinline__ uint32_t finish32_pair_part(const uint64_t* tile, int kc, uint32_t S, uint32_t modes,
                                                        uint8_t* img, uint32_t img_cap, ScanSmem& s, unsigned int* err,
                                                        const uint32_t h[VPT], uint32_t cc, uint32_t o0, uint32_t total,
-                                                       bool allzero, bool allconst, bool gtop) {
+                                                       bool allzero, bool allconst, bool gtop, bool write) {
   const uint32_t N = 2u << kc, A = 1u << kc;
   const uint32_t j0 = threadIdx.x * VPT;
   const ulonglong2* t2 = reinterpret_cast<const ulonglong2*>(tile);
@@ -1421,6 +1427,7 @@ __device__ __forceinline__ uint32_t finish32_pair_part(const uint64_t* tile, int
     hd[2] = nv;
     hd[3] = rbits;
   }
+  if (!write) return best;
   uint64_t* pay64 = reinterpret_cast<uint64_t*>(img + 16);
   if (mode == M_CONST) {
     if (threadIdx.x == 0) {
@@ -1452,11 +1459,11 @@ __device__ __forceinline__ uint32_t finish32_pair_part(const uint64_t* tile, int
 template <int VPT>
 __device__ bool encode_pair32(uint64_t* tile0, uint64_t* tile1, int kc, uint32_t S, uint32_t modes, uint8_t* img0,
                               uint8_t* img1, uint32_t img_cap, ScanSmem& s, int& pp, unsigned int* err, uint32_t& n0,
-                              uint32_t& n1) {
+                              uint32_t& n1, bool write = true) {
   const uint32_t N = 2u << kc;
   const uint32_t j0 = threadIdx.x * VPT;
   // 0. clear both payload areas the packers OR into
-  {
+  if (write) {
     const uint32_t span = (min(img_cap, max_coded_bytes(kc)) - 16u) / 16u;
     uint4* z0 = reinterpret_cast<uint4*>(img0 + 16);
     uint4* z1 = reinterpret_cast<uint4*>(img1 + 16);
@@ -1515,9 +1522,9 @@ __device__ bool encode_pair32(uint64_t* tile0, uint64_t* tile1, int kc, uint32_t
               &total1, &f_or, &f_and);
   // 4-6. period, choice and image of each chunk
   n0 = finish32_pair_part<VPT>(tile0, kc, S, modes, img0, img_cap, s, err, h0, cc0, o0, total0, (f_or & 1u) == 0u,
-                               (f_and & 1u) != 0u, (f_and & 2u) != 0u);
+                               (f_and & 1u) != 0u, (f_and & 2u) != 0u, write);
   n1 = finish32_pair_part<VPT>(tile1, kc, S, modes, img1, img_cap, s, err, h1, cc1, o1, total1, (f_or & 2u) == 0u,
-                               (f_and & 4u) != 0u, (f_and & 8u) != 0u);
+                               (f_and & 4u) != 0u, (f_and & 8u) != 0u, write);
   __syncthreads();
   return true;
 }

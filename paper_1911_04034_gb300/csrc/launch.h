@@ -124,9 +124,12 @@ int fast_warp_cache();   // page ids each of its warps may hold
 cudaError_t launch_gate_fast(const GateLaunch& L, int grid, cudaStream_t st);
 // Whole circuits in one launch: every simulator's gates in order by the general kernel's
 // items, its CTAs meeting after each gate.  All CTAs must be resident at once: at most
-// run_ctas_per_sm * num_sms().
-int run_ctas_per_sm(int kc);
-cudaError_t launch_run(const RunJob* jobs, int njobs, int kc, int grid, cudaStream_t st);
+// run_ctas_per_sm * num_sms().  wide: the form with two CTAs an SM (0 a SM: not for this
+// chunk size).
+int run_ctas_per_sm(int kc, bool wide);
+cudaError_t launch_run(const RunJob* jobs, int njobs, int kc, int grid, bool wide, cudaStream_t st);
+int run_wide_ctas_per_sm(int kc);
+cudaError_t launch_run_wide(const RunJob* jobs, int njobs, int kc, int grid, cudaStream_t st);
 // Several gates on the chunk pairs of a large state at the settled bound; the pairs it
 // leaves go to launch_run with job.list right after it, which also books the gates.  grid:
 // at most group_ctas_per_sm * num_sms(), and at most the warps wcache has room for.

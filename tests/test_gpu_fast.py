@@ -6,7 +6,7 @@ first; items it cannot finish as STREAM images go to the general kernel.  Both m
 the oracle's bytes.  The circuits cover every work-item kind of the streaming kernel:
 cross-chunk targets, in-chunk targets 0-1 (partner in the lane), 2-6 (partner in another
 lane of the warp), diagonal gates on any in-chunk target, in-chunk controls, and targets
-7..kc-1 (general kernel only).
+7..kc-1 (partner in another pass).
 """
 import numpy as np
 import pytest
@@ -232,16 +232,18 @@ def group_circuit(n, kc, seed):
 
 @pytest.mark.parametrize("kc,n", [(7, 17), (8, 18), (9, 19), (11, 20)])
 def test_groups_of_gates_on_larger_states(kc, n):
-    """States of more chunk pairs than a whole-circuit launch takes: once the bound is
-    settled, groups of gates per pass (pairs of chunks that leave the STREAM form on the way
+    """States of more chunk pairs than one round of a whole-circuit launch (lossless ones run
+    by it all the same): once the bound is settled, groups of gates per pass (pairs of chunks that leave the STREAM form on the way
     taken through the same gates by the general path) end in the oracle's images, and in the
     counters of the same circuit gate by gate: bytes and pages after every gate."""
     keys = ("gates", "encoded_bytes", "max_encoded_bytes", "eps_switch_gate", "chunks_by_mode", "fidelity_lb_sum", "wide_images",
             "pages_in_use_bytes", "peak_pages_bytes", "amp_updates", "level", "sig_bits_current")
-    for gates, eps, ladder in ((group_circuit(n, kc, kc), 1e-4, 0), (Cc.grover(n, 1, seed=6)[0][: 3 * n], 1e-3, 1)):
+    for gates, eps, ladder in ((group_circuit(n, kc, kc), 1e-4, 0), (Cc.grover(n, 1, seed=6)[0][: 3 * n], 1e-3, 1),
+                               (group_circuit(n, kc, n)[: 120], 0.0, 0)):
         sims = []
+        budget = (16 << n) // 4 if eps else 2 * (16 << n)
         for whole in (True, False):
-            s = qc().Sim(n, n, eps, chunk_log2=kc, budget=(16 << n) // 4, ladder=ladder, pool_bytes=2 * (16 << n) + (64 << 20))
+            s = qc().Sim(n, n, eps, chunk_log2=kc, budget=budget, ladder=ladder, pool_bytes=2 * (16 << n) + (64 << 20))
             if whole:
                 s.apply_circuit(gates[: n + 5])
                 s.apply_circuit(gates[n + 5:])
@@ -252,7 +254,7 @@ def test_groups_of_gates_on_larger_states(kc, n):
         a, b = (s.stats() for s in sims)
         assert {k: a[k] for k in keys} == {k: b[k] for k in keys}
         assert a["kernel_launches"] < b["kernel_launches"]
-        orc = O.CSim(n, n, kc, eps, (16 << n) // 4, ladder=ladder)
+        orc = O.CSim(n, n, kc, eps, budget, ladder=ladder)
         orc.apply(gates)
         want = [orc.image(c) for c in range(orc.nchunks)]
         assert all_images(sims[0]) == want
