@@ -604,7 +604,8 @@ static bool fast_applies(const sim* s, const sim_gate* g, GateLaunch& L) {
                          u[4], -u[5], u[6], -u[7], u[4], u[5], u[6], u[7]};
   for (int k = 0; k < 16; ++k) L.cf[k] = cf[k];
   const bool real = u[1] == 0.0 && u[3] == 0.0 && u[5] == 0.0 && u[7] == 0.0;
-  L.arith = diag ? 1 : (anti ? 2 : (real ? 3 : 0));
+  const bool rx = u[1] == 0.0 && u[2] == 0.0 && u[4] == 0.0 && u[7] == 0.0;
+  L.arith = diag ? 1 : (anti ? 2 : (real ? 3 : (rx ? 5 : 0)));
   if (L.arith == 0) {
     // every coefficient part of the same magnitude 2^k, none zero: exact products
     const double c = std::fabs(cf[0]);

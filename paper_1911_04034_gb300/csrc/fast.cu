@@ -294,13 +294,13 @@ __device__ __forceinline__ int fast_item(const GateLaunch& L, unsigned long long
             const uint32_t ar = row ? w[2 * k] : v[2 * k], ai = row ? w[2 * k + 1] : v[2 * k + 1];
             const uint32_t br = row ? v[2 * k] : w[2 * k], bi = row ? v[2 * k + 1] : w[2 * k + 1];
             signed_rows(L, row, ar, ai, br, bi, mh, outr, outi, spec);
-          } else if constexpr (ARITH == 0 || ARITH == 3) {
+          } else if constexpr (ARITH == 0 || ARITH == 3 || ARITH == 5) {
             // a = the pair's first amplitude, b = its second
             const uint32_t ar = row ? w[2 * k] : v[2 * k], ai = row ? w[2 * k + 1] : v[2 * k + 1];
             const uint32_t br = row ? v[2 * k] : w[2 * k], bi = row ? v[2 * k + 1] : w[2 * k + 1];
             const double2 a = make_double2(hi_as_double(ar), hi_as_double(ai));
             const double2 b = make_double2(hi_as_double(br), hi_as_double(bi));
-            const double2 out = ARITH == 0 ? dense_rows(L.cf + 8u * row, a, b) : real_rows(L.cf + 8u * row, a, b);
+            const double2 out = form_rows<ARITH>(L.cf, row, a, b);
             outr = fast_trunc(out.x, mh, spec);
             outi = fast_trunc(out.y, mh, spec);
           } else if constexpr (ARITH == 1) {
@@ -519,7 +519,7 @@ static cudaError_t launch_fast_as(const GateLaunch& L, int grid, size_t smem, cu
 }
 
 // Kinds and arithmetic forms that occur: cross-chunk pairs of any gate class, in-chunk
-// partners of dense, real, power-of-two or anti-diagonal gates, in-chunk diagonal gates,
+// partners of dense, real, RX-like, power-of-two or anti-diagonal gates, in-chunk diagonal gates,
 // cross-chunk diagonal gates with a row that is an exact copy.
 cudaError_t launch_gate_fast(const GateLaunch& L, int grid, cudaStream_t st) {
   const uint32_t held = fast_held(L.fast_kind, L.target);
@@ -532,19 +532,23 @@ cudaError_t launch_gate_fast(const GateLaunch& L, int grid, cudaStream_t st) {
     case 2: return launch_fast_as<0, 2>(L, grid, smem, st);
     case 3: return launch_fast_as<0, 3>(L, grid, smem, st);
     case 4: return launch_fast_as<0, 4>(L, grid, smem, st);
+    case 5: return launch_fast_as<0, 5>(L, grid, smem, st);
     case 8: return launch_fast_as<1, 0>(L, grid, smem, st);
     case 10: return launch_fast_as<1, 2>(L, grid, smem, st);
     case 11: return launch_fast_as<1, 3>(L, grid, smem, st);
     case 12: return launch_fast_as<1, 4>(L, grid, smem, st);
+    case 13: return launch_fast_as<1, 5>(L, grid, smem, st);
     case 16: return launch_fast_as<2, 0>(L, grid, smem, st);
     case 18: return launch_fast_as<2, 2>(L, grid, smem, st);
     case 19: return launch_fast_as<2, 3>(L, grid, smem, st);
     case 20: return launch_fast_as<2, 4>(L, grid, smem, st);
+    case 21: return launch_fast_as<2, 5>(L, grid, smem, st);
     case 25: return launch_fast_as<3, 1>(L, grid, smem, st);
     case 32: return launch_fast_as<4, 0>(L, grid, smem, st);
     case 34: return launch_fast_as<4, 2>(L, grid, smem, st);
     case 35: return launch_fast_as<4, 3>(L, grid, smem, st);
     case 36: return launch_fast_as<4, 4>(L, grid, smem, st);
+    case 37: return launch_fast_as<4, 5>(L, grid, smem, st);
     case 41: return launch_fast_as<5, 1>(L, grid, smem, st);
     default: return cudaErrorInvalidValue;
   }

@@ -20,168 +20,163 @@ namespace qc {
 constexpr int kGroupWarps = 4;  // two pairs; 20 warps an SM with 2^10-amplitude chunks (43 KB a CTA)
 constexpr int kGroupPairs = kGroupWarps / 2;
 
-// Per warp: its chunk's high words, two windows (the first also the output window), input
-// and output page ids, its page cache.
+// Per warp: its chunk's high words, what is known of each pass of it (see group_note), two
+// windows (the first also the output window), input and output page ids, its page cache.
+constexpr uint32_t kGroupPasses = 16;  // of a chunk, at most
 __host__ __device__ __forceinline__ uint32_t group_warp_bytes(int kc) {
-  return 4u * (2u << kc) + 2u * kFastWin + 8u * fast_pg_words(kc) + 4u * kWarpCache + 16u;
+  return 4u * (2u << kc) + 4u * kGroupPasses + 2u * kFastWin + 8u * fast_pg_words(kc) + 4u * kWarpCache + 16u;
 }
 
-// The lane's 8 values of pass p: two 16-byte units 512 bytes apart (no bank conflicts).
-__device__ __forceinline__ void vals_load(const uint32_t* vals, uint32_t p, uint32_t v[8]) {
-  const uint4* q = reinterpret_cast<const uint4*>(vals) + 64u * p + (threadIdx.x & 31u);
-  const uint4 a = q[0], b = q[32];
-  v[0] = a.x; v[1] = a.y; v[2] = a.z; v[3] = a.w; v[4] = b.x; v[5] = b.y; v[6] = b.z; v[7] = b.w;
+// A chunk's values stand in order; a lane takes amplitude 32 j + lane of a pass (128
+// amplitudes), so that one loop body serves every target and an instruction cache holds the
+// whole kernel (unrolled over a lane's 8 consecutive values, with a body per kind of target,
+// it was 228 KB and waited for instructions more than for anything else).
+__device__ __forceinline__ uint2* amps(uint32_t* vals, uint32_t p) { return reinterpret_cast<uint2*>(vals) + 128u * p; }
+__device__ __forceinline__ const uint2* amps(const uint32_t* vals, uint32_t p) {
+  return reinterpret_cast<const uint2*>(vals) + 128u * p;
 }
-__device__ __forceinline__ void vals_store(uint32_t* vals, uint32_t p, const uint32_t v[8]) {
-  uint4* q = reinterpret_cast<uint4*>(vals) + 64u * p + (threadIdx.x & 31u);
-  q[0] = make_uint4(v[0], v[1], v[2], v[3]);
-  q[32] = make_uint4(v[4], v[5], v[6], v[7]);
-}
-// Word of value 0 and of value 5 of a lane's pass (the period filter's samples).
-__device__ __forceinline__ const uint32_t* val0(const uint32_t* vals, uint32_t p) {
-  return vals + 256u * p + 4u * (threadIdx.x & 31u);
-}
-__device__ __forceinline__ const uint32_t* val5(const uint32_t* vals, uint32_t p) {
-  return vals + 256u * p + 128u + 4u * (threadIdx.x & 31u) + 1u;
+__device__ __forceinline__ uint32_t code_bits(uint32_t x, uint32_t S) { return rest_bits(code_rest(x), S); }
+
+// The passes of a chunk whose index bits satisfy a gate's controls (bit p), for a diagonal
+// gate on an in-chunk target those not on an exact copy's row: the others stay.
+__device__ __forceinline__ uint32_t group_passes(const GroupGate& g, uint32_t NP) {
+  const uint32_t hm = g.lo_mask >> 7, hv = g.lo_vals >> 7, lane = threadIdx.x & 31u;
+  bool on = lane < NP && (lane & hm) == hv;
+  if (g.kind == 3 && !g.pair_bit && g.target >= 7) on = on && !((g.copy >> ((lane >> (g.target - 7)) & 1u)) & 1u);
+  return __ballot_sync(0xffffffffu, on);
 }
 
-// signed_rows / signed_pair need every input at least 2^-959 or zero.
+// Notes what the byte count needs to know of the passes in `mask`: the residual bits of all
+// but a pass's first value (whose predecessor lies in the pass before), and in the top bit
+// whether some lane's amplitudes differ (the chunk is then neither constant nor zero).
+// Passes a gate leaves keep their notes.
+__device__ __forceinline__ void group_note(const uint32_t* vals, uint32_t* notes, uint32_t mask, uint32_t S) {
+  const uint32_t lane = threadIdx.x & 31u;
+#pragma unroll 1
+  while (mask) {
+    const uint32_t p = (uint32_t)__ffs((int)mask) - 1u;
+    mask &= mask - 1u;
+    const uint2* a = amps(vals, p) + lane;
+    uint2 v[4];
+#pragma unroll
+    for (int j = 0; j < 4; ++j) v[j] = a[32 * j];
+    uint32_t sum = 0u, carry = 0u, varies = 0u;
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      uint32_t before = __shfl_up_sync(0xffffffffu, v[j].y, 1);
+      if (lane == 0) before = carry;
+      carry = __shfl_sync(0xffffffffu, v[j].y, 31);
+      if (j > 0 || lane > 0) sum += code_bits(v[j].x ^ before, S);
+      sum += code_bits(v[j].y ^ v[j].x, S);
+      varies |= (v[j].x ^ v[0].x) | (v[j].y ^ v[0].y);
+    }
+    const uint32_t bits = __reduce_add_sync(0xffffffffu, sum);
+    const bool any = __any_sync(0xffffffffu, varies != 0u);
+    if (lane == 0) notes[p] = bits | (any ? 0x80000000u : 0u);
+  }
+  __syncwarp();
+}
+
+// signed_pair needs every input at least 2^-959 or zero.
 __device__ __forceinline__ bool too_small(uint32_t h) { return ((h & 0x7fffffffu) - 1u) < ((64u << 20) - 1u); }
 
-// A gate that is not diagonal on this warp's chunk; kind 4 (the pair's chunks a and b): this
-// warp's half of the amplitudes, both rows.
+// The pairs of one pass (in-chunk target below 7: A = B, 64 pairs) or of two (A and B hold the
+// pairs' first and second amplitudes, 128 pairs); i0: in-chunk index of A's first amplitude.
+template <int ARITH>
+__device__ __forceinline__ void group_pairs(const GroupGate& g, uint2* A, uint2* B, uint32_t i0, bool inner, uint32_t mh,
+                                            bool& spec) {
+  const uint32_t lane = threadIdx.x & 31u, tb = inner ? 1u << g.target : 0u, low = tb - 1u;
+#pragma unroll 1
+  for (uint32_t q = lane; q < (inner ? 64u : 128u); q += 32u) {
+    const uint32_t ia = inner ? ((q & ~low) << 1) | (q & low) : q, ib = ia | tb;
+    if (((i0 + ia) & g.lo_mask) != g.lo_vals) continue;
+    uint2 a = A[ia], b = B[ib];
+    if constexpr (ARITH == 4) spec |= too_small(a.x) | too_small(a.y) | too_small(b.x) | too_small(b.y);
+    fast_pair<ARITH>(g, i0 + ia, a.x, a.y, b.x, b.y, mh, spec);
+    A[ia] = a;
+    B[ib] = b;
+  }
+}
+// A gate that is not diagonal on the passes `mask` of this warp's chunk; a cross-chunk gate
+// (chunks ca and cb): this warp's half of them, both rows.
 template <int ARITH>
 __device__ __forceinline__ void group_apply(const GroupGate& g, uint32_t* mine, uint32_t* ca, uint32_t* cb, uint32_t side,
-                                            uint32_t NP, uint32_t mh, bool& spec) {
-  const uint32_t lane = threadIdx.x & 31u;
-  auto pair_of = [&](uint32_t* a, uint32_t pa, uint32_t* b, uint32_t pb) {
-    uint32_t x[8], y[8];
-    vals_load(a, pa, x);
-    vals_load(b, pb, y);
-    if constexpr (ARITH == 4) {
-#pragma unroll
-      for (int k = 0; k < 8; ++k) spec |= too_small(x[k]) | too_small(y[k]);
-    }
-#pragma unroll
-    for (int k = 0; k < 4; ++k)
-      fast_pair<ARITH>(g, 128u * pa + 4u * lane + (uint32_t)k, x[2 * k], x[2 * k + 1], y[2 * k], y[2 * k + 1], mh, spec);
-    vals_store(a, pa, x);
-    vals_store(b, pb, y);
-  };
+                                            uint32_t NP, uint32_t mask, uint32_t mh, bool& spec) {
+  const bool inner = g.kind < 2;
+  uint32_t todo = mask, d = 0u;
   if (g.kind == 4) {
-    const uint32_t lo = NP > 1u ? side * (NP / 2u) : side, hi = NP > 1u ? lo + NP / 2u : 1u;
-    for (uint32_t p = lo; p < hi; ++p) pair_of(ca, p, cb, p);
+    const uint32_t half = NP > 1u ? (1u << (NP / 2u)) - 1u : 1u;
+    todo &= side ? ~half : half;
   } else if (g.kind == 2) {
-    const uint32_t d = 1u << (g.target - 7);
-    for (uint32_t q = 0; q < NP / 2u; ++q) {
-      const uint32_t p = ((q & ~(d - 1u)) << 1) | (q & (d - 1u));
-      pair_of(mine, p, mine, p + d);
-    }
-  } else {
-    for (uint32_t p = 0; p < NP; ++p) {
-      uint32_t v[8];
-      vals_load(mine, p, v);
-      if constexpr (ARITH == 4) {
-#pragma unroll
-        for (int k = 0; k < 8; ++k) spec |= too_small(v[k]);
-      }
-      const uint32_t i = 128u * p + 4u * lane;
-      if (g.kind == 0) {
-        if (g.target == 0) {
-          fast_pair<ARITH>(g, i, v[0], v[1], v[2], v[3], mh, spec);
-          fast_pair<ARITH>(g, i + 2u, v[4], v[5], v[6], v[7], mh, spec);
-        } else {
-          fast_pair<ARITH>(g, i, v[0], v[1], v[4], v[5], mh, spec);
-          fast_pair<ARITH>(g, i + 1u, v[2], v[3], v[6], v[7], mh, spec);
-        }
-      } else {  // partner in lane ^ 2^(t-2): this lane forms its own row
-        const uint32_t row = (lane >> (g.target - 2)) & 1u;
-        uint32_t w[8];
-#pragma unroll
-        for (int k = 0; k < 8; ++k) w[k] = __shfl_xor_sync(0xffffffffu, v[k], 1u << (g.target - 2));
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          uint32_t outr = v[2 * k], outi = v[2 * k + 1];
-          if ((((i + (uint32_t)k) & ~(1u << g.target)) & g.lo_mask) == g.lo_vals) {
-            const uint32_t ar = row ? w[2 * k] : v[2 * k], ai = row ? w[2 * k + 1] : v[2 * k + 1];
-            const uint32_t br = row ? v[2 * k] : w[2 * k], bi = row ? v[2 * k + 1] : w[2 * k + 1];
-            if constexpr (ARITH == 4) {
-              signed_rows(g, row, ar, ai, br, bi, mh, outr, outi, spec);
-            } else if constexpr (ARITH == 2) {
-              row_op(g, row, w[2 * k], w[2 * k + 1], mh, outr, outi, spec);
-            } else {
-              const double2 a = make_double2(hi_as_double(ar), hi_as_double(ai));
-              const double2 b = make_double2(hi_as_double(br), hi_as_double(bi));
-              const double2 o = ARITH == 0 ? dense_rows(g.cf + 8u * row, a, b) : real_rows(g.cf + 8u * row, a, b);
-              outr = fast_trunc(o.x, mh, spec);
-              outi = fast_trunc(o.y, mh, spec);
-            }
-          }
-          v[2 * k] = outr;
-          v[2 * k + 1] = outi;
-        }
-      }
-      vals_store(mine, p, v);
-    }
+    d = 1u << (g.target - 7);
+  }
+#pragma unroll 1
+  while (todo) {
+    const uint32_t p = (uint32_t)__ffs((int)todo) - 1u;
+    todo &= todo - 1u;
+    if (p & d) continue;  // the second pass of a pair of passes
+    group_pairs<ARITH>(g, amps(g.kind == 4 ? ca : mine, p), amps(g.kind == 4 ? cb : mine, p + d), 128u * p, inner, mh, spec);
   }
 }
 
-// A diagonal gate on this warp's chunk: row by the chunk (pair_bit) or by the amplitude.
-__device__ __forceinline__ void group_diag(const GroupGate& g, uint32_t* mine, uint32_t chunk_row, uint32_t NP, uint32_t mh,
+// A diagonal gate on the passes `mask` of this warp's chunk: row by the chunk (a cross-chunk
+// target) or by the amplitude.
+__device__ __forceinline__ void group_diag(const GroupGate& g, uint32_t* mine, uint32_t chunk_row, uint32_t mask, uint32_t mh,
                                            bool& spec) {
-  const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t tb = g.pair_bit ? 0u : 1u << g.target;
-  for (uint32_t p = 0; p < NP; ++p) {
-    const uint32_t i = 128u * p + 4u * lane;
-    // a pass whose index bits miss the controls, or whose row is a copy, stays
-    if (((128u * p) & g.lo_mask & ~127u) != (g.lo_vals & ~127u)) continue;
-    if (tb >= 128u && ((g.copy >> ((128u * p & tb) ? 1u : 0u)) & 1u)) continue;
-    uint32_t v[8];
-    vals_load(mine, p, v);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) {
-      const uint32_t a = i + (uint32_t)k, row = tb ? ((a & tb) ? 1u : 0u) : chunk_row;
-      if (((a & ~tb) & g.lo_mask) == g.lo_vals) {
-        uint32_t x, y;
-        row_op(g, row, v[2 * k], v[2 * k + 1], mh, x, y, spec);
-        v[2 * k] = x;
-        v[2 * k + 1] = y;
-      }
+  const uint32_t lane = threadIdx.x & 31u, tb = g.pair_bit ? 0u : 1u << g.target;
+#pragma unroll 1
+  while (mask) {
+    const uint32_t p = (uint32_t)__ffs((int)mask) - 1u;
+    mask &= mask - 1u;
+    uint2* a = amps(mine, p);
+#pragma unroll 1
+    for (uint32_t q = lane; q < 128u; q += 32u) {
+      const uint32_t i = 128u * p + q, row = tb ? ((i & tb) ? 1u : 0u) : chunk_row;
+      if (((i & ~tb) & g.lo_mask) != g.lo_vals || ((g.copy >> row) & 1u)) continue;
+      uint2 v = a[q], o;
+      row_op(g, row, v.x, v.y, mh, o.x, o.y, spec);
+      a[q] = o;
     }
-    vals_store(mine, p, v);
   }
 }
 
-// Residual bits of the chunk's values, and whether its image is surely STREAM (fast_item's
-// filters: not constant, not zero, no period).  All lanes get both.
-__device__ __forceinline__ bool group_size(const uint32_t* vals, uint32_t NP, uint32_t S, uint32_t& bits) {
+// Whether some amplitude of the chunk differs from its first (a chunk of zeros: no), and
+// whether some amplitude differs from the one half a chunk on (a period: none does).
+__device__ __forceinline__ bool group_differs(const uint32_t* vals, uint32_t NP) {
   const uint32_t lane = threadIdx.x & 31u;
-  const uint32_t refr = vals[0], refi = vals[1];
-  uint32_t sum = 0u, prv = 0u, nzor = 0u;
-  bool cst = true, halves = true;
-  for (uint32_t p = 0; p < NP; ++p) {
-    uint32_t v[8];
-    vals_load(vals, p, v);
-    uint32_t pr = __shfl_up_sync(0xffffffffu, v[7], 1);
-    if (lane == 0) pr = prv;
-    prv = __shfl_sync(0xffffffffu, v[7], 31);
-#pragma unroll
-    for (int k = 0; k < 8; ++k) {
-      const uint32_t x = v[k] ^ (k ? v[k - 1] : pr);
-      sum += rlen(S, min((uint32_t)__clz((int)x), 24u) & 0x18u);
-      nzor |= v[k];
-      cst &= v[k] == ((k & 1) ? refi : refr);
-    }
-    if (NP == 1u) {
-      const uint32_t a = __shfl_xor_sync(0xffffffffu, v[0], 16), b = __shfl_xor_sync(0xffffffffu, v[5], 16);
-      halves &= (a == v[0]) & (b == v[5]);
-    } else if (p >= NP / 2u) {
-      halves &= *val0(vals, p - NP / 2u) == v[0] && *val5(vals, p - NP / 2u) == v[5];
-    }
+  bool any = false;
+#pragma unroll 1
+  for (uint32_t q = 0; q < 4u * NP && !any; ++q) {
+    const uint2 v = amps(vals, 0u)[32u * q + lane];
+    any = __any_sync(0xffffffffu, v.x != vals[0] || v.y != vals[1]);
   }
-  bits = __reduce_add_sync(0xffffffffu, sum);
-  const bool c = __all_sync(0xffffffffu, cst), z = __any_sync(0xffffffffu, nzor != 0u), h = __all_sync(0xffffffffu, halves);
-  return !c && z && !h;
+  return any;
+}
+__device__ __forceinline__ bool group_moves(const uint32_t* vals, uint32_t NP) {
+  const uint32_t lane = threadIdx.x & 31u;
+  bool any = false;
+#pragma unroll 1
+  for (uint32_t q = 0; q < 2u * NP && !any; ++q) {
+    const uint2 v = amps(vals, 0u)[32u * q + lane], w = amps(vals, 0u)[32u * (q + 2u * NP) + lane];
+    any = __any_sync(0xffffffffu, v.x != w.x || v.y != w.y);
+  }
+  return any;
+}
+
+// Residual bits of the chunk's values from its notes, and whether its image is surely STREAM
+// (fast_item's filters: not constant, not zero, no period).  All lanes get both.
+__device__ __forceinline__ bool group_size(const uint32_t* vals, const uint32_t* notes, uint32_t NP, uint32_t S,
+                                           uint32_t& bits) {
+  const uint32_t lane = threadIdx.x & 31u;
+  uint32_t mine = 0u, varies = 0u;
+  if (lane < NP) {
+    const uint32_t x = vals[256u * lane] ^ (lane ? vals[256u * lane - 1u] : 0u);  // a pass's first value and the one before
+    mine = (notes[lane] & 0x7fffffffu) + code_bits(x, S);
+    varies = notes[lane] >> 31;
+  }
+  bits = __reduce_add_sync(0xffffffffu, mine);
+  // (lanes that vary: not constant, not zero)
+  return (__any_sync(0xffffffffu, varies != 0u) || group_differs(vals, NP)) && group_moves(vals, NP);
 }
 
 __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_constant__ GroupLaunch L) {
@@ -198,7 +193,8 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
   const uint32_t per = group_warp_bytes(kc);
   uint32_t* const vals = reinterpret_cast<uint32_t*>(smem + (size_t)wid * per);
   uint32_t* const peer = reinterpret_cast<uint32_t*>(smem + (size_t)(wid ^ 1u) * per);
-  uint32_t* const win0 = vals + N;
+  uint32_t* const notes = vals + N;
+  uint32_t* const win0 = notes + kGroupPasses;
   uint32_t* const win1 = win0 + kFastWin / 4u;
   uint32_t* const ipg = win1 + kFastWin / 4u;
   uint32_t* const opg = ipg + fast_pg_words(kc);
@@ -207,6 +203,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
   wp.n = wp.ids + kWarpCache;
   const size_t gw = (size_t)blockIdx.x * kGroupWarps + wid;
   const uint32_t n_start = P.wcache_n[gw];
+#pragma unroll 1
   for (uint32_t q = lane; q < n_start; q += 32u) wp.ids[q] = P.wcache[gw * kWarpCache + q];
   if (lane == 0) *wp.n = n_start;
   __syncwarp();
@@ -221,6 +218,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
     // the gates that rewrite this chunk (bit g), and whether one leaves it by a copy row
     uint32_t mine = 0u;
     bool copied = false;
+#pragma unroll 1
     for (int g = 0; g < L.ngates; ++g) {
       const GroupGate& q = L.g[g];
       if ((ch & q.fixed) != q.hi_vals) continue;
@@ -237,6 +235,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
       ok = inp >= 1u && ib <= fast_max_image(kc) && inp == (ib + kPage - 1u) / kPage;
       if (ok) {
         bool good = true;
+#pragma unroll 1
         for (uint32_t k = lane; k < inp; k += 32u) {
           const uint32_t pid = e[4 + k];
           ipg[k] = pid;
@@ -271,10 +270,16 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
     bool corrupt = false, lost = false, keep = true, spec = false;
     if (mine)
       corrupt = !stream_decode(PagedImage{P.pages, ipg}, kc, S, bits_in, ib, win0, win1,
-                               [&](uint32_t p, const uint32_t v[8]) { vals_store(vals, p, v); });
+                               [&](uint32_t p, const uint32_t v[8], uint32_t, uint32_t) {
+                                 uint4* q = reinterpret_cast<uint4*>(vals + 256u * p) + 2u * lane;
+                                 q[0] = make_uint4(v[0], v[1], v[2], v[3]);
+                                 q[1] = make_uint4(v[4], v[5], v[6], v[7]);
+                               });
     __syncwarp();
     uint32_t size = ib;  // lane g: the image's bytes after gate g
     const int last = mine ? 31 - __clz((int)mine) : -1;
+    // the byte count after a gate in the middle needs a note of every pass
+    if (mine & (mine - 1u)) group_note(vals, notes, (1u << NP) - 1u, S);
     for (int g = 0; g <= last; ++g) {
       if (!((mine >> g) & 1u)) continue;
       const GroupGate& q = L.g[g];
@@ -283,16 +288,18 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
         ++phase;
         if (!lost) lost = !pair_sync(seq, side, phase, ctl, 6u);
       }
+      const uint32_t passes = group_passes(q, NP);
       if (q.kind == 3) {
-        group_diag(q, vals, (ch & q.pair_bit) ? 1u : 0u, NP, mh, spec);
+        group_diag(q, vals, (ch & q.pair_bit) ? 1u : 0u, passes, mh, spec);
       } else {
         uint32_t* const ca = side ? peer : vals;
         uint32_t* const cbv = side ? vals : peer;
         switch (q.arith) {
-          case 0: group_apply<0>(q, vals, ca, cbv, side, NP, mh, spec); break;
-          case 2: group_apply<2>(q, vals, ca, cbv, side, NP, mh, spec); break;
-          case 3: group_apply<3>(q, vals, ca, cbv, side, NP, mh, spec); break;
-          default: group_apply<4>(q, vals, ca, cbv, side, NP, mh, spec); break;
+          case 0: group_apply<0>(q, vals, ca, cbv, side, NP, passes, mh, spec); break;
+          case 2: group_apply<2>(q, vals, ca, cbv, side, NP, passes, mh, spec); break;
+          case 3: group_apply<3>(q, vals, ca, cbv, side, NP, passes, mh, spec); break;
+          case 5: group_apply<5>(q, vals, ca, cbv, side, NP, passes, mh, spec); break;
+          default: group_apply<4>(q, vals, ca, cbv, side, NP, passes, mh, spec); break;
         }
       }
       if (cross) {
@@ -302,7 +309,8 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
       __syncwarp();
       if (g < last) {  // the last one's bytes come from the encoder
         uint32_t bits;
-        keep &= group_size(vals, NP, S, bits);
+        group_note(vals, notes, passes, S);
+        keep &= group_size(vals, notes, NP, S, bits);
         if ((int)lane >= g) size = 16u + cb + resid_bytes(bits);
       }
     }
@@ -312,29 +320,19 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
     if (mine) {
       uint32_t* const owin = win0;
       uint4* const w4 = reinterpret_cast<uint4*>(owin);
+#pragma unroll 1
       for (uint32_t k = lane; k < kWinBlocks; k += 32u) w4[k] = make_uint4(0u, 0u, 0u, 0u);
       oom = !wp_grow(P, wp, opg, onp, (16u + cb + kPage - 1u) / kPage);
       __syncwarp();
-      const uint32_t refr = vals[0], refi = vals[1];
-      uint32_t prv = 0u, nzor = 0u;
-      bool cst = true, halves = true;
+      uint32_t prv = 0u;
+#pragma unroll 1
       for (uint32_t p = 0; p < NP; ++p) {
-        uint32_t v[8];
-        vals_load(vals, p, v);
+        const uint4* q8 = reinterpret_cast<const uint4*>(vals + 256u * p) + 2u * lane;
+        const uint4 va = q8[0], vb = q8[1];
+        const uint32_t v[8] = {va.x, va.y, va.z, va.w, vb.x, vb.y, vb.z, vb.w};
         uint32_t before = __shfl_up_sync(0xffffffffu, v[7], 1);
         if (lane == 0) before = prv;
         prv = __shfl_sync(0xffffffffu, v[7], 31);
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          nzor |= v[k];
-          cst &= v[k] == ((k & 1) ? refi : refr);
-        }
-        if (NP == 1u) {
-          const uint32_t a = __shfl_xor_sync(0xffffffffu, v[0], 16), b = __shfl_xor_sync(0xffffffffu, v[5], 16);
-          halves &= (a == v[0]) & (b == v[5]);
-        } else if (p >= NP / 2u) {
-          halves &= *val0(vals, p - NP / 2u) == v[0] && *val5(vals, p - NP / 2u) == v[5];
-        }
         uint32_t osum, otot;
         const uint32_t ocw = fast_codes(v, before, S, osum);
         const uint32_t ob = ooff >> 7;
@@ -350,6 +348,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
         const uint32_t endb = end ? (ooff + 127u) >> 7 : ooff >> 7, nb = endb - ob;
         if (!oom) oom = !wp_grow(P, wp, opg, onp, (16u + cb + 16u * endb + kPage - 1u) / kPage);
         if (!oom)
+#pragma unroll 1
           for (uint32_t k = lane; k < nb; k += 32u) {
             const uint32_t b = 16u + cb + 16u * (ob + k);
             reinterpret_cast<uint4*>(P.pages + (unsigned long long)opg[b >> 9] * kPage + (b & (kPage - 1u)))[0] = w4[k];
@@ -358,13 +357,12 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
           uint4 carry = make_uint4(0u, 0u, 0u, 0u);
           if (lane == 0) carry = w4[nb];
           __syncwarp();
+#pragma unroll 1
           for (uint32_t k = lane; k <= nb; k += 32u) w4[k] = k == 0u ? carry : make_uint4(0u, 0u, 0u, 0u);
           __syncwarp();
         }
       }
-      const bool c = __all_sync(0xffffffffu, cst), z = __any_sync(0xffffffffu, nzor != 0u), hh = __all_sync(0xffffffffu, halves);
-      const bool any_spec = __any_sync(0xffffffffu, spec);
-      keep = keep && !c && z && !hh && !any_spec;
+      keep = keep && group_differs(vals, NP) && group_moves(vals, NP) && !__any_sync(0xffffffffu, spec);
       if ((int)lane >= last) size = 16u + cb + resid_bytes(ooff);
     }
     if (corrupt && lane == 0) atomicOr(&ctl->err, (unsigned)E_CORRUPT);
@@ -384,6 +382,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
       if (lane == 0)
         reinterpret_cast<uint4*>(P.pages + (unsigned long long)opg[0] * kPage)[0] = make_uint4(M_STREAM | (S << 8), plen, N, ooff);
       uint32_t* e = dir_entry(P, ch);
+#pragma unroll 1
       for (uint32_t k = lane; k < onp; k += 32u) e[4 + k] = opg[k];
       uint32_t prev = __shfl_up_sync(0xffffffffu, size, 1);
       if (lane == 0) prev = ib;
@@ -403,6 +402,7 @@ __global__ void __launch_bounds__(32 * kGroupWarps, 5) k_group(const __grid_cons
   __syncwarp();
   {
     const uint32_t n = *wp.n;
+#pragma unroll 1
     for (uint32_t q = lane; q < n; q += 32u) P.wcache[gw * kWarpCache + q] = wp.ids[q];
     if (lane == 0) {
       P.wcache_n[gw] = n;

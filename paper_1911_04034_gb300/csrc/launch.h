@@ -49,7 +49,8 @@ struct alignas(16) GateLaunch {
   int arith;                     // 0 dense: the four sums with every coefficient, zeros included;
                                  // 1 diagonal (u01 = u10 = 0); 2 anti-diagonal (u00 = u11 = 0);
                                  // 3 real (every imaginary part zero): the real products only;
-                                 // 4 every coefficient part +-2^sk, none zero: signed sums, then scaled
+                                 // 4 every coefficient part +-2^sk, none zero: signed sums, then scaled;
+                                 // 5 real diagonal, imaginary off-diagonal (RX): the two products left of each sum
   int rop[2];                    // diagonal / anti-diagonal, per output row: 0 complex product, 1 copy
                                  // (the entry is exactly 1), 2 negation (exactly -1)
   double cf[16];                 // dense: row r's coefficients of (ar, ai, br, bi) / (ai, ar, bi, br) at 4r

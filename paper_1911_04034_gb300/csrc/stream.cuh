@@ -161,19 +161,30 @@ __device__ __forceinline__ void fast_rebuild(uint32_t e[8], uint32_t cw, uint32_
   }
 }
 
+// 24 - 8 (code) of a value whose XOR with its predecessor is x: with f the index of the
+// highest set bit of x | 1, 8 times the leading identical bytes, at most 3, is 24 - (f & 24).
+__device__ __forceinline__ uint32_t code_rest(uint32_t x) {
+  uint32_t f;
+  asm("bfind.u32 %0, %1;" : "=r"(f) : "r"(x | 1u));
+  return f & 0x18u;
+}
+// Its residual bits max(S - 8 code, 0).
+__device__ __forceinline__ uint32_t rest_bits(uint32_t rest, uint32_t S) {
+  return (uint32_t)max((int)(S + rest) - 24, 0);
+}
+
 // Codes of a lane's 8 truncated values (predecessor of the first: pr), as the lane's
 // 16-bit code field; `sum` receives their residual-length sum.
 __device__ __forceinline__ uint32_t fast_codes(const uint32_t t[8], uint32_t pr, uint32_t S, uint32_t& sum) {
-  uint32_t cw = 0u, s = 0u;
+  uint32_t inv = 0u, s = 0u;  // inv: 3 - code, the codes' bits inverted
 #pragma unroll
   for (int k = 0; k < 8; ++k) {
-    const uint32_t x = t[k] ^ (k ? t[k - 1] : pr);
-    const uint32_t c8 = min((uint32_t)__clz((int)x), 24u) & 0x18u;
-    s += rlen(S, c8);
-    cw |= (c8 >> 3) << code_shift(k);
+    const uint32_t r = code_rest(t[k] ^ (k ? t[k - 1] : pr));
+    s += rest_bits(r, S);
+    inv |= (r >> 3) << code_shift(k);
   }
   sum = s;
-  return cw;
+  return ~inv & 0xffffu;
 }
 
 // Packs the residuals of a lane's 8 values (high words t, codes in the lane's code
@@ -207,8 +218,8 @@ __device__ __forceinline__ void fast_pack(uint32_t* win, uint32_t w4, uint32_t o
 }
 
 // Decodes a STREAM image of ib bytes (header checked: width S, `bits` residual bits) pass by
-// pass: f(p, v) receives the high words of the lane's 8 values of pass p.  win: two windows
-// of kFastWin bytes.  False if the residual lengths disagree with the header.
+// pass: f(p, v, tot, cw) receives the high words of the lane's 8 values of pass p, the
+// pass's residual bits and the lane's code field.  win: two windows of kFastWin bytes.  False if the residual lengths disagree with the header.
 template <class Image, class F>
 __device__ __forceinline__ bool stream_decode(const Image& img, int kc, uint32_t S, uint32_t bits, uint32_t ib,
                                               uint32_t* win0, uint32_t* win1, const F& f) {
@@ -218,6 +229,7 @@ __device__ __forceinline__ bool stream_decode(const Image& img, int kc, uint32_t
   uint32_t cw_next = codes(0u), off = 0u, lead = 0u;
   fast_issue_window(img, win0, cb, 0u, nbs);
   cp_async_commit();
+#pragma unroll 1
   for (uint32_t p = 0; p < NP; ++p) {
     uint32_t* const win = (p & 1u) ? win1 : win0;
     const uint32_t cw = (cw_next >> (16u * (lane & 1u))) & 0xffffu;
@@ -234,7 +246,7 @@ __device__ __forceinline__ bool stream_decode(const Image& img, int kc, uint32_t
     const uint32_t before = lead_scan_warp(W, lead, after);
     lead = after;
     fast_rebuild(v, cw, before);
-    f(p, v);
+    f(p, v, tot, cw);
     __syncwarp();  // every lane is done with the window the next pass refills
   }
   return off == bits;
@@ -291,6 +303,7 @@ __device__ __forceinline__ void wp_free(const Pool& P, const WarpPages& wp, cons
     if (lane == 0) base = atomicAdd(&P.ctl->nfreed, (unsigned long long)(cnt - room));
     base = __shfl_sync(0xffffffffu, base, 0);
   }
+#pragma unroll 1
   for (uint32_t q = lane; q < cnt; q += 32u) {
     const uint32_t id = ids[q];
     if (q < room) {
@@ -382,6 +395,20 @@ __device__ __forceinline__ double2 real_rows(const double* cf, double2 a, double
   return make_double2(__fma_rn(cf[2], b.x, __dmul_rn(cf[0], a.x)), __fma_rn(cf[2], b.y, __dmul_rn(cf[0], a.y)));
 }
 
+// The same output for a matrix with a real diagonal and imaginary off-diagonal entries (RX):
+// the two products of each chain that are left, in their order (row 0: cf[0], cf[3] and cf[4],
+// cf[7]; row 1: cf[1], cf[2] and cf[5], cf[6]).
+__device__ __forceinline__ double2 rx_rows(const double* cf, uint32_t row, double2 a, double2 b) {
+  const double ax = row ? a.y : a.x, ay = row ? a.x : a.y, bx = row ? b.x : b.y, by = row ? b.y : b.x;
+  return make_double2(__fma_rn(cf[3u - row], bx, __dmul_rn(cf[row], ax)), __fma_rn(cf[7u - row], by, __dmul_rn(cf[4u + row], ay)));
+}
+// Row pair `row` of the dense (0), real (3) or RX (5) form; cf: all sixteen coefficients.
+template <int ARITH>
+__device__ __forceinline__ double2 form_rows(const double* cf, uint32_t row, double2 a, double2 b) {
+  return ARITH == 0 ? dense_rows(cf + 8u * row, a, b)
+                    : (ARITH == 3 ? real_rows(cf + 8u * row, a, b) : rx_rows(cf + 8u * row, row, a, b));
+}
+
 // The same output for a gate whose coefficient parts are all +-2^k, none zero (sqrt(X),
 // sqrt(Y)): every product of the chains above is exact, so each chain equals 2^k times
 // the chain of the signed inputs in the same order (scaling by a power of two commutes
@@ -467,10 +494,9 @@ __device__ __forceinline__ void fast_pair(const Gate& L, uint32_t i, uint32_t& a
   if ((i & L.lo_mask) == L.lo_vals) {
     if constexpr (ARITH == 4) {
       signed_pair(L, ar, ai, br, bi, mh, o, spec);
-    } else if constexpr (ARITH == 0 || ARITH == 3) {
+    } else if constexpr (ARITH == 0 || ARITH == 3 || ARITH == 5) {
       const double2 a = make_double2(hi_as_double(ar), hi_as_double(ai)), b = make_double2(hi_as_double(br), hi_as_double(bi));
-      const double2 x = ARITH == 0 ? dense_rows(L.cf, a, b) : real_rows(L.cf, a, b);
-      const double2 y = ARITH == 0 ? dense_rows(L.cf + 8, a, b) : real_rows(L.cf + 8, a, b);
+      const double2 x = form_rows<ARITH>(L.cf, 0u, a, b), y = form_rows<ARITH>(L.cf, 1u, a, b);
       o[0] = fast_trunc(x.x, mh, spec);
       o[1] = fast_trunc(x.y, mh, spec);
       o[2] = fast_trunc(y.x, mh, spec);

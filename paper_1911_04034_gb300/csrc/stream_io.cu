@@ -73,7 +73,7 @@ __device__ __forceinline__ bool read_warp(const ReadArgs& R, unsigned long long 
       r[k] = vec ? reinterpret_cast<const double2*>(s)[k] : make_double2(s[2 * k], s[2 * k + 1]);
   };
   if constexpr (MODE == kReadDot) fetch(0u);
-  auto pass = [&](uint32_t p, const uint32_t v[8]) {
+  auto pass = [&](uint32_t p, const uint32_t v[8], uint32_t, uint32_t) {
     if constexpr (MODE == kReadRange || MODE == kReadCodec) {
       // through shared memory: a warp's stores then cover whole lines
       reinterpret_cast<uint4*>(stage)[2u * lane] = make_uint4(v[0], v[1], v[2], v[3]);

@@ -88,3 +88,22 @@ def test_power_of_two_identity_holds_below_the_kernel_floor():
             assert bits(0.5 * signed) == bits(want)
             checked += 1
     assert checked > n
+
+
+def test_rx_form_takes_the_kept_terms_of_both_rows():
+    """Real diagonal, imaginary off-diagonal entries: the sixteen coefficients in the kernel's
+    order leave two terms a chain, at (row, 3 - row) of the real and (4 + row, 7 - row) of the
+    imaginary chain of row pair `row`."""
+    rng = np.random.default_rng(5)
+    c, s = float(np.cos(0.15)), float(np.sin(0.15))
+    u = [c, 0.0, 0.0, -s, 0.0, -s, c, 0.0]
+    cf = [u[0], -u[1], u[2], -u[3], u[0], u[1], u[2], u[3], u[4], -u[5], u[6], -u[7], u[4], u[5], u[6], u[7]]
+    for _ in range(200):
+        ar, ai, br, bi = (float(v) for v in truncate_hi(rng.standard_normal(4), 26))
+        for row in (0, 1):
+            k = cf[8 * row: 8 * row + 8]
+            re = kept_chain(k[:4], [ar, ai, br, bi])
+            im = kept_chain(k[4:], [ai, ar, bi, br])
+            ax, ay, bx, by = (ai, ar, br, bi) if row else (ar, ai, bi, br)
+            assert bits(fma(k[3 - row], bx, k[row] * ax)) == bits(re)
+            assert bits(fma(k[7 - row], by, k[4 + row] * ay)) == bits(im)
