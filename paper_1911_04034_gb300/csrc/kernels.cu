@@ -8,7 +8,7 @@
 //          to the page pool.  Decoded amplitudes never leave shared memory.
 // k_post   after each gate: returns freed pages to the stack, adds the gate's byte
 //          change to E, and records the controller's level and fidelity bounds.
-// others   initialisation, codec entry points, readout and the uncompressed path.
+// others   image exchange, initialisation, the general codec encoder, checkpoints.
 #include "launch.h"
 #include "gate_item.cuh"
 
@@ -418,9 +418,9 @@ cudaError_t launch_codec_encode(const double* in, unsigned long long nchunks, in
   const size_t smem = codec_smem_bytes(kc);
   const unsigned long long sms = (unsigned long long)num_sms(), g = nchunks < sms * 8 ? nchunks : sms * 8;
   // Solution C's modes at S <= 32 on enough chunks: a warp per chunk first, then the general
-  // encoder on the chunks it left.  (Below two CTAs an SM a CTA per chunk is sooner done.)
+  // encoder on the chunks it left.  (With fewer chunks a CTA each is sooner done.)
   const bool warp = todo && force < 0 && modes == kDefaultModes && S <= 32u && kc >= kFastMinKC &&
-                    nchunks >= 2ull * kWarps * sms && (reinterpret_cast<uintptr_t>(in) & 15u) == 0u;
+                    nchunks >= 12ull * sms && (reinterpret_cast<uintptr_t>(in) & 15u) == 0u;
   if (warp) {
     const cudaError_t e = launch_stream_encode(in, nchunks, kc, S, out, stride, lens, todo, pad, st);
     if (e != cudaSuccess) return e;

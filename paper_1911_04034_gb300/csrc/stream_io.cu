@@ -348,8 +348,9 @@ static cudaError_t launch_read(ReadArgs& R, cudaStream_t st) {
   const int kc = R.P.kc;
   const size_t smem = read_smem_bytes(kc);
   const unsigned long long sms = (unsigned long long)num_sms();
-  // a warp per chunk where that still leaves two CTAs an SM; fewer chunks decode sooner by a CTA each
-  R.per = kc >= kFastMinKC && R.nchunks >= 2ull * kWarps * sms ? (uint32_t)kWarps : 1u;
+  // A warp per chunk from about 2000 chunks on; fewer decode sooner by a CTA each (measurement
+  // in 2^9-amplitude chunks: 512 of them 68 us by CTAs, 81 by warps; 2048, 81 and 78).
+  R.per = kc >= kFastMinKC && R.nchunks >= 12ull * sms ? (uint32_t)kWarps : 1u;
   const unsigned long long want = (R.nchunks + R.per - 1ull) / R.per, grid = want < 8ull * sms ? want : 8ull * sms;
   QC_VPT_DISPATCH(kc, {
     const cudaError_t e = prep(k_read<V, MODE>, smem);
