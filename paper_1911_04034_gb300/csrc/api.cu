@@ -131,6 +131,10 @@ int device_sms() {
 
 void qc::set_last_error(const char* msg) { g_last_error = msg; }
 
+// Largest state (in chunks) that k_run takes in several rounds: its CTAs wait for the slowest
+// of them after each step, and that wait is bounded.
+constexpr uint64_t kRunChunks = 1ull << 18;
+
 struct sim {
   int n = 0, b = 0, kc = 0, ladder = 0;
   double eps_max = 0.0, tau = 0.9;
@@ -376,7 +380,7 @@ sim_status sim_create_ex(int n_qubits, int block_log2, int chunk_log2, double er
     const uint64_t fit = sms * qc::run_ctas_per_sm(s->kc, false), items = (s->nchunks + 1) / 2;
     // a lossless run has nothing to settle: its groups share passes at any size (23 qubits,
     // 11.1 ms a random-circuit layer gate by gate, 7.1 ms by groups)
-    const bool any = cp.nlevels == 0 && s->nchunks <= (1ull << 20);
+    const bool any = cp.nlevels == 0 && s->nchunks <= kRunChunks;
     s->run_wide = wide > 0 && (items <= wide || (any && items > fit));
     if (items <= fit || any) s->run_grid = (int)(s->run_wide ? (items < wide ? items : wide) : (items < fit ? items : fit));
     // larger states: groups of gates (see group_circuit)
@@ -1377,7 +1381,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
     // numbered consecutively.
     const int resident = device_sms() * qc::run_ctas_per_sm(kc, false);
     bool whole = count <= resident / 2;
-    for (int k = 0; k < count; ++k) whole = whole && run_options(sims[k]) && n_gates[k] < (1u << 20);
+    for (int k = 0; k < count; ++k) whole = whole && run_options(sims[k]) && n_gates[k] < (1u << 20) && sims[k]->nchunks <= kRunChunks;
     std::vector<qc::BatchJob> jobs;
     std::vector<sim*> job_sim;  // the handle of each job
     std::vector<size_t> off(steps + 1, 0);
