@@ -536,6 +536,15 @@ static GateLaunch make_launch(sim* s, const sim_gate* g) {
     L.gfeat = (real ? 1u : 0u) | (diag ? 2u : 0u) | (perm ? 4u : 0u) | (t < kc ? 8u : 0u);
     // a cross-chunk diagonal gate with a row that is an exact copy: the row that is not
     L.diag = diag ? 1 : 0;
+    int e = 0;
+    L.pow2 = u[0] != 0.0 && std::fabs(std::frexp(u[0], &e)) == 0.5 && e >= -9 && e <= 1 ? 1 : 0;
+    for (int k = 1; k < 8; ++k)
+      if (std::fabs(u[k]) != std::fabs(u[0])) L.pow2 = 0;
+    if (L.pow2) {
+      L.sk = e - 1;
+      for (int q = 0; q < 16; ++q)
+        if (L.g.c[q] < 0.0) L.sgn |= 1u << q;
+    }
     L.copy = diag ? (u[0] == 1.0 && u[1] == 0.0 ? 1u : 0u) | (u[6] == 1.0 && u[7] == 0.0 ? 2u : 0u) : 0u;
     L.solo = -1;
     if (t >= kc && diag) L.solo = u[0] == 1.0 && u[1] == 0.0 ? 1 : (u[6] == 1.0 && u[7] == 0.0 ? 0 : -1);
@@ -610,20 +619,7 @@ static bool fast_applies(const sim* s, const sim_gate* g, GateLaunch& L) {
   const bool real = u[1] == 0.0 && u[3] == 0.0 && u[5] == 0.0 && u[7] == 0.0;
   const bool rx = u[1] == 0.0 && u[2] == 0.0 && u[4] == 0.0 && u[7] == 0.0;
   L.arith = diag ? 1 : (anti ? 2 : (real ? 3 : (rx ? 5 : 0)));
-  if (L.arith == 0) {
-    // every coefficient part of the same magnitude 2^k, none zero: exact products
-    const double c = std::fabs(cf[0]);
-    bool pow2 = c > 0.0;
-    for (int k = 1; k < 16 && pow2; ++k) pow2 = std::fabs(cf[k]) == c;
-    int e = 0;
-    if (pow2 && std::frexp(c, &e) == 0.5 && e - 1 >= -64 && e - 1 <= 0) {
-      L.arith = 4;
-      L.sk = e - 1;
-      L.sgn = 0;
-      for (int k = 0; k < 16; ++k)
-        if (cf[k] < 0.0) L.sgn |= 1u << k;
-    }
-  }
+  if (L.arith == 0 && L.pow2) L.arith = 4;  // exact products
   if (L.arith == 1 || L.arith == 2) {
     // the one nonzero entry of each row: a' = d0 x, b' = d1 y (x, y = a, b or b, a)
     const double d[4] = {diag ? u[0] : u[2], diag ? u[1] : u[3], diag ? u[6] : u[4], diag ? u[7] : u[5]};

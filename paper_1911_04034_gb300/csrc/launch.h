@@ -27,6 +27,7 @@ struct alignas(16) GateLaunch {
   int pair;                      // 1: target >= chunk_log2
   int diag;                      // 1: the matrix is diagonal
   uint32_t copy;                 // diagonal: bit r, row r is an exact copy
+  int pow2;                      // 1: every coefficient part is +-2^sk (sgn: see below)
   int group;                     // k_run: gates, this one first, that one step can take (see mark_groups)
   unsigned long long group_bit;  // ... and the chunk-index bit of their cross-chunk target, 0 if none
   int swap;                      // 1: X between chunks that may exchange whole images (see swap_item)
@@ -55,8 +56,8 @@ struct alignas(16) GateLaunch {
                                  // (the entry is exactly 1), 2 negation (exactly -1)
   double cf[16];                 // dense: row r's coefficients of (ar, ai, br, bi) / (ai, ar, bi, br) at 4r
   double du[4];                  // diagonal: u00, u11; anti-diagonal: u01, u10 (re, im)
-  uint32_t sgn;                  // arith 4: bit q set if coefficient cf[q] is negative
-  int sk;                        // arith 4: log2 of the coefficients' common magnitude
+  uint32_t sgn;                  // pow2, arith 4: bit q set if coefficient cf[q] is negative
+  int sk;                        // pow2, arith 4: log2 of the coefficients' common magnitude
 };
 
 // One gate of one simulator inside a batched launch; its work items are the global

@@ -185,7 +185,7 @@ __device__ __forceinline__ bool run_item(const Pool& P, GateLaunch* rec, int b, 
         if ((i & L.lo_mask) != L.lo_vals) continue;
         const uint32_t pi = tile_amp(i);
         double2 x = t0[pi], y = t1[pi];
-        apply_pair(L.g, x, y);
+        if (!L.pow2 || !pow2_pair(L.sgn, L.sk, x, y)) apply_pair(L.g, x, y);
         t0[pi] = x;
         t1[pi] = y;
       }
@@ -208,7 +208,7 @@ __device__ __forceinline__ bool run_item(const Pool& P, GateLaunch* rec, int b, 
         double2* const t = second ? t1 : t0;
         const uint32_t p0 = tile_amp(i0), p1 = tile_amp(i0 | tb);
         double2 x = t[p0], y = t[p1];
-        apply_pair(L.g, x, y);
+        if (!L.pow2 || !pow2_pair(L.sgn, L.sk, x, y)) apply_pair(L.g, x, y);
         t[p0] = x;
         t[p1] = y;
       }

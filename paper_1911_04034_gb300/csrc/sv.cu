@@ -18,51 +18,6 @@ namespace qc {
 
 constexpr int kSvThreads = 256;
 
-// The four sums of a dense gate whose coefficient parts are all +-2^k (k <= 0): every
-// product is exact, so a chain of four equals 2^k times the chain of the signed inputs in
-// the same order while no partial sum leaves the normal range.  The first sums of the four
-// chains are +-(ar + ai) and +-(ar - ai), so two additions serve all four: 10 instead of
-// 16 FP64 operations.  False (nothing done) if an input is nonzero below 2^-959 or above
-// 2^1020: inputs of at least 2^-959 are multiples of 2^-1011, so a nonzero sum times 2^k
-// (k >= -10) stays normal, and no sum overflows.
-__device__ __forceinline__ bool sv_pow2_pair(uint32_t sgn, int sk, double2& a, double2& b) {
-  auto bad = [](double v) {
-    const uint64_t u = (uint64_t)__double_as_longlong(v);
-    const uint32_t h = (uint32_t)(u >> 32) & 0x7fffffffu;
-    return (h - (64u << 20)) >= ((0x7fcu - 64u) << 20) && (h | (uint32_t)u) != 0u;
-  };
-  if (bad(a.x) | bad(a.y) | bad(b.x) | bad(b.y)) return false;
-  auto hi = [](double v) { return (uint32_t)__double2hiint(v); };
-  auto sbit = [sgn](int q) { return ((sgn >> q) & 1u) << 31; };
-  auto sg = [&](int q, double v) { return __hiloint2double((int)(hi(v) ^ sbit(q)), __double2loint(v)); };
-  const double sum = __dadd_rn(a.x, a.y), dif = __dsub_rn(a.x, a.y);
-  // Zero tests on the words: a double comparison would take the FP64 pipe.
-  const bool zs = ((hi(sum) << 1) | (uint32_t)__double2loint(sum)) == 0u;
-  const bool zd = ((hi(dif) << 1) | (uint32_t)__double2loint(dif)) == 0u;
-  // (+-x) + (+-y) for the chain whose first term is coefficient q: x = a.x, y = a.y for the
-  // real chains, the other way round for the imaginary ones.  A zero sum is +0 unless both
-  // its terms are -0.
-  auto first = [&](int q, bool im) {
-    const uint32_t sx = sbit(im ? q + 1 : q), sy = sbit(im ? q : q + 1);  // the signs of a.x and a.y
-    const bool same = sx == sy;
-    const double m = same ? sum : dif;
-    const uint32_t h = (same ? zs : zd) ? ((hi(a.x) ^ sx) & (hi(a.y) ^ sy) & 0x80000000u) : hi(m) ^ sx;
-    return __hiloint2double((int)h, __double2loint(m));
-  };
-  auto scaled = [&](double y) {
-    const uint32_t h = hi(y);
-    const bool zero = ((h << 1) | (uint32_t)__double2loint(y)) == 0u;
-    return zero ? y : __hiloint2double((int)(h + ((uint32_t)sk << 20)), __double2loint(y));
-  };
-  const double re0 = __dadd_rn(__dadd_rn(first(0, false), sg(2, b.x)), sg(3, b.y));
-  const double im0 = __dadd_rn(__dadd_rn(first(4, true), sg(6, b.y)), sg(7, b.x));
-  const double re1 = __dadd_rn(__dadd_rn(first(8, false), sg(10, b.x)), sg(11, b.y));
-  const double im1 = __dadd_rn(__dadd_rn(first(12, true), sg(14, b.y)), sg(15, b.x));
-  a = make_double2(scaled(re0), scaled(im0));
-  b = make_double2(scaled(re1), scaled(im1));
-  return true;
-}
-
 // State index of tile index i, less the tile's base.
 __device__ __forceinline__ unsigned long long sv_offset(const SvGroup& G, uint32_t i) {
   unsigned long long o = i & ((1u << G.L) - 1u);
@@ -115,7 +70,7 @@ __global__ void __launch_bounds__(kSvThreads) k_sv_group(double2* psi, const __g
         const uint32_t i = ((p & ~lowm) << 1) | (p & lowm);
         if ((i & g.lo_mask) != g.lo_vals) continue;
         double2 a = s_tile[i], b = s_tile[i | tb];
-        if (g.form != 1 || !sv_pow2_pair(g.sgn, g.sk, a, b)) apply_pair(g.g, a, b);
+        if (g.form != 1 || !pow2_pair(g.sgn, g.sk, a, b)) apply_pair(g.g, a, b);
         s_tile[i] = a;
         s_tile[i | tb] = b;
       }
