@@ -181,3 +181,26 @@ def test_budget_and_named_options():
     d.apply_circuit(gates)
     e.apply_circuit(gates)
     assert images(d) == images(e)
+
+
+def test_batch_with_large_states_among_small_ones():
+    """Circuits on large states run one by one in groups of gates, the small ones together
+    under the kept graph: every circuit ends as it does alone, on a replay too."""
+    kc, eps = 7, 1e-4
+    specs = [(19, 3), (11, 5), (19, 2), (13, 4)]
+    circuits = [Cc.rcs_n(n, d, seed=500 + k) for k, (n, d) in enumerate(specs)]
+    batch = [make(n, kc, eps) for n, _ in specs]
+    alone = []
+    for k, (n, _) in enumerate(specs):
+        solo = make(n, kc, eps)
+        solo.apply_circuit(circuits[k])
+        alone.append((images(solo), solo.stats()))
+    for replay in (0, 1):
+        qc().batch_apply(batch, circuits, use_graph=True)
+        for k, s in enumerate(batch):
+            assert images(s) == alone[k][0], (replay, k)
+            for key in ("gates", "encoded_bytes", "max_encoded_bytes", "eps_switch_gate", "level", "amp_updates", "peak_pages_bytes"):
+                assert s.stats()[key] == alone[k][1][key], (replay, k, key)
+        assert batch[0].stats()["graph_replays"] == replay
+        for s in batch:
+            s.reset()
