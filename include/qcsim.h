@@ -150,19 +150,24 @@ sim_status sim_set_stream(sim_t* sim, void* cuda_stream);
  * synchronising call.  Kernels per gate: the selector's decisions (selector 2 only);
  * at chunk sizes 2^7..2^11 and widths S <= 32 the streaming kernel (a warp pair per
  * work item, STREAM images in and out); the general kernel over the items the
- * streaming kernel left, or the whole gate; the bookkeeping kernel.  Every path writes
- * the same bytes. */
+ * streaming kernel left, or the whole gate; the bookkeeping kernel.  X between chunks
+ * exchanges whole images where they stand as the encoder would write them.  Every path
+ * writes the same bytes. */
 sim_status sim_apply_gate(sim_t* sim, const sim_gate* gate);
 
 /* Applies n_gates gates in order.  All gates are validated first (none runs if one
  * is invalid).  `gates` is a host array.  Synchronises the stream at the end and
- * returns any device-side error. */
+ * returns any device-side error.  With the default options a small or a lossless state
+ * runs its circuit in one launch, a large one groups of gates per pass once the error
+ * bound is settled: the same images and counters as gate by gate. */
 sim_status sim_apply_circuit(sim_t* sim, const sim_gate* gates, size_t n_gates);
 
 /* Batched form: runs `count` circuits, circuits[k] (n_gates[k] gates) on handle
- * sims[k], together.  Gate step t applies gate t of every circuit that has one with a
- * single fused-kernel launch covering the work items of all of them (and one
- * bookkeeping launch); with use_graph != 0 the whole launch sequence is captured into a
+ * sims[k], together: one launch in which every circuit has thread blocks of its own and
+ * goes at its own pace or, where an option of a handle needs kernels around each gate
+ * (timing, selector network, traces, block cache, a mode set other than the default),
+ * gate step t of every circuit that has one in a single fused-kernel launch and one
+ * bookkeeping launch; with use_graph != 0 the launch sequence is captured into a
  * CUDA graph, launched, and kept by sims[0]: a later call whose launches are the same
  * (same handles and settings, same gates; e.g. after sim_reset) replays it without
  * capturing or uploading again (sim_stats_t.graph_replays).  Each handle keeps its own
