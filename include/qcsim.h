@@ -164,7 +164,8 @@ sim_status sim_apply_circuit(sim_t* sim, const sim_gate* gates, size_t n_gates);
 
 /* Batched form: runs `count` circuits, circuits[k] (n_gates[k] gates) on handle
  * sims[k], together: one launch in which every circuit has thread blocks of its own and
- * goes at its own pace or, where an option of a handle needs kernels around each gate
+ * goes at its own pace (circuits on large lossy states, which fill the chip by themselves,
+ * one by one before it, as sim_apply_circuit runs them) or, where an option of a handle needs kernels around each gate
  * (timing, selector network, traces, block cache, a mode set other than the default),
  * gate step t of every circuit that has one in a single fused-kernel launch and one
  * bookkeeping launch; with use_graph != 0 the launch sequence is captured into a
