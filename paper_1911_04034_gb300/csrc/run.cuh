@@ -292,16 +292,17 @@ __device__ __forceinline__ bool run_item(const Pool& P, GateLaunch* rec, int b, 
 // Bookkeeping of a step of G gates (one block; every CTA of the simulator has arrived).
 __device__ __forceinline__ void run_book(const Pool& P, const CtlParams& cp, int G) {
   DevCtl* ctl = P.ctl;
-  __shared__ unsigned long long s_top;
+  __shared__ unsigned long long s_top, s_nf;
   __shared__ int s_skip;
   if (threadIdx.x == 0) {
     const long long top = *(volatile long long*)&ctl->top;
     s_skip = *(volatile unsigned int*)&ctl->err != 0u || top < 0;  // see post_body
     s_top = s_skip ? 0ull : (unsigned long long)top;
+    s_nf = ctl->nfreed;  // read here alone: thread 0 clears it below while other warps still copy
   }
   __syncthreads();
   if (s_skip) return;
-  const unsigned long long nf = ctl->nfreed;
+  const unsigned long long nf = s_nf;
   const unsigned long long top = s_top;
   for (unsigned long long i = threadIdx.x; i < nf; i += blockDim.x) {
     if (top + i < P.npages) P.stack[top + i] = P.freed[i];

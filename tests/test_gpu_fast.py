@@ -259,3 +259,23 @@ def test_groups_of_gates_on_larger_states(kc, n):
         want = [orc.image(c) for c in range(orc.nchunks)]
         assert all_images(sims[0]) == want
         assert all_images(sims[1]) == want
+
+
+@pytest.mark.parametrize("ladder", [0, 1])
+def test_pages_freed_by_a_whole_circuit_come_back_once(ladder):
+    """A pool that just holds every chunk RAW (no CTA keeps a page id between steps), and
+    bounds that settle in between: a step then frees thousands of pages at once, and the
+    bookkeeping has to put each of them on the stack once.  A page handed out twice or lost
+    shows in the images that follow, or as a dry pool."""
+    n, kc, eps = 15, 8, 1e-3
+    raw = 16 << n
+    gates = Cc.rcs_n(n, 10, seed=21)
+    orc = O.CSim(n, 9, kc, eps, raw * 9 // 10, ladder=ladder)
+    orc.apply(gates)
+    want = [orc.image(c) for c in range(orc.nchunks)]
+    s = qc().Sim(n, 9, eps, chunk_log2=kc, budget=raw * 9 // 10, ladder=ladder, pool_bytes=512 * ((16 << kc) // 512 + 1) << (n - kc))
+    for _ in range(12):
+        s.apply_circuit(gates)
+        assert all_images(s) == want
+        assert s.stats()["max_encoded_bytes"] > 2 * s.stats()["encoded_bytes"]
+        s.reset()
