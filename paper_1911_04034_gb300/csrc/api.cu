@@ -131,8 +131,8 @@ int device_sms() {
 
 void qc::set_last_error(const char* msg) { g_last_error = msg; }
 
-// Largest state (in chunks) that k_run takes in several rounds: its CTAs wait for the slowest
-// of them after each step, and that wait is bounded.
+// Largest state (in chunks) that k_run takes in several rounds: after a step one CTA returns the
+// freed pages (up to 33 a chunk of 2^10 amplitudes) while the others wait.
 constexpr uint64_t kRunChunks = 1ull << 18;
 
 struct sim {
@@ -169,6 +169,7 @@ struct sim {
   size_t run_cap = 0;
   int run_grid = 0;                  // its CTAs (0: not used for this state)
   bool run_wide = false;             // ... two an SM
+  uint32_t run_polls = qc::kRunPolls;  // ... polls without progress before a wait of theirs gives up
   int group_grid = 0;                // CTAs of k_group (0: not used for this state)
   int rest_grid = 0;                 // ... and of the k_run launch after it
   int fast_grid = 0;                 // CTAs of the streaming kernel (0: chunk size outside its range)
@@ -749,7 +750,7 @@ static sim_status run_circuit(sim* s, const sim_gate* gates, size_t n, bool* ran
         s->amp_updates += s->h_run[off + k].nact << s->kc;
       }
       mark_groups(s->h_run + off, m);
-      s->h_run_jobs[seg] = {s->d_run + off, (int)m, 0, s->run_grid, run_keep(s, s->run_grid), nullptr};
+      s->h_run_jobs[seg] = {s->d_run + off, (int)m, 0, s->run_grid, run_keep(s, s->run_grid), nullptr, s->run_polls};
       CK(cudaMemcpyAsync(s->d_run + off, s->h_run + off, m * sizeof(GateLaunch), cudaMemcpyHostToDevice, s->st), "gate records");
       CK(cudaMemcpyAsync(s->d_run_jobs + seg, s->h_run_jobs + seg, sizeof(qc::RunJob), cudaMemcpyHostToDevice, s->st), "gate records");
       CK(qc::launch_run(s->d_run_jobs + seg, 1, s->kc, s->run_grid, s->run_wide, s->st), "circuit kernel launch");
@@ -884,7 +885,7 @@ static sim_status group_circuit(sim* s, const sim_gate* gates, size_t n) {
     size_t jobs = 0;
     for (size_t k = 0; k < block; k += (size_t)s->h_run[k].group)
       if (s->h_run[k].group > 1)
-        s->h_run_jobs[jobs++] = {s->d_run + k, s->h_run[k].group, 0, s->rest_grid, 0u, s->d_defer};
+        s->h_run_jobs[jobs++] = {s->d_run + k, s->h_run[k].group, 0, s->rest_grid, 0u, s->d_defer, s->run_polls};
     CK(cudaMemcpyAsync(s->d_run, s->h_run, block * sizeof(GateLaunch), cudaMemcpyHostToDevice, s->st), "gate records");
     CK(cudaMemcpyAsync(s->d_run_jobs, s->h_run_jobs, jobs * sizeof(qc::RunJob), cudaMemcpyHostToDevice, s->st), "gate records");
     jobs = 0;
@@ -1033,6 +1034,11 @@ sim_status sim_set_option(sim_t* s, const char* key, int64_t value) {
   if (k == "fast_path") {
     if (value != 0 && value != 1) return fail(SIM_ERR_INVALID, "fast_path must be 0 or 1");
     s->fast = value != 0;
+    return SIM_OK;
+  }
+  if (k == "wait_polls") {
+    if (value < 1 || value > (int64_t)qc::kRunPolls) return fail(SIM_ERR_INVALID, "wait_polls must be in [1, %u]", qc::kRunPolls);
+    s->run_polls = (uint32_t)value;
     return SIM_OK;
   }
   if (k == "tau_ppm") {
@@ -1448,7 +1454,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
         if (!n_gates[k]) continue;
         const size_t at = (size_t)(reinterpret_cast<const uint8_t*>(first[k]) - run_list.data());
         const qc::RunJob j{reinterpret_cast<const GateLaunch*>((const uint8_t*)d_jobs + at), (int)n_gates[k], run_grid,
-                           ctas[k], run_keep(sims[k], ctas[k]), nullptr};
+                           ctas[k], run_keep(sims[k], ctas[k]), nullptr, sims[k]->run_polls};
         std::memcpy(run_list.data() + (size_t)njobs++ * sizeof j, &j, sizeof j);
         run_grid += ctas[k];
       }

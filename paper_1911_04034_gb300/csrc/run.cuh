@@ -8,7 +8,11 @@ namespace qc {
 // bookkeeping, 12 to 30 us a gate), so one launch runs a whole circuit.  Each CTA takes its
 // share of a step's chunk pairs, the simulator's CTAs meet at a counter in device memory,
 // and the last to arrive does the bookkeeping and releases the others.  Every CTA is
-// resident (a cooperative launch) and every wait is bounded (E_TIMEOUT, site 4).  Page ids
+// resident (a cooperative launch) and every wait is bounded: a CTA that sees nothing move --
+// no CTA of its simulator arrive, none finish an item that is not its last -- during job.polls
+// polls gives up (E_TIMEOUT, site 4).  (Polls alone would bound a step's work instead: a CTA
+// that holds all the chunks of a batch's circuit that are not zero takes seconds over 32 gates,
+// while the others wait.)  Page ids
 // freed by a CTA's items stay with it between steps, up to job.keep of them (counted in
 // wc_pages like the streaming kernel's); the rest goes to the freed list.
 //
@@ -20,7 +24,6 @@ namespace qc {
 // Lossy random circuits, gate by gate in one launch -> by steps: 12 qubits in 2^8-amplitude
 // chunks 14.1 -> 7.0 us a gate, 17 in 2^9 17.5 -> 9.3, 18 in 2^10 24.0 -> 14.5, 19 in 2^11
 // 28.2 -> 18.7 (a streaming, a general and a bookkeeping launch per gate: 26, 31, 46, 73).
-constexpr uint32_t kRunSpins = 1u << 22;
 
 // What a step's gates changed, per gate (shared memory, thread 0 of a CTA writes).
 struct RunSums {
@@ -385,7 +388,8 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : CTAS)
   }
   __syncthreads();
   if (threadIdx.x == 0) s_P = s_rec[0].P;
-  __syncthreads();
+  // a wait that gave up in an earlier launch: its CTAs' counts do not add up any more
+  if (__syncthreads_or(threadIdx.x == 0 && (*(volatile unsigned int*)&s_rec[0].P.ctl->err & (unsigned)E_TIMEOUT) != 0u)) return;
   const Pool& P = s_P;
   const unsigned long long nchunks = s_rec[0].ctl.nchunks;
   const GateSmem m = gate_smem(smem, P.kc, P.dir_words, nullptr, &s_oom, s_np);
@@ -427,9 +431,11 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : CTAS)
         __syncthreads();
         const bool done = s_swapped != 0;
         __syncthreads();  // the flag is read before the next item sets it
-        if (done) continue;
-        const unsigned long long c0 = item_chunk(L, item) | L.hi_vals;
-        if (!run_item<VPT>(P, s_rec, b, job, k, 1, c0, c0 | L.pair_bit, true, S, false, m, st, s_sums)) break;
+        if (!done) {
+          const unsigned long long c0 = item_chunk(L, item) | L.hi_vals;
+          if (!run_item<VPT>(P, s_rec, b, job, k, 1, c0, c0 | L.pair_bit, true, S, false, m, st, s_sums)) break;
+        }
+        if (threadIdx.x == 0 && item + (unsigned)job.ctas < swaps) atomicAdd(&ctl->run_progress, 1u);
       }
     } else {
       bool reload = false;
@@ -438,6 +444,7 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : CTAS)
         const unsigned long long c0 = ((item & ~low) << 1) | (item & low);
         if (!run_item<VPT>(P, s_rec, b, job, k, G, c0, c0 | bit, nchunks > 1ull, S, reload, m, st, s_sums)) break;
         reload = G > 2;  // the first record's buffer has held others
+        if (threadIdx.x == 0 && it + (unsigned)job.ctas < items) atomicAdd(&ctl->run_progress, 1u);
       }
     }
     cp_async_wait_all();
@@ -495,15 +502,21 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : CTAS)
       __syncthreads();
     } else if (!end) {
       if (threadIdx.x == 0) {
-        uint32_t it = 0;
-        while (*(volatile unsigned int*)&ctl->run_gate != steps) {
-          if (++it > kRunSpins) {
-            atomicOr(&ctl->err, (unsigned)E_TIMEOUT);
-            atomicExch(&ctl->timeout_site, 4u);
-            break;
-          }
+        auto moved = [&]() { return *(volatile unsigned int*)&ctl->run_arrived + *(volatile unsigned int*)&ctl->run_progress; };
+        uint32_t it = 0, seen = moved();
+        bool late = false;
+        while (!late && *(volatile unsigned int*)&ctl->run_gate != steps) {
+          if (++it <= job.polls) continue;
+          const uint32_t now = moved();
+          late = now == seen;
+          seen = now;
+          it = 0;
         }
-        s_late = it > kRunSpins;
+        if (late) {
+          atomicOr(&ctl->err, (unsigned)E_TIMEOUT);
+          atomicExch(&ctl->timeout_site, 4u);
+        }
+        s_late = late;
         __threadfence();
       }
       __syncthreads();

@@ -204,3 +204,62 @@ def test_batch_with_large_states_among_small_ones():
         assert batch[0].stats()["graph_replays"] == replay
         for s in batch:
             s.reset()
+
+
+def test_uneven_step_on_two_thread_blocks_outlasts_no_wait():
+    """A lossless circuit on two thread blocks (as many circuits as leave each two share the
+    chip) whose lowest chunk qubit stays |0>: the pairs of chunks of the top qubit go to the
+    blocks in turn, so one of them has every chunk that is not zero and works for seconds on
+    the step of 32 gates that begins with H on that qubit, while the other waits for it.
+    The circuit ends as it does alone."""
+    import torch
+
+    n, kc = 27, 11
+    count = torch.cuda.get_device_properties(0).multi_processor_count // 2
+    rng = np.random.default_rng(4)
+    some = [Cc.gate(int(rng.integers(0, kc)), [Cc.SX, Cc.SY, Cc.rx(0.3), Cc.ry(0.4), Cc.T][int(rng.integers(5))]) for _ in range(40)]
+    spread = [Cc.gate(q, Cc.H) for q in range(n) if q != kc]
+    wide = Cc.to_array(spread + some)
+    # the others count as much work but hold a single chunk that is not zero
+    narrow = Cc.to_array([Cc.gate(q % kc, Cc.H) for q in range(len(spread))] + some)
+    raw = 16 << n
+
+    def make27(pool):
+        return qc().Sim(n, kc, 0.0, chunk_log2=kc, budget=2 * raw, pool_bytes=pool)
+
+    batch = [make27(raw * 9 // 16 + (32 << 20))] + [make27(8 << 20) for _ in range(count - 1)]
+    qc().batch_apply(batch, [wide] + [narrow] * (count - 1), use_graph=False)
+    a, b = (torch.empty(2 << n, dtype=torch.float64, device="cuda") for _ in range(2))
+    for circuit, got in ((wide, batch[0]), (narrow, batch[-1])):
+        solo = make27(raw * 9 // 16 + (32 << 20))
+        solo.apply_circuit(circuit)
+        got.amplitudes(0, 1 << n, out=a)
+        solo.amplitudes(0, 1 << n, out=b)
+        assert torch.equal(a.view(torch.int64), b.view(torch.int64))
+        for key in ("gates", "encoded_bytes", "max_encoded_bytes", "chunks_by_mode", "amp_updates"):
+            assert got.stats()[key] == solo.stats()[key], key
+
+
+@pytest.mark.parametrize("batched", [False, True])
+def test_wait_that_sees_no_progress_returns_an_error(batched):
+    """wait_polls 1: the blocks that have only zero chunks look twice, find that nothing has
+    moved (the one chunk that is not zero takes longer) and give up.  The call returns
+    SIM_ERR_TIMEOUT, the handle refuses further work, others go on."""
+    n, kc = 14, 8
+    gates = Cc.to_array([Cc.gate(q % kc, Cc.SX) for q in range(40)] + [Cc.gate(n - 1, Cc.H)] * 40)
+    s = make(n, kc, 0.0)
+    with pytest.raises(qc().SimError):
+        s.set_option("wait_polls", 0)
+    s.set_option("wait_polls", 1)
+    with pytest.raises(qc().SimError) as ei:
+        if batched:
+            qc().batch_apply([s, make(n, kc, 0.0)], [gates, gates])
+        else:
+            s.apply_circuit(gates)
+    assert ei.value.code == qc().ERR_TIMEOUT
+    with pytest.raises(qc().SimError) as ei:
+        s.apply_circuit(gates)
+    assert ei.value.code == qc().ERR_STATE
+    other = make(n, kc, 0.0)
+    other.apply_circuit(gates)
+    assert other.stats()["gates"] == len(gates)
