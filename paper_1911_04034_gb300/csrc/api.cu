@@ -801,12 +801,13 @@ static sim_status enqueue_gate(sim* s, const sim_gate* g) {
     s->kernel_launches += 1;
   }
   CK(qc::launch_gate(L, grid, s->st), "gate kernel launch");
-  s->kernel_launches += 2;  // with the post kernel below
+  s->kernel_launches += 1;
   if (s->timing) {
     CK(cudaEventRecord(e1, s->st), "event record");
     s->ev_pending.emplace_back(e0, e1);
   }
   CK(qc::launch_post(s->P, L.ctl, grid, s->st), "post kernel launch");
+  s->kernel_launches += 1;
   if (s->timing) {
     // the traffic counters after this gate, for the per-launch figures of sim_timing_launches
     const size_t k = s->ev_pending.size() - 1;
@@ -896,8 +897,9 @@ static sim_status group_circuit(sim* s, const sim_gate* gates, size_t n) {
       } else {
         fill_group(s, gates + i + k, s->h_run + k, G);
         CK(qc::launch_group(G, s->group_grid, s->st), "gate group kernel launch");
+        s->kernel_launches += 1;
         CK(qc::launch_run(s->d_run_jobs + jobs++, 1, s->kc, s->rest_grid, false, s->st), "circuit kernel launch");
-        s->kernel_launches += 2;
+        s->kernel_launches += 1;
         for (int q = 0; q < len; ++q) s->amp_updates += s->h_run[k + q].nact << s->kc;
       }
       k += (size_t)len;
@@ -908,12 +910,20 @@ static sim_status group_circuit(sim* s, const sim_gate* gates, size_t n) {
   return SIM_OK;
 }
 
+// A call that failed after launches of its own has left its gates half applied: the handle is
+// finished (`launches`: the count when the call began).
+static sim_status applied(sim* s, uint64_t launches, sim_status r) {
+  if (r != SIM_OK && s->kernel_launches != launches && s->poisoned == SIM_OK) s->poisoned = SIM_ERR_CUDA;
+  return r;
+}
+
 sim_status sim_apply_gate(sim_t* s, const sim_gate* g) {
   if (!s || !g) return fail(SIM_ERR_INVALID, "NULL argument");
   if (sim_status r = s->guard()) return r;
   std::string why;
   if (!gate_ok(g, s->n, &why)) return fail(SIM_ERR_INVALID, "invalid gate: %s", why.c_str());
-  return enqueue_gate(s, g);
+  const uint64_t launches = s->kernel_launches;
+  return applied(s, launches, enqueue_gate(s, g));
 }
 
 sim_status sim_apply_circuit(sim_t* s, const sim_gate* gates, size_t n_gates) {
@@ -922,15 +932,16 @@ sim_status sim_apply_circuit(sim_t* s, const sim_gate* gates, size_t n_gates) {
   std::string why;
   for (size_t k = 0; k < n_gates; ++k)
     if (!gate_ok(gates + k, s->n, &why)) return fail(SIM_ERR_INVALID, "invalid gate %zu: %s", k, why.c_str());
+  const uint64_t launches = s->kernel_launches;
   bool ran = false;
   if (run_applies(s) && n_gates)
-    if (sim_status r = run_circuit(s, gates, n_gates, &ran)) return r;
+    if (sim_status r = run_circuit(s, gates, n_gates, &ran)) return applied(s, launches, r);
   if (!ran && n_gates > 1 && group_applies(s)) {
-    if (sim_status r = group_circuit(s, gates, n_gates)) return r;
+    if (sim_status r = group_circuit(s, gates, n_gates)) return applied(s, launches, r);
     ran = true;
   }
   for (size_t k = 0; k < n_gates && !ran; ++k)
-    if (sim_status r = enqueue_gate(s, gates + k)) return r;
+    if (sim_status r = enqueue_gate(s, gates + k)) return applied(s, launches, r);
   return s->check_device();
 }
 
@@ -1370,7 +1381,8 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
       for (int k : large) {
         const cudaStream_t own = sims[k]->st;
         sims[k]->st = st;  // launches go to sims[0]'s stream
-        sim_status r = group_circuit(sims[k], circuits[k], n_gates[k]);
+        const uint64_t launches = sims[k]->kernel_launches;
+        sim_status r = applied(sims[k], launches, group_circuit(sims[k], circuits[k], n_gates[k]));
         if (r == SIM_OK) r = sims[k]->check_device();
         sims[k]->st = own;
         if (r != SIM_OK && worst == SIM_OK) worst = r;
