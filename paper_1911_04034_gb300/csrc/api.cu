@@ -134,6 +134,8 @@ void qc::set_last_error(const char* msg) { g_last_error = msg; }
 // Largest state (in chunks) that k_run takes in several rounds: after a step one CTA returns the
 // freed pages (up to 33 a chunk of 2^10 amplitudes) while the others wait.
 constexpr uint64_t kRunChunks = 1ull << 18;
+constexpr size_t kRunBlock = 4096;     // gate records staged at once
+constexpr size_t kRunSegments = 64;    // launches they make at most
 
 struct sim {
   int n = 0, b = 0, kc = 0, ladder = 0;
@@ -179,6 +181,7 @@ struct sim {
   // the graph of the last sim_batch_apply call this handle led, kept for replay
   cudaGraphExec_t bexec = nullptr;
   void* bjobs = nullptr;             // its job list (device)
+  size_t bjobs_bytes = 0;
   std::vector<uint8_t> bkey;         // what its launches depend on
   std::vector<uint64_t> bupd;        // the amplitude updates it makes, per handle
   uint64_t uid = 0;                  // creation number (never reused)
@@ -191,6 +194,7 @@ struct sim {
     cudaFree(bjobs);
     bexec = nullptr;
     bjobs = nullptr;
+    bjobs_bytes = 0;
     bkey.clear();
     bupd.clear();
   }
@@ -233,6 +237,17 @@ struct sim {
     cudaFree(d_ctl);
     cudaFree(d_counts);
     cudaFree(d_scratch);
+  }
+
+  // Device memory allocated beyond what the handle was created with.
+  uint64_t later_bytes() const {
+    uint64_t b = scratch_bytes + bjobs_bytes + tlog_cap * 2 * sizeof(unsigned long long);
+    if (run_cap) b += run_cap * sizeof(GateLaunch) + (run_cap + kRunSegments) * sizeof(qc::RunJob);
+    if (d_mlp) b += qc::kMlpParams * 2;
+    if (d_dec) b += nchunks + 16;
+    if (d_trace) b += trace_cap * qc::kTraceFloats * sizeof(float);
+    if (d_bc) b += (uint64_t)qc::kBcLines * qc::bc_line_bytes(qc::round16(qc::max_image_bytes(kc)));
+    return b;
   }
 
   sim_status scratch(size_t bytes) {
@@ -714,8 +729,6 @@ static std::vector<int> run_shares(const std::vector<const GateLaunch*>& first, 
   return c;
 }
 
-constexpr size_t kRunBlock = 4096;     // gate records staged at once
-constexpr size_t kRunSegments = 64;    // launches they make at most
 // The staging buffers for a circuit of n gates; false: no memory for them.
 static bool run_stage(sim* s, size_t n) {
   const size_t want = n < kRunBlock ? n : kRunBlock;
@@ -1291,7 +1304,7 @@ sim_status sim_stats(sim_t* s, sim_stats_t* o) {
   o->pool_bytes = s->npages * qc::kPage;
   o->pages_in_use_bytes = (s->npages - (uint64_t)h.top - h.wc_pages) * qc::kPage;  // pages holding images
   o->peak_pages_bytes = h.peak_pages * qc::kPage;
-  o->device_bytes = s->device_bytes + s->scratch_bytes;
+  o->device_bytes = s->device_bytes + s->later_bytes();
   o->amp_updates = s->amp_updates;
   o->ratio = h.E ? (double)o->raw_bytes / (double)h.E : 0.0;
   o->min_ratio = h.Emax ? (double)o->raw_bytes / (double)h.Emax : 0.0;
@@ -1535,6 +1548,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
       // kept for the next call with the same key (the job list stays with it)
       lead->bexec = exec;
       lead->bjobs = d_jobs;
+      lead->bjobs_bytes = whole ? run_list.size() : jobs.size() * sizeof(qc::BatchJob);
       lead->bkey.swap(key);
       lead->bupd = upd;
     } else {

@@ -71,3 +71,27 @@ def test_call_that_fails_halfway_poisons_its_handle(run, n, how):
         assert code(s.apply_circuit, gates) == (0 if nth == 1 else q.ERR_STATE), nth
         assert code(other.apply_circuit, Cc.h_all(9)) == 0
     """)
+
+
+def test_device_bytes_is_what_the_handle_allocated(run):
+    """sim_stats_t.device_bytes against the runtime's own count: after creation, a circuit's
+    staged gate records (a small state's and a longer circuit's), a kept batch graph, readout
+    scratch, the block cache, timing, the selector network and training records."""
+    run("""
+    import numpy as np
+    s = make(9)
+    count = C.c_longlong.in_dll(fake, "fake_device_bytes")
+    def check(what):
+        assert s.stats()["device_bytes"] == count.value, (what, s.stats()["device_bytes"], count.value)
+    check("created")
+    s.apply_circuit(Cc.h_all(9)); check("circuit")
+    s.apply_circuit(Cc.rcs_n(9, 40, seed=1)); check("longer circuit")
+    q.batch_apply([s], [Cc.h_all(9)], use_graph=True); check("batch graph")
+    s.amplitudes(0, 4); check("readout")
+    s.set_block_cache(True); check("block cache")
+    s.set_timing(1); check("timing")
+    s.apply_circuit(Cc.h_all(9)); check("timed circuit")
+    s.set_selector(2, np.zeros(1864, dtype=np.uint16)); check("selector")
+    s.trace(100); check("trace")
+    s.trace(0); s.set_block_cache(False); check("given back")
+    """)
