@@ -11,7 +11,8 @@
 enum { kOps = 1 << 20, kNames = 4096 };
 
 /* what the test reads and sets */
-API char fake_log[kOps];      /* one letter per operation: L launch, R event record, W event wait, S stream or device wait */
+API char fake_log[kOps];      /* one letter per operation: L launch, S stream or device wait, W wait for an event
+                                * with nothing launched after it, w the same with launches after it */
 API int fake_ops = 0;
 API int fake_launches = 0;
 API int fake_fail_launch = 0; /* this launch (counted from 1) fails */
@@ -127,11 +128,11 @@ API cudaError_t cudaStreamSynchronize(cudaStream_t s) { (void)s; op('S'); return
 API cudaError_t cudaStreamWaitEvent(cudaStream_t s, cudaEvent_t e, unsigned f) { (void)s; (void)e; (void)f; return cudaSuccess; }
 API cudaError_t cudaStreamBeginCapture(cudaStream_t s, enum cudaStreamCaptureMode m) { (void)s; (void)m; return cudaSuccess; }
 API cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t* g) { (void)s; *g = (cudaGraph_t)malloc(1); return cudaSuccess; }
-API cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned f) { (void)f; *e = (cudaEvent_t)malloc(1); return cudaSuccess; }
+API cudaError_t cudaEventCreateWithFlags(cudaEvent_t* e, unsigned f) { (void)f; *e = (cudaEvent_t)calloc(1, sizeof(int)); return cudaSuccess; }
 API cudaError_t cudaEventCreate(cudaEvent_t* e) { return cudaEventCreateWithFlags(e, 0); }
 API cudaError_t cudaEventDestroy(cudaEvent_t e) { free(e); return cudaSuccess; }
-API cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { (void)e; (void)s; op('R'); return cudaSuccess; }
-API cudaError_t cudaEventSynchronize(cudaEvent_t e) { (void)e; op('W'); return cudaSuccess; }
+API cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { (void)s; *(int*)e = fake_launches; return cudaSuccess; }
+API cudaError_t cudaEventSynchronize(cudaEvent_t e) { op(*(int*)e == fake_launches ? 'W' : 'w'); return cudaSuccess; }
 API cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t a, cudaEvent_t b) { (void)a; (void)b; *ms = 1.0f; return cudaSuccess; }
 API cudaError_t cudaGraphInstantiate(cudaGraphExec_t* x, cudaGraph_t g, unsigned long long f) { (void)g; (void)f; *x = (cudaGraphExec_t)malloc(1); return cudaSuccess; }
 API cudaError_t cudaGraphLaunch(cudaGraphExec_t x, cudaStream_t s) { (void)x; (void)s; return cudaSuccess; }

@@ -73,6 +73,21 @@ def test_call_that_fails_halfway_poisons_its_handle(run, n, how):
     """)
 
 
+def test_looking_for_the_settled_bound_keeps_the_queue_full(run):
+    """A large lossy state whose bound never settles: apart from the first look the host never
+    waits for gates it enqueued last, until it synchronises at the end of the call."""
+    run("""
+    gates = Cc.rcs_n(12, 20, seed=1)
+    s = make(12)
+    start = num("fake_ops").value
+    s.apply_circuit(gates)
+    ops = log()[start:]
+    assert ops.count("L") >= 2 * len(gates) > 400
+    assert ops.count("W") + ops.count("S") <= 2 and ops.rstrip("S").count("S") == 0, ops
+    assert ops.count("w") >= len(gates) // 8
+    """)
+
+
 def test_device_bytes_is_what_the_handle_allocated(run):
     """sim_stats_t.device_bytes against the runtime's own count: after creation, a circuit's
     staged gate records (a small state's and a longer circuit's), a kept batch graph, readout
