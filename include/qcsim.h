@@ -193,9 +193,9 @@ sim_status sim_batch_run(int n_circ, const int* n_qubits, const sim_gate* const*
                          double err_bound, sim_stats_t* out);
 
 /* Chunk-size autotuner: for each candidate chunk_log2, creates a handle (budget raw/4,
- * pool raw + 1/8), applies the first half of the probe circuit, then times the fused
- * kernel over the second half; *best receives the candidate with the most amplitude
- * updates per second of kernel time, rates[i] (if not NULL) each candidate's rate. */
+ * pool raw + 1/8), applies the first half of the probe circuit, then times the
+ * sim_apply_circuit call of the second half; *best receives the candidate with the most
+ * amplitude updates per second of it, rates[i] (if not NULL) each candidate's rate. */
 sim_status sim_autotune_chunk(int n_qubits, int block_log2, double err_bound, const sim_gate* probe, size_t n_probe,
                               const int* candidates, int n_candidates, int* best, double* rates);
 
@@ -205,7 +205,7 @@ typedef struct {
   int32_t chunk_log2;      /* the coding tile: 2^chunk_log2 amplitudes decoded and encoded as one unit */
   int32_t ladder;          /* codec schedule: bound ladder 0 jump, 1 the paper's ladder, 2 guarded */
   uint32_t modes;          /* codec schedule: the chunk modes the encoder may choose */
-  double rate;             /* amplitude updates per second of gate-kernel time over the probe's second half */
+  double rate;             /* amplitude updates per second over the probe's second half, one sim_apply_circuit */
   double ratio;            /* raw bytes over the peak encoded bytes of the probe run */
   double fidelity_lb_sum;  /* the probe run's provable fidelity bound */
 } sim_tune_point;
@@ -215,7 +215,7 @@ typedef struct {
  * ladders and the mode sets with the other settings at their best so far, until a
  * sweep changes nothing (3 sweeps at most).  Each point is measured as in
  * sim_autotune_chunk: a fresh handle (budget raw/4, pool raw + 1/8 + 64 MiB) runs the
- * first half of the probe, then the second half with gate-kernel timing; the best
+ * first half of the probe, then the timed call of the second half; the best
  * point has the highest rate (every point keeps the bound err_bound).  Blocks clamp to
  * n_qubits and chunks to the block, as sim_create_ex does; points that coincide after
  * clamping are measured once.  *best receives the winner; tried (cap_tried entries,

@@ -88,6 +88,22 @@ def test_looking_for_the_settled_bound_keeps_the_queue_full(run):
     """)
 
 
+def test_autotuner_times_the_call_that_is_made(run):
+    """A probe on a small state runs whole-circuit launches in both halves, as
+    sim_apply_circuit does, and no gate kernel of its own per gate."""
+    run("""
+    probe = Cc.rcs_n(9, 6, seed=1)
+    s = make(9)
+    a = fake.fake_count(b"k_run")
+    s.apply_circuit(probe[: len(probe) // 2]); s.apply_circuit(probe[len(probe) // 2:])
+    per_point = fake.fake_count(b"k_run") - a
+    a = fake.fake_count(b"k_run")
+    best, rates = q.autotune_chunk(9, 8, 1e-4, probe, candidates=(7, 8))
+    assert all(r > 0 for r in rates.values()) and best in rates
+    assert fake.fake_count(b"k_run") - a == 2 * per_point and fake.fake_count(b"k_gate") == 0
+    """)
+
+
 def test_device_bytes_is_what_the_handle_allocated(run):
     """sim_stats_t.device_bytes against the runtime's own count: after creation, a circuit's
     staged gate records (a small state's and a longer circuit's), a kept batch graph, readout
