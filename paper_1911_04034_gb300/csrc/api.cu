@@ -121,6 +121,17 @@ GateCoef coef_of(const sim_gate* g) {
 
 int popcount64(uint64_t x) { return __builtin_popcountll(x); }
 
+// True if every coefficient part of a 2x2 matrix (eight doubles) is +-2^k, -10 <= k <= 0 (the
+// range in which pow2_pair's scaling is exact); *sk = k.
+bool pow2_parts(const double* u, int* sk) {
+  int e = 0;
+  if (u[0] == 0.0 || std::fabs(std::frexp(u[0], &e)) != 0.5 || e < -9 || e > 1) return false;
+  for (int k = 1; k < 8; ++k)
+    if (std::fabs(u[k]) != std::fabs(u[0])) return false;
+  *sk = e - 1;
+  return true;
+}
+
 int device_sms() {
   int dev = 0, sms = 0;
   cudaGetDevice(&dev);
@@ -568,20 +579,15 @@ static GateLaunch make_launch(sim* s, const sim_gate* g) {
     const bool diag = u[2] == 0 && u[3] == 0 && u[4] == 0 && u[5] == 0;
     const bool perm = u[0] == 0 && u[1] == 0 && u[6] == 0 && u[7] == 0;
     L.gfeat = (real ? 1u : 0u) | (diag ? 2u : 0u) | (perm ? 4u : 0u) | (t < kc ? 8u : 0u);
-    // a cross-chunk diagonal gate with a row that is an exact copy: the row that is not
     L.diag = diag ? 1 : 0;
-    int e = 0;
-    L.pow2 = u[0] != 0.0 && std::fabs(std::frexp(u[0], &e)) == 0.5 && e >= -9 && e <= 1 ? 1 : 0;
-    for (int k = 1; k < 8; ++k)
-      if (std::fabs(u[k]) != std::fabs(u[0])) L.pow2 = 0;
+    L.pow2 = pow2_parts(u, &L.sk) ? 1 : 0;
     if (L.pow2) {
-      L.sk = e - 1;
       for (int q = 0; q < 16; ++q)
         if (L.g.c[q] < 0.0) L.sgn |= 1u << q;
     }
     L.copy = diag ? (u[0] == 1.0 && u[1] == 0.0 ? 1u : 0u) | (u[6] == 1.0 && u[7] == 0.0 ? 2u : 0u) : 0u;
-    L.solo = -1;
-    if (t >= kc && diag) L.solo = u[0] == 1.0 && u[1] == 0.0 ? 1 : (u[6] == 1.0 && u[7] == 0.0 ? 0 : -1);
+    // a cross-chunk diagonal gate with a row that is an exact copy: the row that is not
+    L.solo = t >= kc ? ((L.copy & 1u) ? 1 : ((L.copy & 2u) ? 0 : -1)) : -1;
     // a coefficient that can turn a normal value into a subnormal (see next_level)
     L.ctl.wide_gate = 0;
     for (int k = 0; k < 8; ++k)
@@ -2229,7 +2235,7 @@ static void sv_group(int n, const sim_gate* gates, const uint8_t* form, size_t c
     const bool z01 = u[2] == 0.0 && u[3] == 0.0, z10 = u[4] == 0.0 && u[5] == 0.0;
     g.copy = (u[0] == 1.0 && u[1] == 0.0 && z01 ? 1u : 0u) | (u[6] == 1.0 && u[7] == 0.0 && z10 ? 2u : 0u);
     if (form[k] == 1) {
-      g.sk = std::ilogb(u[0]);
+      pow2_parts(u, &g.sk);
       for (int q = 0; q < 16; ++q)
         if (g.g.c[q] < 0.0) g.sgn |= 1u << q;
     }
@@ -2278,13 +2284,11 @@ sim_status sim_sv_apply_circuit(sim_sv_t* v, const sim_gate* gates, size_t n_gat
     const double* u = gates[k].u;
     const bool diag = u[2] == 0.0 && u[3] == 0.0 && u[4] == 0.0 && u[5] == 0.0;
     if (diag && u[0] == 1.0 && u[1] == 0.0 && u[6] == 1.0 && u[7] == 0.0) continue;  // the identity
-    int e = 0;
-    bool pow2 = u[0] != 0.0 && std::fabs(std::frexp(u[0], &e)) == 0.5 && e >= -9 && e <= 1;
-    for (int q = 1; q < 8 && pow2; ++q) pow2 = std::fabs(u[q]) == std::fabs(u[0]);
     const uint64_t bit = !diag && gates[k].target >= L ? 1ull << gates[k].target : 0ull;
     if (count == (size_t)qc::kSvMaxGates || popcount64(high | bit) > T - L) CK(flush(), "state vector gates");
     high |= bit;
-    form[count] = diag ? 2 : (pow2 ? 1 : 0);
+    int sk = 0;
+    form[count] = diag ? 2 : (pow2_parts(u, &sk) ? 1 : 0);
     run[count++] = gates[k];
   }
   CK(flush(), "state vector gates");
