@@ -230,7 +230,7 @@ def group_circuit(n, kc, seed):
     return Cc.to_array(g)
 
 
-@pytest.mark.parametrize("kc,n", [(7, 17), (8, 18), (9, 19), (11, 20)])
+@pytest.mark.parametrize("kc,n", [(7, 17), (8, 18), (9, 19), (10, 20), (11, 20)])
 def test_groups_of_gates_on_larger_states(kc, n):
     """States of more chunk pairs than one round of a whole-circuit launch (lossless ones run
     by it all the same): once the bound is settled, groups of gates per pass (pairs of chunks that leave the STREAM form on the way
