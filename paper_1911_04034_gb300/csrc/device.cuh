@@ -94,7 +94,9 @@ struct DevCtl {
   unsigned int fast_pad;
   unsigned long long fast_items;       // work items the streaming kernel committed (cumulative)
   unsigned long long fast_deferred;    // work items it left to the general kernel (cumulative)
-  unsigned int timeout_site;           // where a bounded wait gave up (E_TIMEOUT): 1 item start, 2 pass, 3 item end, 4 between gates (k_run)
+  unsigned int timeout_site;           // where a bounded wait gave up (E_TIMEOUT): streaming kernel 1 item start, 2 pass, 3 item
+                                       // end; k_run 4 between steps; k_group 5 item start, 6 and 7 before and after a
+                                       // cross-chunk gate, 8 item end
   unsigned int timeout_pad;
   unsigned long long wc_pages;         // free pages the streaming kernel's warps keep in their caches
   unsigned long long palette_trials;   // chunk encodes that ran the PALETTE trial

@@ -56,8 +56,8 @@ __device__ __forceinline__ bool image_stands(const Pool& P, unsigned long long c
 // product is exact, so a chain of four equals 2^k times the chain of the signed inputs in
 // the same order while no partial sum leaves the normal range.  The first sums of the four
 // chains are +-(ar + ai) and +-(ar - ai), so two additions serve all four: 10 instead of
-// 16 FP64 operations.  False (nothing done) if an input is nonzero below 2^-959 or above
-// 2^1020: inputs of at least 2^-959 are multiples of 2^-1011, so a nonzero sum times 2^k
+// 16 FP64 operations.  False (nothing done) if an input is nonzero below 2^-959 or at least
+// 2^1021: inputs of at least 2^-959 are multiples of 2^-1011, so a nonzero sum times 2^k
 // (k >= -10) stays normal, and no sum overflows.
 __device__ __forceinline__ bool pow2_pair(uint32_t sgn, int sk, double2& a, double2& b) {
   auto bad = [](double v) {

@@ -11,14 +11,15 @@
 //
 // Bound: instructions, about a third as many per value for a gate in the middle of a group
 // (load, gate, truncation, length of the codes) as for one by itself.
-// 2^10-amplitude chunks, 1e-4: a 30-qubit random-circuit layer 517 -> 434 ms, a 26-qubit
-// QAOA round 104 -> 71.5 ms; 21 qubits in 2^9, two layers 3.16 -> 1.76 ms.
+// Gate by gate -> by groups, 2^10-amplitude chunks, 1e-4: a 30-qubit random-circuit layer 490
+// -> 348 ms, a 26-qubit QAOA round 96 -> 65 ms; 21 qubits in 2^9, two layers 2.95 -> 1.56 ms.
 #include "stream.cuh"
 
 namespace qc {
 
 constexpr int kGroupWarps = 4;  // two pairs; 20 warps an SM with 2^10-amplitude chunks (43 KB a CTA)
 constexpr int kGroupPairs = kGroupWarps / 2;
+static_assert(kRunGroup <= 32, "a lane and a mask bit per gate of a group");
 
 // Per warp: its chunk's high words, what is known of each pass of it (see group_note), two
 // windows (the first also the output window), input and output page ids, its page cache.

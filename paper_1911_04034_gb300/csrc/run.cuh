@@ -370,7 +370,7 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : CTAS)
   __shared__ uint32_t s_cache_n;
   __shared__ CtaAcc s_acc;
   static_assert(sizeof(GateLaunch) % 16 == 0, "gate records are copied in 16-byte units");
-  static_assert(sizeof(RunSums) == 3u * 8u * kRunGroup && 3 * kRunGroup <= kThreads, "one thread per sum");
+  static_assert(sizeof(RunSums) == 3u * 8u * kRunGroup && 3 * kRunGroup <= kThreads - 32, "a thread per sum beside warp 0");
   int lo = 0, hi = njobs - 1;  // the job of this CTA
   while (lo < hi) {
     const int mid = (lo + hi + 1) >> 1;
