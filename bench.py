@@ -8,12 +8,14 @@ blocks of 2^20 amplitudes (chunks of 2^10), lossless first and lossy at pointwis
 relative bound 1e-4 once the state passes 90 % of the budget (raw/4).  Synthetic,
 seeded circuits; the compressed state (several GB) is larger than L2, so no flush.
 
-One step = one circuit layer (about 42 gates) on the evolving compressed state: every
-gate runs the whole path (classify, decode, apply, controller, truncate, XOR-code,
-mode select, page commit, stats).  Warm-up steps are the first layers after the
+One step = one circuit layer (about 42 gates) on the evolving compressed state, one
+sim_apply_circuit: groups of gates share a pass over the state (decode, apply, truncate
+and count bytes after every gate, XOR-code, page commit), every other gate runs the
+whole path by itself.  Warm-up steps are the first layers after the
 Hadamard layer; timed steps follow.  `value` is device-timed (CUDA events on the
 simulator's stream); `e2e` times the same calls from the host, including the
-per-step read-back of the statistics.  Fidelity is measured against the uncompressed
+per-step read-back of the statistics.  `gate_by_gate` times every gate of a few further
+layers by itself (sim_set_timing, which leaves groups out), by gate class.  Fidelity is measured against the uncompressed
 complex128 state vector run on the same GPU (same gates).
 
 --impl reference times the CPU oracle (tests' reference implementation) on a
@@ -44,8 +46,8 @@ METRIC = "compressed-state amplitude updates/s"
 UNIT = "amp-updates/s"
 ROWS, COLS, BLOCK_LOG2, CHUNK_LOG2, SEED = 5, 6, 20, 10, 2024  # defaults; --rows/--cols override
 
-# DRAM traffic of a gate's launches from the last ncu capture, with the hash of the kernel
-# sources it applies to.  A 30-qubit launch is too large to capture, so the capture ran the
+# DRAM traffic of a gate's launches (gate by gate) from the last ncu capture, with the hash of
+# the kernel sources it applies to.  A 30-qubit launch is too large to capture, so the capture ran the
 # 26-qubit 2 x 13 grid in its steady state (k_gate_fast launches 801-804, every item on the
 # streaming kernel): dram__bytes_read.sum + dram__bytes_write.sum = 832 MB per launch
 # against 860.5 MB of image bytes per gate, a ratio of 0.968 (reads 447 MB: the input
@@ -58,7 +60,8 @@ NCU_TRAFFIC = {"ratio_to_image_bytes": 0.968, "source_sha": "4880ea788b2bc48a"}
 def kernel_sha() -> str:
     h = hashlib.sha256()
     for f in ("paper_1911_04034_gb300/csrc/fast.cu", "paper_1911_04034_gb300/csrc/kernels.cu",
-              "paper_1911_04034_gb300/csrc/gate_common.cuh", "paper_1911_04034_gb300/csrc/device.cuh"):
+              "paper_1911_04034_gb300/csrc/gate_common.cuh", "paper_1911_04034_gb300/csrc/gate_item.cuh",
+              "paper_1911_04034_gb300/csrc/stream.cuh", "paper_1911_04034_gb300/csrc/device.cuh"):
         h.update(open(os.path.join(ROOT, f), "rb").read())
     return h.hexdigest()[:16]
 
@@ -268,8 +271,10 @@ def run_gpu(args) -> dict | None:
 
         dist.init_process_group("nccl")
     n = ROWS * COLS
-    # the depth-20 circuit, then further layers of the same family for the timed steps
-    depth = CFG2_DEPTH + args.warmup + 2 * args.steps
+    # the depth-20 circuit, then further layers of the same family for the timed steps, the
+    # end-to-end steps and the gates timed one by one
+    class_layers = min(args.steps, 4)
+    depth = CFG2_DEPTH + args.warmup + 2 * args.steps + class_layers
     gates = Cc.rcs(ROWS, COLS, depth, seed=replica_seed(rank))
     layers = layers_of(gates, n, depth)
     d20 = np.concatenate(layers[: 1 + CFG2_DEPTH])
@@ -313,7 +318,7 @@ def run_gpu(args) -> dict | None:
     t_first = 1 + CFG2_DEPTH + args.warmup
     timed = layers[t_first: t_first + args.steps]
     clocks = Clocks(local)
-    sim.set_timing(2 if args.phases else 1)
+    sim.timing()  # the traffic counters from here
     barrier()
     clocks.start()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -325,14 +330,13 @@ def run_gpu(args) -> dict | None:
     barrier()
     clk = clocks.stop()
     ms = ev0.elapsed_time(ev1)
-    tl = sim.timing_launches()
-    tm = sim.timing()
-    sim.set_timing(False)
+    moved = sim.timing()
     st1 = sim.stats()
     updates = st1["amp_updates"] - st0["amp_updates"]
     assert updates == amp_updates(np.concatenate(timed), n, kc)
     # end to end through the public API: host gate records in, statistics read back
     e2e_layers = layers[t_first + args.steps: t_first + 2 * args.steps]
+    class_gates = np.concatenate(layers[t_first + 2 * args.steps:])
     barrier()
     t0 = time.perf_counter()
     h2d = d2h = 0
@@ -345,6 +349,13 @@ def run_gpu(args) -> dict | None:
     e2e_s = time.perf_counter() - t0
     e2e_updates = amp_updates(np.concatenate(e2e_layers), n, kc)
     st2 = sim.stats()
+    # every gate by itself
+    sim.set_timing(2 if args.phases else 1)
+    sim.apply_circuit(class_gates)
+    tl = sim.timing_launches()
+    tm = sim.timing()
+    sim.set_timing(False)
+    st3 = sim.stats()
     sim.close()
     # the bound sweep of the configuration: the depth-20 circuit at 1e-5 and 1e-3 (and
     # 1e-4 above), each from |0...0> with its fidelity against the same state vector
@@ -365,11 +376,14 @@ def run_gpu(args) -> dict | None:
                        "note": "the timed simulator itself at depth 20"}
     pk = peaks()
     hbm = pk.get("hbm_gbs")
-    kernel_ms_avg = tm["gate_kernel_ms"] / max(1, tm["launches"])
-    bytes_per_launch = (tm["bytes_read"] + tm["bytes_written"]) / max(1, tm["launches"])
-    achieved = bytes_per_launch / (kernel_ms_avg * 1e-3) / 1e9 if kernel_ms_avg > 0 else 0.0
-    traffic = (NCU_TRAFFIC["ratio_to_image_bytes"] * bytes_per_launch
-               if NCU_TRAFFIC["source_sha"] == kernel_sha() else None)
+    launches = st1["kernel_launches"] - st0["kernel_launches"]
+    kernel_ms_avg = ms / max(1, launches)
+    bytes_per_launch = (moved["bytes_read"] + moved["bytes_written"]) / max(1, launches)
+    achieved = bytes_per_launch / (kernel_ms_avg * 1e-3) / 1e9
+    gate_ms = tm["gate_kernel_ms"] / max(1, tm["launches"])
+    gate_bytes = (tm["bytes_read"] + tm["bytes_written"]) / max(1, tm["launches"])
+    gate_traffic = (NCU_TRAFFIC["ratio_to_image_bytes"] * gate_bytes
+                    if NCU_TRAFFIC["source_sha"] == kernel_sha() else None)
     flops = fp64_flops(np.concatenate(timed), n, kc)
     out = {
         "metric": METRIC,
@@ -411,26 +425,35 @@ def run_gpu(args) -> dict | None:
             "peak": hbm,
             "unit": "GB/s",
             "frac": (achieved / hbm) if hbm else None,
-            "traffic": traffic,
-            "kernel": "k_gate_fast + k_gate (one gate's launches)",
+            "traffic": None,
+            "kernel": "k_group + k_run (groups of gates), k_gate_fast + k_gate + k_post (single gates); whole steps over their launches",
             "kernel_ms_avg": kernel_ms_avg,
             "algorithmic_bytes_per_launch": bytes_per_launch,
             "peak_source": "MEASURED_PEAKS.json hbm_gbs (measured)" if hbm else None,
         },
         "roofline_fp64": {
             "bound": "alu",
-            "achieved": flops / (tm["gate_kernel_ms"] * 1e-3) / 1e12,
+            "achieved": flops / (ms * 1e-3) / 1e12,
             "peak": FP64_PEAK_TFLOPS,
             "unit": "TFLOP/s",
-            "frac": flops / (tm["gate_kernel_ms"] * 1e-3) / 1e12 / FP64_PEAK_TFLOPS,
-            "kernel": "k_gate_fast + k_gate",
+            "frac": flops / (ms * 1e-3) / 1e12 / FP64_PEAK_TFLOPS,
+            "kernel": "as above",
             "peak_source": FP64_PEAK_SOURCE,
             "note": "the fused kernels' arithmetic ceiling: dense gates cost 28 flops per amplitude pair",
         },
-        "roofline_by_class": per_class(np.concatenate(timed), tl, n, kc, hbm),
-        "gpu_launches": st1["kernel_launches"] - st0["kernel_launches"],
-        "phase_share": ({k: round(v / max(1, sum(st1["phase_cycles"])), 4) for k, v in
-                         zip(("stage", "decode", "apply", "encode", "commit", "const"), st1["phase_cycles"])}
+        "gate_by_gate": {
+            "note": "every gate by itself (k_gate_fast + k_gate), CUDA events around its kernels",
+            "gates": int(len(class_gates)),
+            "amp_updates_per_s": amp_updates(class_gates, n, kc) / (tm["gate_kernel_ms"] * 1e-3),
+            "kernel_ms_avg": gate_ms,
+            "algorithmic_bytes_per_launch": gate_bytes,
+            "hbm_gbs": gate_bytes / (gate_ms * 1e-3) / 1e9,
+            "traffic": gate_traffic,
+        },
+        "roofline_by_class": per_class(class_gates, tl, n, kc, hbm),
+        "gpu_launches": launches,
+        "phase_share": ({k: round(v / max(1, sum(st3["phase_cycles"])), 4) for k, v in
+                         zip(("stage", "decode", "apply", "encode", "commit", "const"), st3["phase_cycles"])}
                         if args.phases else None),
         "clocks": clk,
         "e2e": {"value": e2e_updates / e2e_s, "unit": UNIT, "h2d_bytes_per_step": h2d // max(1, len(e2e_layers)),
@@ -439,8 +462,8 @@ def run_gpu(args) -> dict | None:
     if not args.no_batch:
         # the batched workload beside the headline: one replayed step after a capture
         bt = run_batch(args, steps=1, warmup=2)
-        out["batch_workload"] = {k: bt[k] for k in ("value", "unit", "ms_per_step", "plain_per_gate_value",
-                                                    "speedup_vs_plain", "graph_replays", "min_fidelity_lb_sum",
+        out["batch_workload"] = {k: bt[k] for k in ("value", "unit", "ms_per_step", "one_by_one_value",
+                                                    "speedup_vs_one_by_one", "graph_replays", "min_fidelity_lb_sum",
                                                     "mean_compression_ratio")}
         out["batch_workload"]["workload"] = bt["config"]["workload"]
         out["batch_workload"]["autotuned"] = bt["autotune"]["best"]
@@ -452,10 +475,10 @@ def run_batch(args, steps: int | None = None, warmup: int | None = None) -> dict
     """256 independent random circuits (qubits uniform in 14..24, depth in 12..24, the
     random-circuit gate set, eps 1e-4).  The autotuner picks block size (2^10..2^16),
     tile (chunk) size and codec schedule (bound ladder, mode set) on a 20-qubit probe;
-    then each step runs the whole batch from |0...0> in one persistent launch per gate
-    step: the first warm-up step captures the CUDA graph, every later step replays it
-    after sim_reset.  Against it: the same circuits on the same handles one after
-    another through the per-gate path.  Wall-clock time of the calls (both synchronise
+    then each step runs the whole batch from |0...0>: circuits on large states one by one
+    in groups of gates, the others together in one launch, which the first warm-up step
+    captures as a CUDA graph and every later step replays after sim_reset.  Against it:
+    the same circuits on the same handles one after another (sim_apply_circuit).  Wall-clock time of the calls (both synchronise
     at the end); the resets between steps are not timed."""
     import torch
 
@@ -497,7 +520,7 @@ def run_batch(args, steps: int | None = None, warmup: int | None = None) -> dict
     def batched():
         qcsim.batch_apply(sims, circuits, use_graph=True)
 
-    def plain():
+    def one_by_one():
         for s_, g in zip(sims, circuits):
             s_.apply_circuit(g)
 
@@ -508,8 +531,8 @@ def run_batch(args, steps: int | None = None, warmup: int | None = None) -> dict
     ratio = [s_.stats()["ratio"] for s_ in sims]
     lb = min(s_.stats()["fidelity_lb_sum"] for s_ in sims)
     upd = sum(s_.stats()["amp_updates"] for s_ in sims)
-    timed(plain, 1)
-    t_plain = timed(plain, steps)
+    timed(one_by_one, 1)
+    t_plain = timed(one_by_one, steps)
     for s_ in sims:
         s_.close()
     assert upd == per_pass, (upd, per_pass)
@@ -517,12 +540,13 @@ def run_batch(args, steps: int | None = None, warmup: int | None = None) -> dict
             "warmup": warmup, "ms_per_step": t_batch / steps * 1e3, "higher_is_better": True, "scaling": "weak",
             "vs_baseline": None, "dtype": "f64", "data": "synthetic",
             "config": {"workload": f"batch of {args.batch} random circuits, 14-24 qubits, depth 12-24, eps {args.eps}, "
-                                   f"one launch per gate step, CUDA graph kept and replayed after sim_reset; "
+                                   f"large states in groups of gates, the others in one launch whose CUDA graph is "
+                                   f"kept and replayed after sim_reset; "
                                    f"blocks 2^{b}, chunks 2^{kc}, ladder {ladder}, modes {modes:#x} (autotuned)",
                        "l2": "no flush: the batch's compressed states exceed L2"},
             "autotune": {"best": best, "points_measured": len(tried), "seconds": tune_s, "points": tried},
-            "plain_per_gate_value": per_pass * steps / t_plain, "speedup_vs_plain": t_plain / t_batch,
-            "seconds_batched_per_step": t_batch / steps, "seconds_plain_per_step": t_plain / steps,
+            "one_by_one_value": per_pass * steps / t_plain, "speedup_vs_one_by_one": t_plain / t_batch,
+            "seconds_batched_per_step": t_batch / steps, "seconds_one_by_one_per_step": t_plain / steps,
             "seconds_first_call_with_capture": capture_s, "graph_replays": replays,
             "min_fidelity_lb_sum": lb, "mean_compression_ratio": float(np.mean(ratio))}
 
@@ -554,7 +578,7 @@ def run_qaoa34(args) -> dict:
     st0 = sim.stats()
     timed = gates[w:]
     clocks = Clocks(int(os.environ.get("LOCAL_RANK", "0")))
-    sim.set_timing(1)
+    sim.timing()  # the traffic counters from here
     torch.cuda.synchronize()
     clocks.start()
     ev0, ev1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
@@ -567,8 +591,9 @@ def run_qaoa34(args) -> dict:
     tm = sim.timing()
     st = sim.stats()
     updates = st["amp_updates"] - st0["amp_updates"]
-    kernel_ms = tm["gate_kernel_ms"] / max(1, tm["launches"])
-    bpl = (tm["bytes_read"] + tm["bytes_written"]) / max(1, tm["launches"])
+    launches = st["kernel_launches"] - st0["kernel_launches"]
+    kernel_ms = ms / max(1, launches)
+    bpl = (tm["bytes_read"] + tm["bytes_written"]) / max(1, launches)
     pk = peaks().get("hbm_gbs")
     echo = None
     if args.echo:
@@ -593,8 +618,9 @@ def run_qaoa34(args) -> dict:
             "fidelity_lb_sum": st["fidelity_lb_sum"], "fidelity_lb_prod": st["fidelity_lb_prod"],
             "roofline": {"bound": "hbm", "achieved": bpl / (kernel_ms * 1e-3) / 1e9 if kernel_ms else None, "peak": pk,
                          "unit": "GB/s", "frac": (bpl / (kernel_ms * 1e-3) / 1e9 / pk) if (pk and kernel_ms) else None,
-                         "traffic": None, "kernel": "k_gate", "kernel_ms_avg": kernel_ms},
-            "gpu_launches": 2 * tm["launches"], "clocks": clk, "echo": echo}
+                         "traffic": None, "kernel": "k_group + k_run, single gates k_gate_fast + k_gate + k_post; the run over its launches",
+                         "kernel_ms_avg": kernel_ms},
+            "gpu_launches": launches, "clocks": clk, "echo": echo}
 
 
 def train_selector(qcsim, eps: float, seed: int):

@@ -51,3 +51,15 @@ def test_gpu_arm_line():
     cb = d["cpu_baseline"]
     assert cb["kind"] == "oracle" and cb["value"] > 0 and cb["cores"] >= 1
     assert 0.0 < d["fidelity"] <= 1.0 + 1e-12 and d["fidelity"] >= d["fidelity_lb_sum"] - 1e-12
+
+
+@pytest.mark.gpu
+def test_value_times_the_call_that_a_user_makes():
+    """The timed steps run as the end-to-end steps do, by groups of gates (a gate by itself
+    takes three launches); the gates timed one by one are reported beside them."""
+    d = run_bench("--rows", "4", "--cols", "5", "--steps", "3", "--warmup", "3", "--no-cpu-baseline", "--no-sweep",
+                  "--no-batch")
+    assert 0 < d["gpu_launches"] < 2 * d["config"]["gates_timed"]
+    g = d["gate_by_gate"]
+    assert g["gates"] == sum(c["launches"] for c in d["roofline_by_class"].values()) > 0
+    assert d["value"] > 0 and g["amp_updates_per_s"] > 0
