@@ -1982,6 +1982,15 @@ sim_status sim_checkpoint_load(sim_t* s, const void* in, uint64_t in_len, int in
     h.err = 0;
     h.n64 = 0;  // counted from the loaded images below
     h.dn64 = 0;
+    // the page caches are emptied below, and nothing is left of a gate or step that was under
+    // way when the handle failed
+    h.wc_pages = 0;
+    h.ndefer = 0;
+    h.fast_all = 0;
+    h.bc_gate_lookups = h.bc_gate_hits = 0;
+    h.timeout_site = 0;
+    h.run_arrived = h.run_gate = h.run_progress = 0;
+    for (int g = 0; g < qc::kRunGroup; ++g) h.run_dE[g] = h.run_dn64[g] = h.run_dpages[g] = 0;
     e = cudaMemcpyAsync(s->d_ctl, &h, sizeof(h), cudaMemcpyHostToDevice, s->st);
   }
   if (e == cudaSuccess) e = cudaMemsetAsync(s->d_counts, 0, 8 * sizeof(unsigned long long), s->st);

@@ -97,3 +97,59 @@ def test_checkpoint_layout_and_rejections():
     bad[256:260] = np.frombuffer(np.uint32(17).tobytes(), dtype=np.uint8)
     with pytest.raises(qc().SimError):
         make(n, kc, 1e-4).restore(bad)
+
+
+@pytest.mark.parametrize("how", ["gates", "circuit"])
+def test_load_into_a_handle_that_ran_on(how):
+    """Back to a checkpoint on the handle that took it, after gates whose free pages stay in
+    the streaming kernel's warp caches: the pages in use are those of the loaded images, and
+    the run goes on as the uninterrupted one."""
+    n, kc, eps = 14, 9, 1e-4
+    gates = Cc.rcs_n(n, 10, seed=31)
+
+    def go(s, part):
+        if how == "circuit":
+            s.apply_circuit(part)
+        else:
+            for g in part:
+                s.apply_gate(g)
+
+    a, b = make(n, kc, eps), make(n, kc, eps)
+    go(a, gates[:100])
+    go(b, gates[:100])
+    ck, before = a.checkpoint(), a.stats()
+    go(a, gates[100:150])
+    a.restore(ck)
+    assert {k: a.stats()[k] for k in KEYS} == {k: before[k] for k in KEYS}
+    go(a, gates[100:])
+    go(b, gates[100:])
+    assert images(a) == images(b)
+    assert {k: a.stats()[k] for k in KEYS} == {k: b.stats()[k] for k in KEYS}
+
+
+@pytest.mark.parametrize("n,kc,error", [(16, 10, "dry"), (20, 8, "dry"), (14, 8, "late")])
+def test_load_revives_a_handle_after_an_error(n, kc, error):
+    """A handle whose pool ran dry, or whose whole-circuit launch gave up a wait, takes a
+    checkpoint: nothing of the step that failed is left in its counters, and circuits run on
+    it, whole and gate by gate, as on a fresh handle."""
+    eps = 0.0 if error == "late" else 1e-4
+    settings = dict(chunk_log2=kc, budget=(16 << n) // 4, pool_bytes=(16 << n) // 5 if error == "dry" else 2 * (16 << n))
+    s, fresh = qc().Sim(n, 10, eps, **settings), qc().Sim(n, 10, eps, **settings)
+    ck = s.checkpoint()
+    if error == "late":
+        s.set_option("wait_polls", 1)
+    with pytest.raises(qc().SimError) as ei:
+        s.apply_circuit(Cc.rcs_n(n, 6, seed=2) if error == "dry" else Cc.to_array([Cc.gate(q % kc, Cc.SX) for q in range(80)]))
+    assert ei.value.code == (qc().ERR_OOM if error == "dry" else qc().ERR_TIMEOUT)
+    s.restore(ck)
+    s.set_option("wait_polls", 1 << 22)
+    narrow = Cc.to_array([Cc.gate(q, [Cc.H, Cc.SX, Cc.T, Cc.SY][k % 4]) for k, q in enumerate(list(range(6)) * 8)] +
+                         [Cc.gate(n - 1, Cc.X, {0: 1}), Cc.gate(n - 2, Cc.X, {1: 1}), Cc.gate(n - 1, Cc.H), Cc.gate(n - 2, Cc.T)])
+    for part in (narrow[:26], narrow[26:]):
+        for x in (s, fresh):
+            x.apply_circuit(part)
+            for g in part:
+                x.apply_gate(g)
+            x.sync()
+        assert images(s) == images(fresh)
+        assert {k: s.stats()[k] for k in KEYS} == {k: fresh.stats()[k] for k in KEYS}
