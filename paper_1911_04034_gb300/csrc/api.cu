@@ -517,6 +517,11 @@ sim_status sim_destroy(sim_t* s) {
   return SIM_OK;
 }
 
+static cudaError_t clear_block_cache(sim* s) {
+  if (!s->d_bc) return cudaSuccess;
+  return cudaMemsetAsync(s->d_bc, 0, (size_t)qc::kBcLines * qc::bc_line_bytes(qc::round16(qc::max_image_bytes(s->kc))), s->st);
+}
+
 sim_status sim_reset(sim_t* s) {
   if (!s) return fail(SIM_ERR_INVALID, "NULL handle");
   if (sim_status r = s->guard()) return r;
@@ -529,9 +534,7 @@ sim_status sim_reset(sim_t* s) {
   cudaError_t e = cudaMemcpyAsync(s->d_ctl, &h, sizeof(h), cudaMemcpyHostToDevice, s->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->P.cache_n, 0, (size_t)s->grid * 4, s->st);
   if (e == cudaSuccess) e = cudaMemsetAsync(s->P.wcache_n, 0, nwc * 4, s->st);
-  if (e == cudaSuccess && s->d_bc)  // lines are tagged by gate serial, which starts over
-    e = cudaMemsetAsync(s->d_bc, 0, (size_t)qc::kBcLines * qc::bc_line_bytes(qc::round16(qc::max_image_bytes(s->kc))),
-                        s->st);
+  if (e == cudaSuccess) e = clear_block_cache(s);  // lines are tagged by gate serial, which starts over
   if (e == cudaSuccess) e = qc::launch_pool_init(s->P, s->nchunks, s->st);
   if (e == cudaSuccess) e = qc::launch_init_chunk0(s->P, s->nchunks, s->st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);  // h is read from the host stack
@@ -2000,6 +2003,7 @@ sim_status sim_checkpoint_load(sim_t* s, const void* in, uint64_t in_len, int in
   if (e == cudaSuccess) e = cudaMemsetAsync(s->P.cache_n, 0, (size_t)s->grid * sizeof(uint32_t), s->st);
   if (e == cudaSuccess)  // the streaming kernel's warp caches held pages of the replaced arena
     e = cudaMemsetAsync(s->P.wcache_n, 0, (size_t)(s->fast_grid ? s->fast_grid : 1) * qc::fast_warps() * 4, s->st);
+  if (e == cudaSuccess) e = clear_block_cache(s);  // lines are tagged by gate serial, which goes back
   if (e == cudaSuccess) e = cudaStreamSynchronize(s->st);
   cudaFree(d_off);
   cudaFree(d_pb);

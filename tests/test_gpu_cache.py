@@ -86,3 +86,22 @@ def test_batched_launch_with_caches():
         solo.apply_circuit(circuits[k])
         assert images(batch[k]) == images(solo)
     assert sum(s.stats()["cache_hits"] for s in batch) > 0
+
+
+def test_lines_do_not_outlive_a_checkpoint_load():
+    """Back to a checkpoint, then another gate on the same state: the lines of the gate that
+    had the same number before the load must not serve it."""
+    n, kc, eps = 18, 5, 1e-4
+    first = Cc.grover(n, 1, seed=6)[0]
+    a = make(n, kc, eps, cache=True)
+    a.apply_circuit(first)
+    ck = a.checkpoint()
+    hits = a.stats()["cache_hits"]
+    a.apply_gate(Cc.gate(n - 1, Cc.SX))
+    assert a.stats()["cache_hits"] > hits
+    a.restore(ck)
+    a.apply_gate(Cc.gate(n - 1, Cc.SY))
+    b = make(n, kc, eps)
+    b.apply_circuit(first)
+    b.apply_gate(Cc.gate(n - 1, Cc.SY))
+    assert images(a) == images(b)
