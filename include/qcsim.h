@@ -94,12 +94,13 @@ typedef struct sim_stats_t {
   uint64_t split_trials;      /* chunk encodes that ran the Solution D trial */
   uint64_t cache_lookups;     /* block-cache lookups (work items that consulted it) */
   uint64_t cache_hits;        /* ... that took a cached result */
-  uint64_t fast_items;        /* work items at S <= 32 the fast path wrote (cumulative): by the streaming gate
-                               * kernel, by an image exchange, or in a whole-circuit launch as STREAM images */
+  uint64_t fast_items;        /* work items at S <= 32 the fast path wrote (cumulative): by the streaming and
+                               * the group kernel, by an image exchange, or in a whole-circuit launch as STREAM images */
   uint64_t fast_deferred;     /* work items it left to the general path (cumulative) */
-  uint64_t kernel_launches;   /* kernels the gates enqueued (selector, streaming, general and post kernels) */
+  uint64_t kernel_launches;   /* kernels the gates enqueued (a gate's selector, streaming, exchange, general and
+                               * post kernels; launches of whole circuits and of groups of gates) */
   uint64_t palette_trials;    /* chunk encodes that ran the PALETTE trial */
-  uint64_t graph_replays;     /* sim_batch_apply calls led by this handle that replayed its kept graph */
+  uint64_t graph_replays;     /* sim_batch_apply calls led by this handle that replayed a kept graph */
   int32_t ladder;             /* the controller's bound ladder (0 jump, 1 the paper's, 2 guarded) */
   uint32_t modes;             /* the mode set of sim_set_modes / sim_set_selector */
   uint64_t wide_images;       /* chunk images coded at 64 bits (the lossless stage, or a subnormal) */
@@ -163,15 +164,16 @@ sim_status sim_apply_gate(sim_t* sim, const sim_gate* gate);
 sim_status sim_apply_circuit(sim_t* sim, const sim_gate* gates, size_t n_gates);
 
 /* Batched form: runs `count` circuits, circuits[k] (n_gates[k] gates) on handle
- * sims[k], together: one launch in which every circuit has thread blocks of its own and
- * goes at its own pace (circuits on large lossy states, which fill the chip by themselves,
- * one by one before it, as sim_apply_circuit runs them) or, where an option of a handle needs kernels around each gate
- * (timing, selector network, traces, block cache, a mode set other than the default),
- * gate step t of every circuit that has one in a single fused-kernel launch and one
- * bookkeeping launch; with use_graph != 0 the launch sequence is captured into a
- * CUDA graph, launched, and kept by sims[0]: a later call whose launches are the same
- * (same handles and settings, same gates; e.g. after sim_reset) replays it without
- * capturing or uploading again (sim_stats_t.graph_replays).  Each handle keeps its own
+ * sims[k].  Circuits on large lossy states, which fill the chip by themselves, run one by
+ * one first, as sim_apply_circuit runs them (no graph).  The others run together: one
+ * launch in which every circuit has thread blocks of its own and goes at its own pace or,
+ * where an option of one of them needs kernels around each gate (timing, selector
+ * network, traces, block cache, a mode set other than the default), gate step t of every
+ * circuit that has one in a single fused-kernel launch and one bookkeeping launch.  With
+ * use_graph != 0 that launch sequence is captured into a CUDA graph, launched, and kept by
+ * the first handle in it: a later call whose launches are the same (same handles and
+ * settings, same gates; e.g. after sim_reset) replays it without capturing or uploading
+ * again (counted in graph_replays of that handle and of sims[0]).  Each handle keeps its own
  * pool, controller and statistics, and ends in exactly the state sim_apply_circuit
  * would give it.  The
  * handles must be distinct and share chunk_log2; launches go to sims[0]'s stream.
@@ -185,9 +187,8 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
  * gates and every circuit at least 8 qubits (blocks 2^10..2^16, chunks 2^8..2^10 up to
  * the smallest circuit, ladders 0..2, mode sets Solution C and Solution C + PALETTE);
  * else blocks 2^20, chunks 2^min(10, smallest n), the jump ladder, Solution C.  Bound
- * err_bound after the lossless stage at budget raw/4, page pool raw + 1/8 + 8 MiB, the
- * gates advanced one step at a time across all circuits in one persistent launch
- * replayed from a CUDA graph (sim_batch_apply).  The handles are created and destroyed
+ * err_bound after the lossless stage at budget raw/4, page pool raw + 1/8 + 8 MiB; then
+ * sim_batch_apply with its graph.  The handles are created and destroyed
  * inside the call.  Errors as sim_create_ex / sim_autotune / sim_batch_apply. */
 sim_status sim_batch_run(int n_circ, const int* n_qubits, const sim_gate* const* circ, const size_t* n_gates,
                          double err_bound, sim_stats_t* out);
@@ -353,12 +354,14 @@ sim_status sim_checkpoint_load(sim_t* sim, const void* in, uint64_t in_len, int 
 /* Number of chunks and chunk_log2 of the handle. */
 sim_status sim_layout(sim_t* sim, uint64_t* n_chunks, int* chunk_log2, int* block_log2);
 
-/* Timing of the fused gate kernel: with timing on (on = 1; on = 2 also counts the
- * SM cycles of each phase of the kernel, see sim_stats_t), every gate-kernel launch is
+/* Timing of the gate kernels: with timing on (on = 1; on = 2 also counts the
+ * SM cycles of each phase of the kernel, see sim_stats_t), circuits run gate by gate --
+ * no whole-circuit launches, no groups of gates -- and every gate's kernels are
  * bracketed by CUDA events on the handle's stream.  sim_timing synchronises and
  * returns, since timing was switched on or last read: the summed kernel time in ms,
- * the number of gate-kernel launches, and the chunk-image bytes those launches read
- * and wrote (the compressed traffic of the gates); then it starts counting anew. */
+ * the number of gates timed (0 with timing off), and the chunk-image bytes that gates read
+ * and wrote (the compressed traffic, counted with timing off too); then it starts counting
+ * anew. */
 sim_status sim_set_timing(sim_t* sim, int on);
 sim_status sim_timing(sim_t* sim, double* gate_kernel_ms, uint64_t* launches, uint64_t* bytes_read,
                       uint64_t* bytes_written);

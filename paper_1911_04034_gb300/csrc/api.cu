@@ -401,7 +401,7 @@ sim_status sim_create_ex(int n_qubits, int block_log2, int chunk_log2, double er
     // or what the pool has beyond every chunk stored RAW; none if not even one CTA fits.
     // The warps keep 64, 32 or 16 ids: the most that leaves every CTA its place.  (With
     // 64 always, a 21-qubit state in a pool of 9/8 raw + 64 MB had 113 of 456 CTAs: 2048
-    // items took five rounds: 170 us a gate, now 57.)
+    // items took five rounds: 170 us a gate instead of 57.)
     const uint64_t items = (s->nchunks + 1) / 2, need = (items + qc::fast_items(0) - 1) / qc::fast_items(0);
     uint64_t cap = (uint64_t)s->fast_grid < need ? (uint64_t)s->fast_grid : need;
     if (pool_bytes) {
@@ -418,13 +418,13 @@ sim_status sim_create_ex(int n_qubits, int block_log2, int chunk_log2, double er
   }
   // Whole circuits in one launch (see run_applies) where the resident CTAs take the largest
   // gate in one round; from two rounds on groups of gates by the streaming code are faster
-  // (2^10-amplitude chunks, 256 items 19 us a gate here; 512 items 36 against 23 by groups
-  // and 50 gate by gate).
+  // (2^10-amplitude chunks: 256 items 12.5 us a gate here, 48 gate by gate; 512 items 31.6 here,
+  // 23.0 by groups, 46.7 gate by gate).
   {
     const uint64_t sms = (uint64_t)device_sms(), wide = sms * qc::run_ctas_per_sm(s->kc, true);
     const uint64_t fit = sms * qc::run_ctas_per_sm(s->kc, false), items = (s->nchunks + 1) / 2;
-    // a lossless run has nothing to settle: its groups share passes at any size (23 qubits,
-    // 11.1 ms a random-circuit layer gate by gate, 7.1 ms by groups)
+    // a lossless run has nothing to settle: its groups share passes at any size (23 qubits in
+    // 2^10-amplitude chunks, 347 us a gate gate by gate, 164 by groups)
     const bool any = cp.nlevels == 0 && s->nchunks <= kRunChunks;
     s->run_wide = wide > 0 && (items <= wide || (any && items > fit));
     if (items <= fit || any) s->run_grid = (int)(s->run_wide ? (items < wide ? items : wide) : (items < fit ? items : fit));
@@ -1445,7 +1445,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
   sim* lead = sims[0];
   // Circuits on states of several rounds of the resident CTAs fill the chip by themselves and
   // run faster one by one in groups of gates than beside others in one launch (256 circuits of
-  // 14 to 24 qubits, all in one launch 3.6e10 amplitude updates/s, one by one 6.3e10); the
+  // 14 to 24 qubits: all in one launch 3.6e10 amplitude updates/s, this way 7.1e10); the
   // others go together as below.
   {
     std::vector<sim_t*> rest;

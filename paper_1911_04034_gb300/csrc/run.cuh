@@ -21,9 +21,9 @@ namespace qc {
 // leave every pair of chunks to itself: gates inside chunks, diagonal gates anywhere, and
 // gates on one cross-chunk target.  Values are truncated and coded after each gate, for its
 // byte count and pages, but decoded once and written once a group, and the CTAs meet once.
-// Lossy random circuits, gate by gate in one launch -> by steps: 12 qubits in 2^8-amplitude
-// chunks 14.1 -> 7.0 us a gate, 17 in 2^9 17.5 -> 9.3, 18 in 2^10 24.0 -> 14.5, 19 in 2^11
-// 28.2 -> 18.7 (a streaming, a general and a bookkeeping launch per gate: 26, 31, 46, 73).
+// Lossy random circuits, a streaming, a general and a bookkeeping launch per gate -> whole
+// circuits: 12 qubits in 2^8-amplitude chunks 22.5 -> 5.3 us a gate, 17 in 2^9 32.6 -> 8.1, 18 in
+// 2^10 44.3 -> 10.0, 19 in 2^11 71.4 -> 14.6 (one gate a step: 14.1, 17.5, 24.0, 28.2).
 
 // What a step's gates changed, per gate (shared memory, thread 0 of a CTA writes).
 struct RunSums {

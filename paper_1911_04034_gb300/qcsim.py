@@ -369,7 +369,7 @@ def batch_run(circuits: list, n_qubits: list, err_bound: float) -> list[dict]:
 
 
 def autotune_chunk(n_qubits: int, block_log2: int, err_bound: float, probe, candidates=(8, 9, 10, 11)):
-    """Returns (best chunk_log2, {candidate: amplitude updates/s of kernel time})."""
+    """Returns (best chunk_log2, {candidate: amplitude updates/s of the probe's second half})."""
     g = gates_array(probe)
     cand = (C.c_int * len(candidates))(*candidates)
     rates = np.zeros(len(candidates))

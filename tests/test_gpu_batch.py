@@ -1,5 +1,5 @@
-"""Batched launches (many circuits of uneven size in one persistent launch per gate
-step, captured in a CUDA graph) and the chunk-size autotuner.  Each circuit must end
+"""Batched launches (many circuits of uneven size in one launch captured in a CUDA graph,
+large states in groups of gates before it) and the chunk-size autotuner.  Each circuit must end
 in exactly the state -- chunk images, counters, controller -- that running it alone
 gives, and the oracle's compressed simulator agrees with both."""
 import numpy as np
