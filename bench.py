@@ -145,8 +145,8 @@ def per_class(gates: np.ndarray, tl: dict, n: int, kc: int, hbm: float | None) -
     return out
 
 
-# GB300 FP64 (vector pipe): the nominal rate of the part; a DFMA-throughput loop on this
-# pool's GB300 (eight independent chains per thread, 1216 CTAs of 256 threads) measured
+# GB300 FP64 (vector pipe): the nominal rate of the part; a DFMA-throughput loop on
+# a GB300 (eight independent chains per thread, 1216 CTAs of 256 threads) measured
 # 6.27e11 fused multiply-adds per second = 1.255 TFLOP/s.
 FP64_PEAK_TFLOPS = 1.25
 FP64_PEAK_SOURCE = "nominal GB300 FP64 (vector) rate; a DFMA-throughput loop measured 1.255 TFLOP/s"
