@@ -237,8 +237,8 @@ sim_status sim_set_budget(sim_t* sim, uint64_t bytes);
  * "fast_path" (1 default: gates run the streaming kernel first where it applies, see
  * sim_apply_gate, and circuits on small states run in one launch; 0: every gate through
  * the general kernel -- same bytes, slower),
- * "wait_polls" (1..2^22, default 2^22: polls without any progress after which a wait inside
- * a whole-circuit launch gives up, SIM_ERR_TIMEOUT),
+ * "wait_polls" (0..2^30: polls after which a wait inside a whole-circuit launch gives up,
+ * SIM_ERR_TIMEOUT; default 0: as many as the work of a step can take, ten times over),
  * "ladder" (0/1/2; only before the first gate).  "chunk_log2" and "block_log2" are fixed
  * at creation.  Unknown keys or values out of range: SIM_ERR_INVALID. */
 sim_status sim_set_option(sim_t* sim, const char* key, int64_t value);

@@ -183,7 +183,7 @@ struct sim {
   size_t run_cap = 0;
   int run_grid = 0;                  // its CTAs (0: not used for this state)
   bool run_wide = false;             // ... two an SM
-  uint32_t run_polls = qc::kRunPolls;  // ... polls without progress before a wait of theirs gives up
+  uint32_t wait_polls = 0;           // ... polls after which a wait of theirs gives up (0: see run_polls)
   int* h_level = nullptr;            // pinned: the controller's level as two looks found it
   cudaEvent_t ev_level[3] = {nullptr, nullptr, nullptr};  // theirs, and the gates' they follow
   cudaStream_t st_level = nullptr;   // the stream that fetches it
@@ -709,6 +709,15 @@ static uint32_t run_keep(const sim* s, int ctas) {
   return (uint32_t)(q < (uint64_t)qc::kCacheCap ? q : (uint64_t)qc::kCacheCap);
 }
 
+// Polls after which a CTA gives up its wait for the others of its circuit: 2^22 (over a second),
+// and 2^14 for every pair of chunks that the slowest of them may have to itself, ten times the
+// longest step on one (32 gates on 2^11-amplitude chunks: half a millisecond).
+static uint32_t run_polls(const sim* s, int ctas) {
+  if (s->wait_polls) return s->wait_polls;
+  const uint64_t items = (s->nchunks + 1) / 2, p = (items + (uint64_t)ctas - 1) / (uint64_t)ctas << 14;
+  return (uint32_t)(p < (1ull << 22) ? 1ull << 22 : (p < 0xfffffffeull ? p : 0xfffffffeull));
+}
+
 // CTAs for each circuit of a batch: as few as let all of them end together.  A gate takes a
 // circuit's CTAs ceil(items / CTAs) rounds and one meeting (about 0.4 of a round).
 static std::vector<int> run_shares(const std::vector<const GateLaunch*>& first, const size_t* n_gates, int count,
@@ -790,7 +799,7 @@ static sim_status run_circuit(sim* s, const sim_gate* gates, size_t n, bool* ran
         s->amp_updates += s->h_run[off + k].nact << s->kc;
       }
       mark_groups(s->h_run + off, m);
-      s->h_run_jobs[seg] = {s->d_run + off, (int)m, 0, s->run_grid, run_keep(s, s->run_grid), nullptr, s->run_polls};
+      s->h_run_jobs[seg] = {s->d_run + off, (int)m, 0, s->run_grid, run_keep(s, s->run_grid), nullptr, run_polls(s, s->run_grid)};
       CK(cudaMemcpyAsync(s->d_run + off, s->h_run + off, m * sizeof(GateLaunch), cudaMemcpyHostToDevice, s->st), "gate records");
       CK(cudaMemcpyAsync(s->d_run_jobs + seg, s->h_run_jobs + seg, sizeof(qc::RunJob), cudaMemcpyHostToDevice, s->st), "gate records");
       CK(qc::launch_run(s->d_run_jobs + seg, 1, s->kc, s->run_grid, s->run_wide, s->st), "circuit kernel launch");
@@ -971,7 +980,7 @@ static sim_status group_circuit(sim* s, const sim_gate* gates, size_t n) {
     size_t jobs = 0;
     for (size_t k = 0; k < block; k += (size_t)s->h_run[k].group)
       if (s->h_run[k].group > 1)
-        s->h_run_jobs[jobs++] = {s->d_run + k, s->h_run[k].group, 0, s->rest_grid, 0u, s->d_defer, s->run_polls};
+        s->h_run_jobs[jobs++] = {s->d_run + k, s->h_run[k].group, 0, s->rest_grid, 0u, s->d_defer, run_polls(s, s->rest_grid)};
     CK(cudaMemcpyAsync(s->d_run, s->h_run, block * sizeof(GateLaunch), cudaMemcpyHostToDevice, s->st), "gate records");
     CK(cudaMemcpyAsync(s->d_run_jobs, s->h_run_jobs, jobs * sizeof(qc::RunJob), cudaMemcpyHostToDevice, s->st), "gate records");
     jobs = 0;
@@ -1133,8 +1142,8 @@ sim_status sim_set_option(sim_t* s, const char* key, int64_t value) {
     return SIM_OK;
   }
   if (k == "wait_polls") {
-    if (value < 1 || value > (int64_t)qc::kRunPolls) return fail(SIM_ERR_INVALID, "wait_polls must be in [1, %u]", qc::kRunPolls);
-    s->run_polls = (uint32_t)value;
+    if (value < 0 || value > (1 << 30)) return fail(SIM_ERR_INVALID, "wait_polls must be in [0, 2^30]");
+    s->wait_polls = (uint32_t)value;
     return SIM_OK;
   }
   if (k == "tau_ppm") {
@@ -1551,7 +1560,7 @@ sim_status sim_batch_apply(sim_t* const* sims, int count, const sim_gate* const*
         if (!n_gates[k]) continue;
         const size_t at = (size_t)(reinterpret_cast<const uint8_t*>(first[k]) - run_list.data());
         const qc::RunJob j{reinterpret_cast<const GateLaunch*>((const uint8_t*)d_jobs + at), (int)n_gates[k], run_grid,
-                           ctas[k], run_keep(sims[k], ctas[k]), nullptr, sims[k]->run_polls};
+                           ctas[k], run_keep(sims[k], ctas[k]), nullptr, run_polls(sims[k], ctas[k])};
         std::memcpy(run_list.data() + (size_t)njobs++ * sizeof j, &j, sizeof j);
         run_grid += ctas[k];
       }
@@ -1992,7 +2001,7 @@ sim_status sim_checkpoint_load(sim_t* s, const void* in, uint64_t in_len, int in
     h.fast_all = 0;
     h.bc_gate_lookups = h.bc_gate_hits = 0;
     h.timeout_site = 0;
-    h.run_arrived = h.run_gate = h.run_progress = 0;
+    h.run_arrived = h.run_gate = 0;
     for (int g = 0; g < qc::kRunGroup; ++g) h.run_dE[g] = h.run_dn64[g] = h.run_dpages[g] = 0;
     e = cudaMemcpyAsync(s->d_ctl, &h, sizeof(h), cudaMemcpyHostToDevice, s->st);
   }

@@ -104,8 +104,6 @@ struct DevCtl {
   long long dn64;                      // ... its change during the running gate
   unsigned int run_arrived;            // k_run: CTAs that finished a step (cumulative over the launch)
   unsigned int run_gate;               // k_run: steps finished and booked in the launch
-  unsigned int run_progress;           // k_run: items finished that were not their CTA's last of a step
-  unsigned int run_pad;
   long long run_dE[kRunGroup];         // k_run: changes of E, n64 and pages by each gate of the running step
   long long run_dn64[kRunGroup];
   long long run_dpages[kRunGroup];

@@ -74,11 +74,8 @@ struct RunJob {
   int first, ctas;          // its CTAs: [first, first + ctas)
   uint32_t keep;            // page ids a CTA may keep between gates
   const uint32_t* list;     // not null: the gates are one step, on the chunk pairs k_group listed here (its ndefer)
-  uint32_t polls;           // a CTA that sees nothing move for so many polls of a wait gives up
+  uint32_t polls;           // a CTA's wait for the others gives up after so many
 };
-// More than a second without an item finished anywhere; the longest item (32 gates on a pair of
-// 2^11-amplitude chunks) takes a millisecond.
-constexpr uint32_t kRunPolls = 1u << 22;
 
 // A gate inside a step of k_group (the streaming kernels' arithmetic: see GateLaunch).
 struct GroupGate {

@@ -8,11 +8,12 @@ namespace qc {
 // bookkeeping, 12 to 30 us a gate), so one launch runs a whole circuit.  Each CTA takes its
 // share of a step's chunk pairs, the simulator's CTAs meet at a counter in device memory,
 // and the last to arrive does the bookkeeping and releases the others.  Every CTA is
-// resident (a cooperative launch) and every wait is bounded: a CTA that sees nothing move --
-// no CTA of its simulator arrive, none finish an item that is not its last -- during job.polls
-// polls gives up (E_TIMEOUT, site 4).  (Polls alone would bound a step's work instead: a CTA
-// that holds all the chunks of a batch's circuit that are not zero takes seconds over 32 gates,
-// while the others wait.)  Page ids
+// resident (a cooperative launch) and every wait is bounded (E_TIMEOUT, site 4) by a number of
+// polls that grows with the pairs a CTA may have to itself (see run_polls): in a batch one CTA
+// may hold all the chunks of a circuit that are not zero and take seconds over 32 gates, while
+// the others wait.  (Counting finished items and waiting anew while the count moves needs no
+// such rule, but made every step a tenth of a microsecond longer: 14-qubit random circuit 1.86
+// -> 1.88 ms.)  Page ids
 // freed by a CTA's items stay with it between steps, up to job.keep of them (counted in
 // wc_pages like the streaming kernel's); the rest goes to the freed list.
 //
@@ -388,8 +389,7 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : CTAS)
   }
   __syncthreads();
   if (threadIdx.x == 0) s_P = s_rec[0].P;
-  // a wait that gave up in an earlier launch: its CTAs' counts do not add up any more
-  if (__syncthreads_or(threadIdx.x == 0 && (*(volatile unsigned int*)&s_rec[0].P.ctl->err & (unsigned)E_TIMEOUT) != 0u)) return;
+  __syncthreads();
   const Pool& P = s_P;
   const unsigned long long nchunks = s_rec[0].ctl.nchunks;
   const GateSmem m = gate_smem(smem, P.kc, P.dir_words, nullptr, &s_oom, s_np);
@@ -431,11 +431,9 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : CTAS)
         __syncthreads();
         const bool done = s_swapped != 0;
         __syncthreads();  // the flag is read before the next item sets it
-        if (!done) {
-          const unsigned long long c0 = item_chunk(L, item) | L.hi_vals;
-          if (!run_item<VPT>(P, s_rec, b, job, k, 1, c0, c0 | L.pair_bit, true, S, false, m, st, s_sums)) break;
-        }
-        if (threadIdx.x == 0 && item + (unsigned)job.ctas < swaps) atomicAdd(&ctl->run_progress, 1u);
+        if (done) continue;
+        const unsigned long long c0 = item_chunk(L, item) | L.hi_vals;
+        if (!run_item<VPT>(P, s_rec, b, job, k, 1, c0, c0 | L.pair_bit, true, S, false, m, st, s_sums)) break;
       }
     } else {
       bool reload = false;
@@ -444,7 +442,6 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : CTAS)
         const unsigned long long c0 = ((item & ~low) << 1) | (item & low);
         if (!run_item<VPT>(P, s_rec, b, job, k, G, c0, c0 | bit, nchunks > 1ull, S, reload, m, st, s_sums)) break;
         reload = G > 2;  // the first record's buffer has held others
-        if (threadIdx.x == 0 && it + (unsigned)job.ctas < items) atomicAdd(&ctl->run_progress, 1u);
       }
     }
     cp_async_wait_all();
@@ -502,21 +499,17 @@ __global__ void __launch_bounds__(kThreads, VPT >= 16 ? 1 : CTAS)
       __syncthreads();
     } else if (!end) {
       if (threadIdx.x == 0) {
-        auto moved = [&]() { return *(volatile unsigned int*)&ctl->run_arrived + *(volatile unsigned int*)&ctl->run_progress; };
-        uint32_t it = 0, seen = moved();
-        bool late = false;
-        while (!late && *(volatile unsigned int*)&ctl->run_gate != steps) {
-          if (++it <= job.polls) continue;
-          const uint32_t now = moved();
-          late = now == seen;
-          seen = now;
-          it = 0;
+        // (once a wait has given up, here or in an earlier launch, the arrivals do not add up)
+        const uint32_t limit = (st.err & (unsigned)E_TIMEOUT) ? 0u : job.polls;
+        uint32_t it = 0;
+        while (*(volatile unsigned int*)&ctl->run_gate != steps) {
+          if (++it > limit) {
+            atomicOr(&ctl->err, (unsigned)E_TIMEOUT);
+            atomicExch(&ctl->timeout_site, 4u);
+            break;
+          }
         }
-        if (late) {
-          atomicOr(&ctl->err, (unsigned)E_TIMEOUT);
-          atomicExch(&ctl->timeout_site, 4u);
-        }
-        s_late = late;
+        s_late = it > limit;
         __threadfence();
       }
       __syncthreads();

@@ -241,15 +241,15 @@ def test_uneven_step_on_two_thread_blocks_outlasts_no_wait():
 
 
 @pytest.mark.parametrize("batched", [False, True])
-def test_wait_that_sees_no_progress_returns_an_error(batched):
-    """wait_polls 1: the blocks that have only zero chunks look twice, find that nothing has
-    moved (the one chunk that is not zero takes longer) and give up.  The call returns
+def test_wait_that_gives_up_returns_an_error(batched):
+    """wait_polls 1: the blocks that have only zero chunks look twice at the block with the one
+    chunk that is not zero, which takes longer, and give up.  The call returns
     SIM_ERR_TIMEOUT, the handle refuses further work, others go on."""
     n, kc = 14, 8
     gates = Cc.to_array([Cc.gate(q % kc, Cc.SX) for q in range(40)] + [Cc.gate(n - 1, Cc.H)] * 40)
     s = make(n, kc, 0.0)
     with pytest.raises(qc().SimError):
-        s.set_option("wait_polls", 0)
+        s.set_option("wait_polls", -1)
     s.set_option("wait_polls", 1)
     with pytest.raises(qc().SimError) as ei:
         if batched:

@@ -142,7 +142,7 @@ def test_load_revives_a_handle_after_an_error(n, kc, error):
         s.apply_circuit(Cc.rcs_n(n, 6, seed=2) if error == "dry" else Cc.to_array([Cc.gate(q % kc, Cc.SX) for q in range(80)]))
     assert ei.value.code == (qc().ERR_OOM if error == "dry" else qc().ERR_TIMEOUT)
     s.restore(ck)
-    s.set_option("wait_polls", 1 << 22)
+    s.set_option("wait_polls", 0)
     narrow = Cc.to_array([Cc.gate(q, [Cc.H, Cc.SX, Cc.T, Cc.SY][k % 4]) for k, q in enumerate(list(range(6)) * 8)] +
                          [Cc.gate(n - 1, Cc.X, {0: 1}), Cc.gate(n - 2, Cc.X, {1: 1}), Cc.gate(n - 1, Cc.H), Cc.gate(n - 2, Cc.T)])
     for part in (narrow[:26], narrow[26:]):
